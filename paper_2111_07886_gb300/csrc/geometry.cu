@@ -154,6 +154,7 @@ static pet_status build_tables(pet_geometry *g, std::vector<ViewGeo> &views,
         vg.inv_minor = minor > 0.0 ? 1.0 / minor : 0.0;
         vg.Lf = (float)vg.L;
         vg.inv_minorf = (float)vg.inv_minor;
+        vg.inv_minorl = (float)(vg.inv_minor - (double)vg.inv_minorf);
         // backprojection: bin coordinate of the centre of pixel (ix, iy)
         vg.t0 = ((0.5 - half) * c + (0.5 - half) * s) / rho + 0.5 * (NB - 1);
         vg.cx = c / rho;
@@ -165,7 +166,9 @@ static pet_status build_tables(pet_geometry *g, std::vector<ViewGeo> &views,
         vg.hq = to_q32(vg.h);
         vg.axis = minor == 0.0 ? 1 : 0;
         vg.wslope = minor > 0.0 ? rho / (major * minor) : 0.0;
+        vg.hf = (float)vg.h;
         vg.wslopef = (float)vg.wslope;
+        vg.wslopel = (float)(vg.wslope - (double)vg.wslopef);
         // forward walk: cross coordinate (grid units) at the start of driving step 0
         const double a = vg.xdrive ? s : c;        // divisor
         const double o = vg.xdrive ? c : s;        // other component
@@ -190,8 +193,11 @@ static pet_status build_tables(pet_geometry *g, std::vector<ViewGeo> &views,
         vg.hp = 0.5 * (ac + as);
         vg.islope = minor > 0.0 ? 1.0 / (major * minor) : 0.0;
         vg.islopef = (float)vg.islope;
+        vg.islopel = (float)(vg.islope - (double)vg.islopef);
         vg.pn0q = to_q32(vg.pn0); vg.pnxq = to_q32(vg.pnx); vg.pnyq = to_q32(vg.pny);
         vg.hpq = to_q32(vg.hp);
+        vg.htq = to_q32((major - minor) / (2.0 * rho));
+        vg.htpq = to_q32(0.5 * (major - minor));
         // candidate bins of a pixel's footprint: one line per bin, or sub-lines within
         // (R - 1) / (2 R) bins of the bin centre on either side (first candidate floor(t - hh));
         // ring bins: any bin whose width meets the footprint, from one bin before the bin

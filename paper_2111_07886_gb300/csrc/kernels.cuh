@@ -211,6 +211,28 @@ __device__ __forceinline__ f2x vrsqrt(f2x a)
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dependents_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// Host side: a launch of a 256-thread (kernel)(args, batch), with programmatic stream serialization
+// when `pdl` (the kernel then waits for the stream's previous kernel in grid_dependency_wait).
+template <typename K, typename A>
+static void launch_pdl(K kernel, int grid, cudaStream_t st, bool pdl, const A &a, const Batch &b)
+{
+    if (!pdl) {
+        kernel<<<grid, 256, 0, st>>>(a, b);
+        return;
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(256);
+    cfg.dynamicSmemBytes = 0;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, a, b);
+}
+
 // 16-byte asynchronous copy global -> shared (cp.async, cached in L2 only), its commit and the
 // wait for all of this thread's copies
 __device__ __forceinline__ void cp_async16(void *smem, const void *gmem)
@@ -363,6 +385,86 @@ template <int KC, int AR, int CAPX = 0> struct BpTable {
     E e[CAP];
 };
 
+// Sums over the R equally spaced lines of a sub-ray bin, in closed form and exact in Q32.32
+// integers up to where a line falls on a kink (a line assigned to the wrong side of one, by the
+// rounding of the float index, adds at most that rounding: every sum is continuous).  Lines are
+// taken one by one below SUB_CLOSED_MIN (a closed sum costs about as much as six lines), on views
+// along an axis (whose half-open membership is not continuous), and for bins wider than
+// SUB_CLOSED_SPAN pixels or bins (the 32-bit index arithmetic).
+constexpr int SUB_CLOSED_MIN = 6;
+constexpr long long SUB_CLOSED_SPAN = 64ll << 32;
+
+// right shift that leaves 30 bits of values up to `top`, and its power of two over Q32.32
+__device__ __forceinline__ int q32_shift(long long top) { return max(0, 34 - __clzll(top)); }
+__device__ __forceinline__ float q32_scale(int shift) { return __int_as_float((127 - 32 + shift) << 23); }
+
+// sum over s = 0..R-1 of max(0, v0 + s ds), ds > 0; inv_ds = 2^9 / ds
+__device__ __forceinline__ long long ramp_sum(long long v0, long long ds, float inv_ds, int R)
+{
+    int s0 = 0;
+    if (v0 < 0) s0 = min(R, (int)ceilf((float)(int)((-v0) >> 9) * inv_ds));
+    const int m = R - s0;
+    return (long long)m * v0 + ds * (long long)((m * (s0 + R - 1)) >> 1);
+}
+
+// summed lengths of a bin's R lines in a pixel: lines at u0 + s ds from the pixel's centre, the
+// trapezoid of half-width h and top half-width ht.  The length per unit is scale + scale_l: the
+// slope's FP32 rounding would otherwise be one common factor of all lengths of the view.
+__device__ __forceinline__ float trapezoid_sum(long long u0, long long ds, float inv_ds, int R,
+                                               long long h, long long ht, int shift, float scale,
+                                               float scale_l)
+{
+    if (u0 >= h || u0 + (long long)(R - 1) * ds <= -h) return 0.f;
+    const long long v = ramp_sum(u0 + h, ds, inv_ds, R) - ramp_sum(u0 + ht, ds, inv_ds, R) -
+                        ramp_sum(u0 - ht, ds, inv_ds, R) + ramp_sum(u0 - h, ds, inv_ds, R);
+    const float d = (float)(int)(v >> shift);
+    return fmaf(d, scale, d * scale_l);
+}
+
+// One driving step of a bin's R lines: line s enters the step at cross coordinate s p (from the
+// lowest line's entry) and leaves it ast higher.
+struct LineFan {
+    long long p, ast, total, span;      // spacing, rise per step, R ast, (R - 1) p + ast
+    float inv_p, astf;                  // 2^9 / p, ast in units of 2^-23 pixel
+    float scale, scale_l;               // length per unit (and the rest of its rounding)
+    int R, shift;
+};
+
+__device__ __forceinline__ LineFan line_fan(int R, long long shq, long long ast, float inv_minor,
+                                          float inv_minor_l)
+{
+    LineFan f;
+    f.R = R;
+    f.p = 2 * (shq < 0 ? -shq : shq);
+    f.ast = ast;
+    f.total = (long long)R * ast;
+    f.span = (long long)(R - 1) * f.p + ast;
+    f.inv_p = 512.f / (float)f.p;
+    f.astf = (float)(int)(ast >> 9);
+    f.shift = q32_shift(f.total);
+    f.scale = inv_minor * q32_scale(f.shift);
+    f.scale_l = inv_minor_l * q32_scale(f.shift);
+    return f;
+}
+
+// sum over the lines of the part of their rise below cross coordinate z: min(ast, max(0, z - s p))
+__device__ __forceinline__ long long line_length_below(const LineFan &f, long long z)
+{
+    if (z <= 0) return 0;
+    if (z >= f.span) return f.total;
+    const float zf = (float)(int)(z >> 9);
+    const int some = min(f.R, (int)ceilf(zf * f.inv_p));                       // lines entered below z
+    const int full = min(some, max(0, (int)floorf((zf - f.astf) * f.inv_p) + 1));   // left below z
+    const int m = some - full;
+    return (long long)full * f.ast + (long long)m * z - f.p * (long long)((m * (full + some - 1)) >> 1);
+}
+
+__device__ __forceinline__ float fan_length(const LineFan &f, long long d)
+{
+    const float x = (float)(int)(d >> f.shift);
+    return fmaf(x, f.scale, x * f.scale_l);
+}
+
 // Sub-ray model (g.R > 1): the weight of bin b is the sum over its R lines, at offsets
 // (2 s + 1 - R) / (2 R) bins from its centre, of the single-line length (the trapezoid of oblique
 // views; for views along an axis, L for each line whose forward-walk start coordinate lies in the
@@ -424,6 +526,19 @@ __device__ __forceinline__ void bp_weights_ring(const GeoDev &g, const ViewGeo &
         }
     } else {
         const long long pq = vw.pn0q + (long long)ix * vw.pnxq + (long long)iy * vw.pnyq;
+        if (R >= SUB_CLOSED_MIN) {
+            const int shift = q32_shift((long long)R * (vw.hpq - vw.htpq));
+            const float one = q32_scale(shift), scale = vw.islopef * one, scale_l = vw.islopel * one;
+#pragma unroll
+            for (int k = 0; k < KC; ++k) {
+                const int b = b0 + k;
+                if ((unsigned)b >= (unsigned)NB) continue;
+                const long long ds = bg[b].dsq;
+                w[k] = trapezoid_sum(bg[b].c0q - pq, ds, 512.f / (float)ds, R, vw.hpq, vw.htpq, shift, scale,
+                                     scale_l);
+            }
+            return;
+        }
         const float ws = vw.islopef * (kQ32 * 256.f);
 #pragma unroll
         for (int k = 0; k < KC; ++k) {
@@ -490,6 +605,20 @@ __device__ __forceinline__ void bp_weights_sub(const GeoDev &g, const ViewGeo &v
         }
     } else {
         const long long tq = vw.t0q + (long long)ix * vw.cxq + (long long)iy * vw.cyq;
+        if (R >= SUB_CLOSED_MIN) {
+            // lines at b + (2 s + 1 - R) offq, offq half their spacing (bin units)
+            const int shift = q32_shift((long long)R * (vw.hq - vw.htq));
+            const float one = q32_scale(shift), scale = vw.wslopef * one, scale_l = vw.wslopel * one;
+            const float inv_ds = 512.f / (float)(2 * g.offq);
+#pragma unroll
+            for (int k = 0; k < KC; ++k) {
+                const int b = b0 + k;
+                if ((unsigned)b >= (unsigned)NB) continue;
+                w[k] = trapezoid_sum(((long long)b << 32) - (long long)(R - 1) * g.offq - tq, 2 * g.offq, inv_ds,
+                                     R, vw.hq, vw.htq, shift, scale, scale_l);
+            }
+            return;
+        }
         const float ws = vw.wslopef * (kQ32 * 256.f);
 #pragma unroll
         for (int k = 0; k < KC; ++k) {
@@ -796,6 +925,47 @@ __device__ void grid_reduce(double (&v)[NV], const Reducer &red, double *result,
     __syncthreads();
 }
 
+// The same in two halves, for a block that runs several virtual blocks of one scan in a row: each
+// writes its partial (reduce_partial), and one fence and ticket per run (reduce_finish, `done`
+// partials written since the last) replace one per virtual block.
+template <int NV>
+__device__ __forceinline__ void reduce_partial(double (&v)[NV], const Reducer &red, int bid, double (*sh)[32])
+{
+    block_sum<NV>(v, sh);
+    if (threadIdx.y * blockDim.x + threadIdx.x == 0)
+#pragma unroll
+        for (int k = 0; k < NV; ++k) red.partials[(size_t)k * red.capacity + bid] = v[k];
+}
+
+template <int NV>
+__device__ __forceinline__ void reduce_finish(const Reducer &red, double *result, int done, int nblocks,
+                                              double (*sh)[32])
+{
+    __shared__ bool last;
+    const int tid = threadIdx.y * blockDim.x + threadIdx.x;
+    if (tid == 0) {
+        __threadfence();
+        last = atomicAdd(red.ticket, (unsigned)done) + (unsigned)done == (unsigned)nblocks;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    const int nthr = blockDim.x * blockDim.y;
+    double acc[NV];
+#pragma unroll
+    for (int k = 0; k < NV; ++k) {
+        acc[k] = 0.0;
+        for (int i = tid; i < nblocks; i += nthr) acc[k] += __ldcg(&red.partials[(size_t)k * red.capacity + i]);
+    }
+    block_sum<NV>(acc, sh);
+    if (tid == 0) {
+#pragma unroll
+        for (int k = 0; k < NV; ++k) result[k] = acc[k];
+        *red.ticket = 0u;
+    }
+    __syncthreads();
+}
+
 template <int NV>
 __device__ void grid_reduce(double (&v)[NV], const Reducer &red, double *result)
 {
@@ -843,6 +1013,47 @@ __device__ __forceinline__ const A &scan_args(const A &one, const Batch &b, int 
     __syncthreads();
     return sh;
 }
+
+// scan_args for a block that takes consecutive virtual blocks: `cur` is the scan whose arguments
+// `sh` holds (-1: none); the copy, and its two barriers, are made only when the scan changes.
+// Returns true when it changed.
+template <class A>
+__device__ __forceinline__ bool scan_args_kept(const A &one, const Batch &b, int vb, int &local, int &count,
+                                               A &sh, int &cur, const A *&out)
+{
+    const A *src = scan_of(one, b, vb, local, count);
+    const int scan = b.nscans == 0 ? 0 : (int)(src - reinterpret_cast<const A *>(b.args));
+    if (scan == cur) return false;
+    cur = scan;
+    out = &one;
+    if (b.nscans == 0) return true;
+    __syncthreads();                                  // the previous virtual block is done with sh
+    const int nthr = blockDim.x * blockDim.y;
+    const int tid = threadIdx.y * blockDim.x + threadIdx.x;
+    const unsigned *s = reinterpret_cast<const unsigned *>(src);
+    unsigned *d = reinterpret_cast<unsigned *>(&sh);
+    for (int k = tid; k < (int)(sizeof(A) / 4); k += nthr) d[k] = __ldg(s + k);
+    __syncthreads();
+    out = &sh;
+    return true;
+}
+
+// The virtual blocks of one block of a persistent grid: runs of consecutive ones (a run mostly stays
+// within one scan, whose arguments and reduction ticket are then handled once), about eight runs
+// per block so that blocks with cheap and with costly scans even out.
+struct VblockRuns {
+    int total, len, base, at;
+    __device__ __forceinline__ explicit VblockRuns(int n)
+        : total(n), len(max(1, n / ((int)gridDim.x * 8))), base((int)blockIdx.x * len), at(0) {}
+    // the next virtual block, -1 when there is none
+    __device__ __forceinline__ int next()
+    {
+        if (at == len) { at = 0; base += (int)gridDim.x * len; }
+        return base + at < total ? base + at++ : -1;
+    }
+    // after next(): that virtual block is the last of its run
+    __device__ __forceinline__ bool ends() const { return at == len || base + at >= total; }
+};
 
 template <class A>
 __device__ __forceinline__ int total_vblocks(const A &one, const Batch &b)

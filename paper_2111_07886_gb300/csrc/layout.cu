@@ -18,6 +18,26 @@ __global__ void img_to_internal(const S *src, D *dst, int npix, int P, int Pp)
     dst[tid] = p < P ? (D)src[(size_t)p * npix + j] : (D)0;
 }
 
+// one plane: dst = src (unless they are the same array) and dst_t[x][y] = src[y][x], through a
+// 32 x 32 shared tile so that both sides are read and written in whole rows
+__global__ void __launch_bounds__(256) plane_transpose(const float *src, float *dst, float *dst_t, int N)
+{
+    __shared__ float t[32][33];
+    const int x0 = blockIdx.x * 32, y0 = blockIdx.y * 32;
+    for (int r = threadIdx.y; r < 32; r += 8) {
+        const int x = x0 + threadIdx.x, y = y0 + r;
+        if (x >= N || y >= N) continue;
+        const float v = src[(size_t)y * N + x];
+        t[r][threadIdx.x] = v;
+        if (dst != src) dst[(size_t)y * N + x] = v;
+    }
+    __syncthreads();
+    for (int r = threadIdx.y; r < 32; r += 8) {
+        const int x = x0 + r, y = y0 + threadIdx.x;
+        if (x < N && y < N) dst_t[(size_t)x * N + y] = t[threadIdx.x][r];
+    }
+}
+
 // [N*N][Pp] -> [P][N*N]
 template <typename S, typename D>
 __global__ void img_from_internal(const S *src, D *dst, int npix, int P, int Pp)
@@ -104,6 +124,15 @@ pet_status to_internal_image(const GeoDev &g, const void *src, void *dst, int sd
     return e == cudaSuccess ? PET_OK : cuda_fail(e, "img_to_internal");
 }
 
+pet_status plane_with_transpose(const GeoDev &g, const void *src, void *dst, void *dst_t, cudaStream_t st)
+{
+    LaunchScope ls(PET_K_LAYOUT, st);
+    const unsigned b = (unsigned)((g.N + 31) / 32);
+    plane_transpose<<<dim3(b, b), dim3(32, 8), 0, st>>>((const float *)src, (float *)dst, (float *)dst_t, g.N);
+    cudaError_t e = cudaGetLastError();
+    return e == cudaSuccess ? PET_OK : cuda_fail(e, "plane_transpose");
+}
+
 pet_status from_internal_image(const GeoDev &g, const void *src, void *dst, int sd, int dd,
                                cudaStream_t st)
 {
@@ -153,9 +182,10 @@ pet_status from_internal_sino(const GeoDev &g, const int *d_view_of_slot, int nv
     return e == cudaSuccess ? PET_OK : cuda_fail(e, "sino_from_internal");
 }
 
-pet_status fill_internal_ones(const GeoDev &g, void *dst, int is_double, cudaStream_t st)
+pet_status fill_internal_ones(const GeoDev &g, void *dst, int is_double, cudaStream_t st,
+                              bool transposed)
 {
-    const long long n = (long long)g.N * g.N * g.Pp;
+    const long long n = (long long)g.N * g.N * g.Pp * (transposed ? 2 : 1);   // the copy follows
     LaunchScope ls(PET_K_LAYOUT, st);
     if (is_double) img_ones_internal<double><<<blocks(n), 256, 0, st>>>((double *)dst, n, g.P, g.Pp);
     else img_ones_internal<float><<<blocks(n), 256, 0, st>>>((float *)dst, n, g.P, g.Pp);

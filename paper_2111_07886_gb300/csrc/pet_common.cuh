@@ -66,12 +66,14 @@ struct ViewGeo {
     double L;             // length per driving step = 1 / major, pixel units
     double inv_minor;     // 1 / minor (0 when minor == 0)
     float Lf, inv_minorf;
+    float inv_minorl;     // inv_minor - inv_minorf (closed sub-ray sums: see fan_length)
     int xdrive;           // 1: driving index is ix (columns), cross index is iy
     // backprojection footprint (bin units, measured from bin 0)
     long long t0q, cxq, cyq, hq;   // t(ix,iy) = t0 + ix cx + iy cy; half-width h; Q32.32
     double t0, cx, cy, h;
     double wslope;        // length per bin unit of (h - |delta|): rho / (major * minor)
-    float wslopef;
+    float hf;             // h
+    float wslopef, wslopel;   // (and wslope - wslopef)
     int axis;             // minor == 0: half-open rule, length L for delta in [-h, h)
     // sub-ray model: cross-coordinate shift of half a sub-ray spacing (rho / (2 R a), a the
     // driving component of the view's direction), grid units; sub-ray s of a bin starts
@@ -87,8 +89,11 @@ struct ViewGeo {
     // normal in pixel units, pn = pn0 + ix pnx + iy pny (double and Q32.32), the pixel's
     // half-footprint hp = (|c| + |s|) / 2 and 1 / (major minor) (pixel units)
     long long pn0q, pnxq, pnyq, hpq;
+    // half-width of the flat top of the pixel's trapezoid (where a line's length is L), bin units
+    // and pixel units: h - minor / rho and hp - minor
+    long long htq, htpq;
     double pn0, pnx, pny, hp, islope;
-    float islopef;
+    float islopef, islopel;
 };
 
 // One bin of a table-driven geometry: its first line's offset c0 and the spacing ds of its R
@@ -176,7 +181,10 @@ struct FwdArgs {
     GeoDev g;
     int slot0;                 // first sorted view slot of the subset
     int nviews;                // views in the subset
-    const void *img;           // [N*N][Pp] (float or double)
+    const void *img;           // [N*N][Pp] (float or double); single-plane FP32 scans: [N*N],
+                               // followed by its transposed copy [x][y]
+    int pad;                   // ratio mode of single-plane FP32 scans: zero bins written on both
+                               // sides of every row of out
     void *out;                 // [nviews*NB][Pp]: y, or w = 1 - counts/(y + gamma)
     const int *counts;         // [nviews*NB][Pp] (ratio / objective modes)
     const float *gamma;        // [nviews*NB][Pp]
@@ -223,6 +231,7 @@ struct UpdateArgs {
     const void *w;             // subset ratio term [nviews*NB][Pp]
     const void *f;             // f^{k,i-1} [N*N][Pp]
     void *fout;                // f^{k,i}
+    int C;                     // single-plane FP32 scans: lanes sharing one pixel
     const void *invp;          // [N*N], or [N*N][Pp] when vox (float or double)
     int vox;                   // 1: p differs per voxel (a scan with per-bin detection factors)
     const void *bptab;         // the subset's precomputed (pixel, view) entries (pet_geometry::
@@ -252,6 +261,15 @@ void update_shape(UpdateArgs &a, int arith);               // fills tpv, nvb
 GeoDev update_geo(const GeoDev &g);                        // plane grouping of the update kernel
 pet_status launch_update_batch(const UpdateArgs &shape, const Batch &b, int arith,
                                cudaStream_t st);
+// single-plane FP32 scans without TOF (plane1.cu; the calls above forward to these)
+bool plane1_path(const GeoDev &g, int arith);
+int plane1_pad();                                          // zero bins beside a row of w
+void forward_shape_p1(FwdArgs &a, int mode, int arith);
+void forward_p1_dispatch(const FwdArgs &a, const Batch &b, int mode, int arith, int grid,
+                         cudaStream_t st, bool pdl);
+void update_shape_p1(UpdateArgs &a, int arith);
+void update_p1_dispatch(const UpdateArgs &a, const Batch &b, int arith, int grid, cudaStream_t st,
+                        bool pdl);
 // the geometry's precomputed backprojection entries (d_bptab; left empty where the packed
 // update kernel does not run or a subset's views do not fit its table), and an upper bound
 // of their size from the description alone (memory accounting before creation)
@@ -291,6 +309,7 @@ struct pet_state {
     size_t esz = 4;                 // bytes per image / ratio element
     void *f[2] = {nullptr, nullptr};
     int cur = 0;
+    bool tr = false;                // single-plane FP32: f[i] is followed by its transposed copy
     void *w = nullptr;              // ratio term of the largest subset
     int *counts = nullptr;          // [V][NB][Pp], views sorted by subset
     float *gamma = nullptr;
@@ -362,10 +381,14 @@ pet_status state_create_loaded(const pet_geometry *g, double sens, const int32_t
 size_t state_bytes(const pet_geometry *g, int precision, int iterations);
 void state_release(pet_state *s, cudaStream_t st);
 pet_status check_params(const pet_params *p);
-pet_status fill_internal_ones(const GeoDev &g, void *dst, int is_double, cudaStream_t st);
+pet_status fill_internal_ones(const GeoDev &g, void *dst, int is_double, cudaStream_t st,
+                              bool transposed = false);
 void objective_args(pet_state *s, double *out3, FwdArgs *fa, ImageArgs *ra);
 
 // layout conversions (layout.cu)
+// single-plane float image [N][N] and its transposed copy (dst may equal src: the copy only)
+pet_status plane_with_transpose(const GeoDev &g, const void *src, void *dst, void *dst_t,
+                                cudaStream_t st);
 pet_status to_internal_image(const GeoDev &g, const void *src, void *dst, int src_is_double,
                              int dst_is_double, cudaStream_t st);
 pet_status from_internal_image(const GeoDev &g, const void *src, void *dst, int src_is_double,

@@ -1,0 +1,494 @@
+// FP32 projector and update of single-plane scans (2-D reconstructions, alone and in batches).
+//
+// With one plane a pixel is 4 bytes, so what bounds these kernels is not the walk's arithmetic but
+// how many cache lines one warp load touches, and how many threads a small image gives:
+//   - forward: neighbouring lanes walk neighbouring rays of a view, so at one driving step they
+//     read neighbouring pixels of the cross axis.  Views driven along x have that axis along y:
+//     they read a transposed copy of the image, which follows every single-plane FP32 image
+//     [N*N] in memory (the update writes both), so both kinds of view read a few consecutive
+//     sectors per warp;
+//   - update: a (pixel, view) entry serves one thread only, so it is computed in registers where
+//     it is used instead of going through a shared-memory table and two barriers; small images
+//     split the neighbours and views of a pixel over C lanes.
+// Sub-ray bins (R lines per bin) are taken in closed form: per driving step the lengths of a
+// bin's R equally spaced lines in one pixel are the difference of a piecewise quadratic
+// cumulative function at the pixel's two edges (line_length_below), exact in Q32.32 integers.
+#include "image.cuh"
+#include "kernels.cuh"
+#include "profile.cuh"
+
+namespace pet {
+
+int sm_count();
+int resident_blocks(const void *fn);
+
+// Single-plane FP32 scans without TOF run the kernels of this file.
+bool plane1_path(const GeoDev &g, int arith) { return g.G == 1 && arith != AR_FP64 && g.T == 1; }
+
+constexpr int P1_PAD = 4;           // zero bins on both sides of a row of w (see update_kernel_p1)
+int plane1_pad() { return P1_PAD; }
+
+constexpr int P1_MAX_CHUNKS = 32;   // most threads sharing one ray (built-in chunking)
+
+// One compensated (Kahan) or plain step of a running sum.
+template <int AR>
+__device__ __forceinline__ void p1_add(float y, float &s, float &e)
+{
+    if constexpr (AR == AR_KAHAN) {
+        y += e;
+        const float t = s + y;
+        e = y - (t - s);
+        s = t;
+    } else {
+        s += y;
+    }
+}
+
+// `steps` driving steps of one line from cross coordinate lo (Q32.32), reading rows of stride N from
+// img + base; four steps at a time (their loads are issued together), each block of four added with
+// one compensated step.  A step rises by ast < 1 pixel, so the carry of the 32-bit fractions says
+// whether it crosses into the next pixel; ast = 1 (45 degrees) is taken as 1 - 2^-32.
+template <int AR>
+__device__ __forceinline__ void p1_walk(const float *__restrict__ img, unsigned N, unsigned base, long long lo,
+                                        long long stp, long long ast, float L, float im, int steps, float &s,
+                                        float &e)
+{
+    const unsigned rise = ast > 0xFFFFFFFFLL ? 0xFFFFFFFFu : (unsigned)ast;
+    auto step = [&](float &bl) {
+        const unsigned r = (unsigned)(int)(lo >> 32), fr = (unsigned)lo, up = fr + rise;
+        const bool cross = up < fr;
+        const float l1 = cross ? __uint2float_rn(up) * im : 0.f;
+        const float *q = img + (int)(base + r);     // r may be -1
+        float x0 = 0.f, x1 = 0.f;
+        if (r < N) x0 = __ldg(q);
+        if (cross && r + 1u < N) x1 = __ldg(q + 1);
+        bl = fmaf(l1, x1, fmaf(L - l1, x0, bl));
+        lo += stp;
+        base += N;
+    };
+    for (; steps >= 4; steps -= 4) {
+        float bl = 0.f;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) step(bl);
+        p1_add<AR>(bl, s, e);
+    }
+    float bl = 0.f;
+    for (; steps > 0; --steps) step(bl);
+    p1_add<AR>(bl, s, e);
+}
+
+// Thread layout: 256 threads = S chunks x R rays (thread = chunk * R + ray), rays in view order so
+// that a warp's lanes are neighbouring bins; chunk c walks driving steps [c Lc, (c + 1) Lc).  The S
+// partial sums of a ray are combined in chunk order.  A virtual block takes a.tpv ray tiles.
+template <int AR, int MODE, bool SUB>
+__device__ __forceinline__ void fwd_p1_vblock(const FwdArgs &a, int vloc, float *comb_s, float *comb_e,
+                                              double (*red_sh)[32])
+{
+    const GeoDev &g = a.g;
+    const int NB = g.NB, N = g.N, S = a.S, R = a.R;
+    const int nrays = a.nviews * NB;
+    const int ntiles = (nrays + R - 1) / R;
+    const int c = threadIdx.x / R, rl = threadIdx.x - c * R;
+    const bool lane_ok = c < S;
+    double obj[2] = {0.0, 0.0};
+    const int t_end = min(ntiles, (vloc + 1) * a.tpv);
+    for (int tile = vloc * a.tpv; tile < t_end; ++tile) {
+        const int ray = tile * R + rl;
+        const bool live = lane_ok && ray < nrays;
+        float s = 0.f, e = 0.f;
+        int cnt = 0;
+        float gam = 0.f, m = 1.f;
+        if (MODE != FWD_PLAIN && live && c == 0) {          // read before the walk, used after it
+            cnt = __ldg(a.counts + ray);
+            gam = __ldg(a.gamma + ray);
+            if (a.mult) m = __ldg(a.mult + ray);
+        }
+        if (live) {
+            const ViewGeo &vw = g.views[a.slot0 + ray / NB];
+            const RayGeo &rg = g.rays[(size_t)a.slot0 * NB + ray];
+            // views driven along x read the transposed copy behind the image: the cross axis is
+            // contiguous and the driving axis has stride N on every view
+            const float *img = reinterpret_cast<const float *>(a.img);
+            const unsigned copy = vw.xdrive ? (unsigned)N * (unsigned)N : 0u;
+            const int Lc = (rg.nd + S - 1) / S;
+            const int k0 = c * Lc, k1 = min(rg.nd, k0 + Lc);
+            const long long stp = vw.stepq, ast = vw.absstepq;
+            const float L = vw.Lf, im = vw.inv_minorf * kQ32;
+            const unsigned base = copy + (unsigned)(rg.d0 + k0) * (unsigned)N;
+            const long long lo = rg.loq + (long long)k0 * stp;
+            if constexpr (SUB) {
+                const int nsr = g.R;
+                if (nsr >= SUB_CLOSED_MIN && !vw.axis && (long long)nsr * (rg.shq < 0 ? -rg.shq : rg.shq) < SUB_CLOSED_SPAN) {
+                    const LineFan fan = line_fan(nsr, rg.shq, ast, vw.inv_minorf, vw.inv_minorl);
+                    long long b = lo - (long long)(nsr - 1) * (rg.shq < 0 ? -rg.shq : rg.shq);
+                    unsigned row = base;
+                    for (int k = k0; k < k1; ++k) {
+                        float bl = 0.f;
+                        const int rlo = max(0, (int)(b >> 32));
+                        const int rtop = (int)((b + fan.span) >> 32), rhi = min(N - 1, rtop);
+                        long long below = line_length_below(fan, ((long long)rlo << 32) - b);
+                        for (int r = rlo; r <= rhi; ++r) {
+                            const long long up = r == rtop ? fan.total
+                                                           : line_length_below(fan, ((long long)(r + 1) << 32) - b);
+                            bl = fmaf(fan_length(fan, up - below), __ldg(img + row + (unsigned)r), bl);
+                            below = up;
+                        }
+                        p1_add<AR>(bl, s, e);
+                        b += stp;
+                        row += (unsigned)N;
+                    }
+                } else {
+                    for (int sr = 0; sr < nsr; ++sr)
+                        p1_walk<AR>(img, (unsigned)N, base, lo + (long long)(2 * sr + 1 - nsr) * rg.shq, stp, ast,
+                                    L, im, k1 - k0, s, e);
+                }
+            } else {
+                p1_walk<AR>(img, (unsigned)N, base, lo, stp, ast, L, im, k1 - k0, s, e);
+            }
+        }
+        if (S > 1) {
+            __syncthreads();
+            comb_s[threadIdx.x] = s;
+            comb_e[threadIdx.x] = e;
+            __syncthreads();
+            if (live && c == 0)
+                for (int cc = 1; cc < S; ++cc) p1_add<AR>(comb_s[cc * R + rl] + comb_e[cc * R + rl], s, e);
+        }
+        if (live && c == 0) {
+            const float tot = s + e, scale = (float)g.scale;
+            if constexpr (MODE == FWD_PLAIN) {
+                reinterpret_cast<float *>(a.out)[ray] = scale * tot;
+            } else {
+                const float af = scale * (tot * m);
+                if constexpr (MODE == FWD_RATIO) {
+                    const int u = ray / NB, b = ray - u * NB;
+                    float *out = reinterpret_cast<float *>(a.out) + (size_t)u * (NB + 2 * a.pad) + a.pad;
+                    out[b] = m * (1.f - (float)cnt / (af + gam));
+                    // the zero bins on both sides of the row (see update_kernel_p1)
+                    if (b == 0)
+                        for (int q = 1; q <= a.pad; ++q) out[-q] = 0.f;
+                    if (b == NB - 1)
+                        for (int q = 0; q < a.pad; ++q) out[NB + q] = 0.f;
+                } else {
+                    // the likelihood terms in FP64 in every mode: ln((double) Af + gamma)
+                    obj[0] += (double)af;
+                    if (cnt != 0) obj[1] += (double)cnt * log((double)af + (double)gam);
+                }
+            }
+        }
+    }
+    if constexpr (MODE == FWD_OBJECTIVE) reduce_partial<2>(obj, a.red, vloc, red_sh);
+}
+
+template <int AR, int MODE, bool SUB>
+__global__ void __launch_bounds__(256, 4) fwd_kernel_p1(const __grid_constant__ FwdArgs one, const Batch bt)
+{
+    grid_dependency_wait();                      // before any memory access
+    __shared__ float comb_s[256], comb_e[256];
+    __shared__ FwdArgs sh_args;
+    __shared__ double red_sh[2][32];
+    VblockRuns runs(total_vblocks(one, bt));
+    const FwdArgs *a = nullptr;
+    int scan = -1, done = 0, vloc = 0, nv = 0;
+    for (int vb; (vb = runs.next()) >= 0;) {
+        if (scan_args_kept(one, bt, vb, vloc, nv, sh_args, scan, a)) done = 0;
+        fwd_p1_vblock<AR, MODE, SUB>(*a, vloc, comb_s, comb_e, red_sh);
+        ++done;
+        if constexpr (MODE == FWD_OBJECTIVE)
+            if (runs.ends() || vloc + 1 == nv) {
+                reduce_finish<2>(a->red, a->result, done, nv, red_sh);
+                done = 0;
+            }
+    }
+}
+
+// What a patch's (pixel, view) entries need of a view: x = t - h at the patch's first pixel relative
+// to bin `bin`, and its slopes, in Q6.26 (a patch spans less than 32 bins: at most 10 pixel steps
+// of at most 1 / 0.36 bins); the row's first bin in w; the trapezoid (0 for views along an axis).
+struct __align__(16) P1View {
+    int x, cx, cy, bin;
+    unsigned row;
+    float h2, ws, L;           // 2 h, length per bin unit, L
+};
+constexpr int P1_VIEWS = 32;   // views of the subset a warp holds at a time
+
+// One of the 8 neighbours of pixel (ix, iy): the RDP gradient term (without its factor 2), and the
+// part in the Matlab-style gradient (q < 4: the axial ones; a missing one counts as the centre).
+__device__ __forceinline__ void p1_neighbour(const float *f, int N, int ix, int iy, int q, float fc, float gamma_r,
+                                             float eps, float &gr, float &gx, float &gy)
+{
+    const int dx = q < 4 ? (q < 2 ? 2 * q - 1 : 0) : 2 * (q & 1) - 1;
+    const int dy = q < 4 ? (q < 2 ? 0 : 2 * q - 5) : (q & 2) - 1;
+    const int x = ix + dx, y = iy + dy;
+    float fk = fc;
+    if ((unsigned)x < (unsigned)N && (unsigned)y < (unsigned)N) {
+        fk = __ldg(f + y * N + x);
+        const float d = fc - fk, ad = fabsf(d), den = fc + fk + gamma_r * ad + eps;
+        gr += __fdividef(d * (gamma_r * ad + fc + 3.f * fk + 2.f * eps), den * den);
+    }
+    if (q < 2) gx += (float)dx * fk;
+    else if (q < 4) gy += (float)dy * fk;
+}
+
+// f^{k,i} = P_t(f - lambda_k alpha_{k,i} nu S(f) (A_i^T w + (beta/M) grad R(f))) for one plane.
+// A warp works alone, without block barriers: it takes a patch of 32 / C pixels (8 x 4, 4 x 4,
+// 4 x 2 or 2 x 2, so that one view's bins are a few sectors of the row of w) with C lanes per
+// pixel, lane = chunk * (32 / C) + pixel.  Its lanes first set up one view each for the patch (the
+// 64-bit positions), then chunk c takes the neighbours and gathers the views c, c + C, ... with one
+// compensated step per view; the chunks are added in order through shuffles.  Candidate bins
+// b0 + k of a view: with e = b0 - (t - h) in [0, 1) the length is min(L, ws min(e + k, 2 h - e - k))
+// where positive; rows of w carry P1_PAD zero bins on both sides, so that an entry at the edge of
+// the sinogram needs no test per bin.  A virtual block is 8 warps x a.tpv patches; only its sum
+// ends in barriers.
+template <int KC, int AR, bool SUB>
+__global__ void __launch_bounds__(256, 4) update_kernel_p1(const __grid_constant__ UpdateArgs one, const Batch bt)
+{
+    __shared__ __align__(16) P1View views[SUB ? 1 : 8][P1_VIEWS];
+    __shared__ UpdateArgs sh_args;
+    __shared__ double red_sh[1][32];
+    __shared__ float part_sh[256];
+    grid_dependents_launch();
+    VblockRuns runs(total_vblocks(one, bt));
+    const UpdateArgs *ap = nullptr;
+    int scan = -1, done = 0, vloc = 0, nv = 0;
+    float inv_mean_f = 1.f, mean_mu = 1.f;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    for (int vb; (vb = runs.next()) >= 0;) {
+        const bool fresh = scan_args_kept(one, bt, vb, vloc, nv, sh_args, scan, ap);
+        const UpdateArgs &a = *ap;
+        const GeoDev &g = a.g;
+        const int N = g.N, NB = g.NB, npix = N * N, C = a.C, stride = NB + 2 * P1_PAD;
+        const bool dyn = a.nu_mode == 1 || a.nu_mode == 2;
+        if (fresh) {
+            done = 0;
+            if (dyn) {
+                inv_mean_f = (float)npix / (float)*a.sum_f;
+                mean_mu = (float)*a.sum_mu / (float)npix;
+            }
+        }
+        const int PX = 32 / C, TX = C == 1 ? 8 : (C == 8 ? 2 : 4), TY = PX / TX;
+        const int c = lane / PX, pl = lane - c * PX, py = pl / TX, px = pl - py * TX;
+        const int ntx = (N + TX - 1) / TX, npatch = ntx * ((N + TY - 1) / TY);
+        const float *w = reinterpret_cast<const float *>(a.w);
+        const float *f = reinterpret_cast<const float *>(a.f);
+        const float U = a.fs_U, tt = a.fs_t, scale = a.fs_scale;
+        float part = 0.f;
+        for (int k = 0; k < a.tpv; ++k) {
+            const int patch = (vloc * a.tpv + k) * 8 + wid;
+            if (patch >= npatch) break;
+            const int x0 = (patch % ntx) * TX, y0 = (patch / ntx) * TY;
+            const int ix = x0 + px, iy = y0 + py, j = iy * N + ix;
+            const bool active = ix < N && iy < N;
+            // stencil
+            float fc = 0.f, gr = 0.f, gx = 0.f, gy = 0.f;
+            if (active) {
+                fc = __ldg(f + j);
+                for (int q = c; q < 8; q += C)
+                    p1_neighbour(f, N, ix, iy, q, fc, a.fs_gamma_r, a.fs_eps, gr, gx, gy);
+            }
+            for (int o = PX; o < 32; o *= 2) {
+                gr += __shfl_xor_sync(0xffffffffu, gr, o);
+                gx += __shfl_xor_sync(0xffffffffu, gx, o);
+                gy += __shfl_xor_sync(0xffffffffu, gy, o);
+            }
+            // gather
+            float s = 0.f, e = 0.f;
+            // the general entry: sub-ray bins, and views along an axis (membership from the forward
+            // walk's own coordinates)
+            auto any_view = [&](int u) {
+                int b0;
+                float wk[KC];
+                bp_weights<KC, AR, SUB>(g, g.views[a.slot0 + u], a.slot0 + u, ix, iy, b0, wk);
+                const float *row = w + (size_t)u * stride + P1_PAD;
+                float y = 0.f;
+#pragma unroll
+                for (int q = 0; q < KC; ++q) y = fmaf(wk[q], __ldg(row + min(max(b0 + q, 0), NB - 1)), y);
+                p1_add<AR>(y, s, e);
+            };
+            if constexpr (SUB) {
+                if (active)
+                    for (int u = c; u < a.nviews; u += C) any_view(u);
+            } else {
+                P1View *vt = views[wid];
+                for (int u0 = 0; u0 < a.nviews; u0 += P1_VIEWS) {
+                    const int nvc = min(P1_VIEWS, a.nviews - u0);
+                    bool axis = false;
+                    __syncwarp();
+                    if (lane < nvc) {
+                        const ViewGeo &vw = g.views[a.slot0 + u0 + lane];
+                        const long long xq = vw.t0q - vw.hq + (long long)x0 * vw.cxq + (long long)y0 * vw.cyq;
+                        axis = vw.axis;
+                        P1View v;
+                        v.bin = (int)(xq >> 32);
+                        v.x = (int)(((unsigned)xq >> 6) + (((unsigned)xq >> 5) & 1u));
+                        v.cx = (int)((vw.cxq + 32) >> 6);
+                        v.cy = (int)((vw.cyq + 32) >> 6);
+                        v.row = (unsigned)(u0 + lane) * (unsigned)stride + P1_PAD;
+                        v.h2 = 2.f * vw.hf;
+                        v.ws = axis ? 0.f : vw.wslopef;
+                        v.L = axis ? 0.f : vw.Lf;
+                        vt[lane] = v;
+                    }
+                    const unsigned axes = __ballot_sync(0xffffffffu, axis);
+                    __syncwarp();
+                    if (!active) continue;
+#pragma unroll 4
+                    for (int u = c; u < nvc; u += C) {
+                        const P1View v = vt[u];
+                        const int x = v.x + px * v.cx + py * v.cy;
+                        const int up = (x + 0x3FFFFFF) >> 26;                            // ceil
+                        const float e0 = (float)((up << 26) - x) * 1.4901161193847656e-8f;   // b0 - (t - h)
+                        const int b0 = min(max(v.bin + up, -P1_PAD), NB + P1_PAD - KC);
+                        const float *row = w + (v.row + (unsigned)b0);
+                        float y = fminf(v.L, fmaxf(0.f, fminf(e0, v.h2 - e0)) * v.ws) * __ldg(row);
+#pragma unroll
+                        for (int q = 1; q < KC; ++q) {
+                            // KC = 2 holds geometries with 2 h < 2: the rising side ends before bin 1
+                            const float r = v.h2 - (e0 + (float)q), d = KC == 2 ? r : fminf(e0 + (float)q, r);
+                            y = fmaf(fminf(v.L, fmaxf(0.f, d) * v.ws), __ldg(row + q), y);
+                        }
+                        p1_add<AR>(y, s, e);
+                    }
+                    if (axes)
+                        for (int u = c; u < nvc; u += C)
+                            if (axes >> u & 1) any_view(u0 + u);
+                }
+            }
+            const float mine = s + e;
+            for (int cc = 1; cc < C; ++cc) p1_add<AR>(__shfl_sync(0xffffffffu, mine, cc * PX + pl), s, e);
+            // step
+            if (c == 0 && active) {
+                float nu = 1.f;
+                if (a.nu_mode == 3) {
+                    nu = __ldg(reinterpret_cast<const float *>(a.nu_frozen) + j);
+                } else if (dyn) {
+                    // central differences inside, one-sided at the border
+                    gx *= ix > 0 && ix < N - 1 ? 0.5f : 1.f;
+                    gy *= iy > 0 && iy < N - 1 ? 0.5f : 1.f;
+                    nu = nu_of<float>(gx, gy, 0.f, inv_mean_f, mean_mu, a.fs_nu1, a.fs_nu2);
+                    if (a.nu_mode == 2) reinterpret_cast<float *>(a.nu_frozen)[j] = nu;
+                }
+                const float ip = __ldg(reinterpret_cast<const float *>(a.invp) + j) * a.fs_ips;
+                const float coef = a.fs_lam * nu * ((fc < 0.5f * U ? fc : U - fc) * ip);
+                float ft = fc - coef * (scale * (s + e) + a.fs_bm * (2.f * gr));
+                ft = ft <= 0.f ? tt : (ft >= U ? U - tt : ft);
+                part += ft;
+                reinterpret_cast<float *>(a.fout)[j] = ft;
+                reinterpret_cast<float *>(a.fout)[npix + ix * N + iy] = ft;   // the transposed copy
+            }
+        }
+        // the block's 256 partial sums, added in FP64 by one warp (the FP64 pipe is narrow)
+        part_sh[threadIdx.x] = part;
+        __syncthreads();
+        if (wid == 0) {
+            double v = 0.0;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) v += (double)part_sh[q * 32 + lane];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+            if (lane == 0) a.red.partials[vloc] = v;
+        }
+        ++done;
+        if (runs.ends() || vloc + 1 == nv) {
+            reduce_finish<1>(a.red, a.sum_fout, done, nv, red_sh);
+            done = 0;
+        }
+        __syncthreads();                     // part_sh is free again
+    }
+}
+
+// ------------------------------------------------------------------------------------------
+// Shapes and launches
+// ------------------------------------------------------------------------------------------
+template <int AR>
+static const void *fwd_p1_fn(int mode, int sub)
+{
+    if (sub) return mode == FWD_PLAIN ? (const void *)fwd_kernel_p1<AR, FWD_PLAIN, true>
+                    : mode == FWD_RATIO ? (const void *)fwd_kernel_p1<AR, FWD_RATIO, true>
+                                        : (const void *)fwd_kernel_p1<AR, FWD_OBJECTIVE, true>;
+    return mode == FWD_PLAIN ? (const void *)fwd_kernel_p1<AR, FWD_PLAIN, false>
+           : mode == FWD_RATIO ? (const void *)fwd_kernel_p1<AR, FWD_RATIO, false>
+                               : (const void *)fwd_kernel_p1<AR, FWD_OBJECTIVE, false>;
+}
+
+// Chunks per ray: enough threads for one wave of 2048 per SM, at least 8 driving steps each.
+void forward_shape_p1(FwdArgs &a, int mode, int arith)
+{
+    const long long nrays = (long long)a.nviews * a.g.NB;
+    const long long want = (long long)sm_count() * 2048;
+    int S = 1;
+    while (S < P1_MAX_CHUNKS && nrays * S < want && a.g.N / (2 * S) >= 8) S *= 2;
+    if (a.g.tuneS > 0 && mode != FWD_OBJECTIVE) S = a.g.tuneS;
+    a.S = S;
+    a.R = 256 / S;
+    const long long ntiles = (nrays + a.R - 1) / a.R;
+    a.tpv = 1;
+    if (mode == FWD_OBJECTIVE) {
+        const void *fn = arith == AR_KAHAN ? fwd_p1_fn<AR_KAHAN>(mode, a.g.table) : fwd_p1_fn<AR_FP32>(mode, a.g.table);
+        const long long slots = (long long)sm_count() * resident_blocks(fn);
+        long long tpv = (ntiles + slots - 1) / slots;
+        if (a.red.capacity > 0) tpv = std::max(tpv, (ntiles + a.red.capacity - 1) / a.red.capacity);
+        a.tpv = (int)std::max(1LL, tpv);
+    }
+    a.nvb = (int)((ntiles + a.tpv - 1) / a.tpv);
+}
+
+template <int AR, bool SUB>
+static void fwd_p1_launch(const FwdArgs &a, const Batch &b, int mode, int grid, cudaStream_t st, bool pdl)
+{
+    if (mode == FWD_PLAIN) launch_pdl(fwd_kernel_p1<AR, FWD_PLAIN, SUB>, grid, st, pdl, a, b);
+    else if (mode == FWD_RATIO) launch_pdl(fwd_kernel_p1<AR, FWD_RATIO, SUB>, grid, st, pdl, a, b);
+    else launch_pdl(fwd_kernel_p1<AR, FWD_OBJECTIVE, SUB>, grid, st, pdl, a, b);
+}
+
+void forward_p1_dispatch(const FwdArgs &a, const Batch &b, int mode, int arith, int grid, cudaStream_t st,
+                         bool pdl)
+{
+    if (a.g.table) {
+        if (arith == AR_KAHAN) fwd_p1_launch<AR_KAHAN, true>(a, b, mode, grid, st, pdl);
+        else fwd_p1_launch<AR_FP32, true>(a, b, mode, grid, st, pdl);
+    } else {
+        if (arith == AR_KAHAN) fwd_p1_launch<AR_KAHAN, false>(a, b, mode, grid, st, pdl);
+        else fwd_p1_launch<AR_FP32, false>(a, b, mode, grid, st, pdl);
+    }
+}
+
+template <int AR>
+static const void *update_p1_fn(const GeoDev &g)
+{
+    if (g.table) return (const void *)update_kernel_p1<4, AR, true>;
+    return g.K <= 2 ? (const void *)update_kernel_p1<2, AR, false> : (const void *)update_kernel_p1<4, AR, false>;
+}
+
+// Lanes per pixel C: the fewest that give 16 warps per SM, at least two views each.
+void update_shape_p1(UpdateArgs &a, int arith)
+{
+    const int N = a.g.N;
+    auto patches = [&](int C) {
+        const int TX = C == 1 ? 8 : (C == 8 ? 2 : 4), TY = 32 / C / TX;
+        return (N + TX - 1) / TX * ((N + TY - 1) / TY);
+    };
+    int C = 1;
+    while (C < 8 && patches(C) < 16 * sm_count() && a.nviews >= 4 * C) C *= 2;
+    a.C = C;
+    const int slots = sm_count() * resident_blocks(arith == AR_KAHAN ? update_p1_fn<AR_KAHAN>(a.g) : update_p1_fn<AR_FP32>(a.g));
+    const int nt = (patches(C) + 7) / 8;
+    a.tpv = std::max({1, (nt + a.red.capacity - 1) / a.red.capacity, (nt + slots - 1) / slots});
+    a.nvb = (nt + a.tpv - 1) / a.tpv;
+}
+
+template <int AR>
+static void update_p1_launch(const UpdateArgs &a, const Batch &b, int grid, cudaStream_t st, bool pdl)
+{
+    if (a.g.table) launch_pdl(update_kernel_p1<4, AR, true>, grid, st, pdl, a, b);
+    else if (a.g.K <= 2) launch_pdl(update_kernel_p1<2, AR, false>, grid, st, pdl, a, b);
+    else launch_pdl(update_kernel_p1<4, AR, false>, grid, st, pdl, a, b);
+}
+
+void update_p1_dispatch(const UpdateArgs &a, const Batch &b, int arith, int grid, cudaStream_t st, bool pdl)
+{
+    if (arith == AR_KAHAN) update_p1_launch<AR_KAHAN>(a, b, grid, st, pdl);
+    else update_p1_launch<AR_FP32>(a, b, grid, st, pdl);
+}
+
+}  // namespace pet

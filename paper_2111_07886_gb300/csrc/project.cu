@@ -36,6 +36,7 @@ template <int G, int AR, int MODE, bool SUB = false>
 __global__ void __launch_bounds__(256, 3) fwd_kernel(const __grid_constant__ FwdArgs one, const Batch bt)
 {
     grid_dependency_wait();                      // before any memory access
+    static_assert(G == 8 || AR == AR_FP64, "single-plane FP32 scans run the kernels of plane1.cu");
     using T = typename ArithT<AR>::T;
     __shared__ T comb_s[256 * G];
     __shared__ T comb_e[256 * G];
@@ -208,27 +209,6 @@ __global__ void __launch_bounds__(256, 3) fwd_kernel(const __grid_constant__ Fwd
                     acc.set(2 * q, a0, b0);
                     acc.set(2 * q + 1, a1, b1);
                 }
-            } else {
-                const long long stp = vw.stepq, ast = vw.absstepq;
-                const float L = vw.Lf, im = vw.inv_minorf * kQ32;
-                for (int sr = 0; sr < nsr; ++sr) {
-                long long lo = rg.loq + (long long)(2 * sr + 1 - nsr) * (SUB ? rg.shq : vw.halfq) + (long long)k0 * stp;
-                for (int k = k0; k < k1; ++k) {
-                    const int d = rg.d0 + k;
-                    const long long hi = lo + ast;
-                    const int r0 = (int)(lo >> 32), r1 = (int)(hi >> 32);
-                    float l1 = (r1 != r0) ? __uint2float_rn((unsigned)(hi & 0xFFFFFFFFLL)) * im : 0.f;
-                    float l0 = L - l1;
-                    const bool ok0 = (unsigned)r0 < (unsigned)N, ok1 = (unsigned)r1 < (unsigned)N;
-                    l0 = ok0 ? l0 : 0.f;
-                    l1 = ok1 ? l1 : 0.f;
-                    T x0[G], x1[G];
-                    load_group<G, T>(img + (unsigned)(d * ds + (ok0 ? r0 : 0) * cs) * (unsigned)Pp, x0);
-                    load_group<G, T>(img + (unsigned)(d * ds + (ok1 ? r1 : 0) * cs) * (unsigned)Pp, x1);
-                    acc.add2terms(l0, x0, l1, x1);
-                    lo += stp;
-                }
-                }
             }
         }
         // combine the S chunks of each (ray, group) in chunk order
@@ -311,51 +291,30 @@ __global__ void __launch_bounds__(256, 3) fwd_kernel(const __grid_constant__ Fwd
     }
 }
 
-// One launch of a forward-projection instantiation; `pdl`: with programmatic stream
-// serialization (the kernel waits for the previous kernel of the stream before its first
-// memory access).
-template <typename K>
-static void fwd_launch(K kernel, int grid, cudaStream_t st, bool pdl, const FwdArgs &a, const Batch &b)
-{
-    if (!pdl) {
-        kernel<<<grid, 256, 0, st>>>(a, b);
-        return;
-    }
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(256);
-    cfg.dynamicSmemBytes = 0;
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, kernel, a, b);
-}
-
 template <int G, int AR>
 static void fwd_dispatch_mode(const FwdArgs &a, const Batch &b, int mode, int grid, cudaStream_t st,
                               bool pdl)
 {
     if (a.g.table) {
-        if (mode == FWD_PLAIN) fwd_launch(fwd_kernel<G, AR, FWD_PLAIN, true>, grid, st, pdl, a, b);
-        else if (mode == FWD_RATIO) fwd_launch(fwd_kernel<G, AR, FWD_RATIO, true>, grid, st, pdl, a, b);
-        else fwd_launch(fwd_kernel<G, AR, FWD_OBJECTIVE, true>, grid, st, pdl, a, b);
+        if (mode == FWD_PLAIN) launch_pdl(fwd_kernel<G, AR, FWD_PLAIN, true>, grid, st, pdl, a, b);
+        else if (mode == FWD_RATIO) launch_pdl(fwd_kernel<G, AR, FWD_RATIO, true>, grid, st, pdl, a, b);
+        else launch_pdl(fwd_kernel<G, AR, FWD_OBJECTIVE, true>, grid, st, pdl, a, b);
         return;
     }
-    if (mode == FWD_PLAIN) fwd_launch(fwd_kernel<G, AR, FWD_PLAIN>, grid, st, pdl, a, b);
-    else if (mode == FWD_RATIO) fwd_launch(fwd_kernel<G, AR, FWD_RATIO>, grid, st, pdl, a, b);
-    else fwd_launch(fwd_kernel<G, AR, FWD_OBJECTIVE>, grid, st, pdl, a, b);
+    if (mode == FWD_PLAIN) launch_pdl(fwd_kernel<G, AR, FWD_PLAIN>, grid, st, pdl, a, b);
+    else if (mode == FWD_RATIO) launch_pdl(fwd_kernel<G, AR, FWD_RATIO>, grid, st, pdl, a, b);
+    else launch_pdl(fwd_kernel<G, AR, FWD_OBJECTIVE>, grid, st, pdl, a, b);
 }
 
 template <int G>
 static void fwd_dispatch(const FwdArgs &a, const Batch &b, int mode, int arith, int grid,
                          cudaStream_t st, bool pdl = false)
 {
-    if (arith == AR_FP32) fwd_dispatch_mode<G, AR_FP32>(a, b, mode, grid, st, pdl);
-    else if (arith == AR_KAHAN) fwd_dispatch_mode<G, AR_KAHAN>(a, b, mode, grid, st, pdl);
-    else fwd_dispatch_mode<G, AR_FP64>(a, b, mode, grid, st, pdl);
+    if constexpr (G == 8) {
+        if (arith == AR_FP32) return fwd_dispatch_mode<G, AR_FP32>(a, b, mode, grid, st, pdl);
+        if (arith == AR_KAHAN) return fwd_dispatch_mode<G, AR_KAHAN>(a, b, mode, grid, st, pdl);
+    }
+    fwd_dispatch_mode<G, AR_FP64>(a, b, mode, grid, st, pdl);
 }
 
 template <int G, int AR>
@@ -374,8 +333,10 @@ static const void *fwd_fn_mode(int mode, int sub)
 template <int G>
 static const void *fwd_fn_g(int mode, int arith, int sub)
 {
-    if (arith == AR_FP32) return fwd_fn_mode<G, AR_FP32>(mode, sub);
-    if (arith == AR_KAHAN) return fwd_fn_mode<G, AR_KAHAN>(mode, sub);
+    if constexpr (G == 8) {
+        if (arith == AR_FP32) return fwd_fn_mode<G, AR_FP32>(mode, sub);
+        if (arith == AR_KAHAN) return fwd_fn_mode<G, AR_KAHAN>(mode, sub);
+    }
     return fwd_fn_mode<G, AR_FP64>(mode, sub);
 }
 
@@ -415,6 +376,7 @@ int sm_count()
 void forward_shape(FwdArgs &a, int mode, int arith)
 {
     if (a.g.T > 1) { forward_shape_tof(a, mode, arith); return; }
+    if (plane1_path(a.g, arith)) { forward_shape_p1(a, mode, arith); return; }
     const long long nrays = (long long)a.nviews * a.g.NB;
     const long long want = (long long)sm_count() * 2048;
     const long long have = std::max<long long>(1, nrays * a.g.NG);
@@ -451,7 +413,8 @@ pet_status launch_forward(const FwdArgs &a0, int mode, int arith, cudaStream_t s
     Batch b{nullptr, nullptr, 0, grid};
     LaunchScope ls(mode == FWD_RATIO ? PET_K_FORWARD_RATIO
                    : (mode == FWD_OBJECTIVE ? PET_K_OBJ_FORWARD : PET_K_OTHER), st);
-    if (a.g.G == 1) fwd_dispatch<1>(a, b, mode, arith, grid, st, after_kernel);
+    if (plane1_path(a.g, arith)) forward_p1_dispatch(a, b, mode, arith, grid, st, after_kernel);
+    else if (a.g.G == 1) fwd_dispatch<1>(a, b, mode, arith, grid, st, after_kernel);
     else fwd_dispatch<8>(a, b, mode, arith, grid, st, after_kernel);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "fwd_kernel launch");
@@ -465,7 +428,8 @@ pet_status launch_forward_batch(const FwdArgs &shape, const Batch &b, int mode, 
     if (shape.g.T > 1) return launch_forward_tof_batch(shape, b, mode, arith, st);
     LaunchScope ls(mode == FWD_RATIO ? PET_K_FORWARD_RATIO
                    : (mode == FWD_OBJECTIVE ? PET_K_OBJ_FORWARD : PET_K_OTHER), st);
-    if (shape.g.G == 1) fwd_dispatch<1>(shape, b, mode, arith, b.grid, st);
+    if (plane1_path(shape.g, arith)) forward_p1_dispatch(shape, b, mode, arith, b.grid, st, false);
+    else if (shape.g.G == 1) fwd_dispatch<1>(shape, b, mode, arith, b.grid, st);
     else fwd_dispatch<8>(shape, b, mode, arith, b.grid, st);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "fwd_kernel batch launch");
@@ -493,7 +457,8 @@ static pet_status autotune_any(pet_geometry *g, int concurrent, cudaStream_t st,
         return PET_OK;
     }
     const int nv = g->voff[1] - g->voff[0];
-    const size_t qb = ((size_t)gd.N * gd.N * gd.Pp * 4 + 255) / 256 * 256;
+    const bool tr = plane1_path(gd, AR_KAHAN);      // the image's transposed copy follows it
+    const size_t qb = ((size_t)gd.N * gd.N * gd.Pp * (tr ? 8 : 4) + 255) / 256 * 256;
     const size_t pb = ((size_t)nv * gd.NB * gd.Pp * 4 + 255) / 256 * 256;
     const size_t ab = ((size_t)concurrent * sizeof(FwdArgs) + 255) / 256 * 256;
     const size_t prb = ((size_t)(concurrent + 1) * sizeof(int) + 255) / 256 * 256;
@@ -503,7 +468,7 @@ static pet_status autotune_any(pet_geometry *g, int concurrent, cudaStream_t st,
     char *img = base, *outs = base + qb;
     FwdArgs *d_args = reinterpret_cast<FwdArgs *>(outs + (size_t)concurrent * pb);
     int *d_pre = reinterpret_cast<int *>(reinterpret_cast<char *>(d_args) + ab);
-    PET_TRY(fill_internal_ones(gd, img, 0, st));
+    PET_TRY(fill_internal_ones(gd, img, 0, st, tr));
     std::vector<FwdArgs> h_args(concurrent);
     std::vector<int> h_pre(concurrent + 1);
     cudaEvent_t a, b;

@@ -109,7 +109,8 @@ static pet_status state_alloc(pet_state *s, const pet_geometry *g, int arith, in
     const size_t q_bytes = (size_t)gd.N * gd.N * gd.Pp * esz;
     int maxv = 0;
     for (int i = 0; i < gd.M; ++i) maxv = std::max(maxv, g->voff[i + 1] - g->voff[i]);
-    const size_t w_bytes = (size_t)maxv * gd.SB * gd.Pp * esz;
+    const int pad = plane1_path(gd, arith) ? 2 * plane1_pad() : 0;
+    const size_t w_bytes = (size_t)maxv * (gd.SB + pad) * gd.Pp * esz;
     const size_t sino = (size_t)gd.V * gd.SB * gd.Pp;
     if (s->g == g && s->esz == esz && s->f[0] && s->objcap >= iterations + 1 && (!tv || s->tvmem) &&
         (!attn || s->mult)) {
@@ -127,8 +128,10 @@ static pet_status state_alloc(pet_state *s, const pet_geometry *g, int arith, in
     auto get = [&](void **p, size_t n) -> cudaError_t {
         return as ? dev_malloc_async(p, n, as) : dev_malloc(p, n);
     };
-    PET_CUDA(get(&s->f[0], q_bytes));
-    PET_CUDA(get(&s->f[1], q_bytes));
+    // single-plane FP32 images are followed by their transposed copy (see plane1.cu)
+    const size_t f_bytes = plane1_path(gd, arith) ? 2 * q_bytes : q_bytes;
+    PET_CUDA(get(&s->f[0], f_bytes));
+    PET_CUDA(get(&s->f[1], f_bytes));
     PET_CUDA(get(&s->w, w_bytes));
     PET_CUDA(get((void **)&s->counts, sino * sizeof(int)));
     PET_CUDA(get((void **)&s->gamma, sino * sizeof(float)));
@@ -147,6 +150,22 @@ static pet_status state_alloc(pet_state *s, const pet_geometry *g, int arith, in
     }
     if (!as) PET_CUDA(cudaStreamSynchronize(nullptr));
     return PET_OK;
+}
+
+// the transposed copy behind image buffer p (NULL where the state keeps none)
+static void *transposed(const pet_state *s, void *p)
+{
+    return s->tr ? static_cast<char *>(p) + s->q_bytes : nullptr;
+}
+
+// f[0] from a C-ABI image (float [P][N][N], NULL: ones), with its transposed copy
+static pet_status load_image(pet_state *s, const float *d_img, cudaStream_t st)
+{
+    const GeoDev &gd = s->g->dev;
+    s->tr = plane1_path(gd, s->arith);
+    if (!d_img) return fill_internal_ones(gd, s->f[0], s->arith == AR_FP64, st, s->tr);
+    if (s->tr) return plane_with_transpose(gd, d_img, s->f[0], transposed(s, s->f[0]), st);
+    return to_internal_image(gd, d_img, s->f[0], 0, s->arith == AR_FP64, st);
 }
 
 // TV variant: the dual variable starts at zero with every (re)started reconstruction.
@@ -241,7 +260,7 @@ static pet_status state_load(pet_state *s, const int32_t *d_counts, const float 
     s->attn = d_mult != nullptr;
     if (d_mult) PET_TRY(load_factors(s, d_mult, st));
     s->cur = 0;
-    PET_TRY(to_internal_image(gd, d_img, s->f[0], 0, s->arith == AR_FP64, st));
+    PET_TRY(load_image(s, d_img, st));
     s->k = s->i = s->J = 0;
     s->tn = 1.0;
     s->have_frozen = false;
@@ -293,6 +312,7 @@ void pet::plan_subiter(pet_state *s, SubiterPlan *pl, bool with_objective)
     fa.slot0 = slot0;
     fa.nviews = nv;
     fa.img = s->f[s->cur];
+    fa.pad = s->tr && p.regularizer != PET_REG_TV ? plane1_pad() : 0;
     fa.out = s->w;
     fa.counts = s->counts + (size_t)slot0 * gd.SB * gd.Pp;
     fa.gamma = s->gamma + (size_t)slot0 * gd.SB * gd.Pp;
@@ -366,7 +386,10 @@ void pet::plan_subiter(pet_state *s, SubiterPlan *pl, bool with_objective)
 static pet_status tv_step(const SubiterPlan &pl, cudaStream_t st)
 {
     if (!pl.tv) return PET_OK;
-    return launch_tv_prox(pl.tv_args, pl.tv_iters, pl.arith, st);
+    PET_TRY(launch_tv_prox(pl.tv_args, pl.tv_iters, pl.arith, st));
+    if (!plane1_path(pl.tv_args.g, pl.arith)) return PET_OK;
+    float *x = reinterpret_cast<float *>(pl.tv_args.x);
+    return plane_with_transpose(pl.tv_args.g, x, x, x + (size_t)pl.tv_args.g.N * pl.tv_args.g.N, st);
 }
 
 // The mu pass and the forward projection only read f^{k,i-1}: the mu pass runs on a side stream
@@ -470,7 +493,7 @@ pet_status pet::state_create_loaded(const pet_geometry *g, double sens, const in
             if (r == PET_OK) r = to_internal_sino(gd, g->d_view_of_slot, 0, gd.V, d_gamma, s->gamma, 1, 0, st);
             s->attn = d_mult != nullptr;
             if (r == PET_OK && d_mult) r = load_factors(s, d_mult, st);
-            if (r == PET_OK) r = fill_internal_ones(gd, s->f[0], s->arith == AR_FP64, st);
+            if (r == PET_OK) r = load_image(s, nullptr, st);
             s->cur = 0;
             s->k = s->i = s->J = 0;
             s->tn = 1.0;
@@ -496,7 +519,8 @@ size_t pet::state_bytes(const pet_geometry *g, int precision, int iterations)
     int maxv = 0;
     for (int i = 0; i < gd.M; ++i) maxv = std::max(maxv, g->voff[i + 1] - g->voff[i]);
     const size_t sino = (size_t)gd.V * gd.SB * gd.Pp;
-    return 3 * q + (size_t)maxv * gd.SB * gd.Pp * esz + sino * 8 + reducer_bytes(kRedCap, 2) +
+    const size_t copies = plane1_path(gd, precision == PET_PREC_FP64 ? AR_FP64 : AR_KAHAN) ? 5 : 3;
+    return copies * q + (size_t)maxv * (gd.SB + 8) * gd.Pp * esz + sino * 8 + reducer_bytes(kRedCap, 2) +
            (size_t)(iterations + 1) * 24 + 1024;
 }
 
@@ -589,9 +613,7 @@ extern "C" pet_status pet_state_reset(pet_state *s, const float *d_img_init, voi
 {
     if (!s) return fail(PET_ERR_INVALID, "pet_state_reset: NULL state");
     cudaStream_t st = as_stream(stream);
-    const GeoDev &gd = s->g->dev;
-    if (d_img_init) PET_TRY(to_internal_image(gd, d_img_init, s->f[0], 0, s->arith == AR_FP64, st));
-    else PET_TRY(fill_internal_ones(gd, s->f[0], s->arith == AR_FP64, st));
+    PET_TRY(load_image(s, d_img_init, st));
     s->cur = 0;
     s->k = s->i = s->J = 0;
     s->tn = 1.0;
@@ -684,6 +706,7 @@ extern "C" pet_status pet_state_import(pet_state *s, const void *h_buf, size_t b
     const char *o = reinterpret_cast<const char *>(h_buf) + sizeof(h);
     s->cur = h.cur;
     PET_CUDA(cudaMemcpyAsync(s->f[s->cur], o, s->q_bytes, cudaMemcpyHostToDevice, st));
+    if (s->tr) PET_TRY(plane_with_transpose(s->g->dev, s->f[s->cur], s->f[s->cur], transposed(s, s->f[s->cur]), st));
     o += s->q_bytes;
     PET_CUDA(cudaMemcpyAsync(s->nu_frozen, o, s->q_bytes, cudaMemcpyHostToDevice, st));
     o += s->q_bytes;
@@ -745,13 +768,14 @@ static pet_status state_objective_beside(pet_state *s, double *out3, cudaStream_
         PET_CUDA(cudaStreamCreateWithFlags(&s->ostream, cudaStreamNonBlocking));
         PET_CUDA(cudaEventCreateWithFlags(&s->ev_ofork, cudaEventDisableTiming));
         PET_CUDA(cudaEventCreateWithFlags(&s->ev_odone, cudaEventDisableTiming));
-        PET_CUDA(dev_malloc(&s->fobj, s->q_bytes));
+        PET_CUDA(dev_malloc(&s->fobj, plane1_path(s->g->dev, s->arith) ? 2 * s->q_bytes : s->q_bytes));
         PET_CUDA(dev_malloc(&s->redobj_mem, reducer_bytes(kRedCap, 2)));
         PET_CUDA(cudaMemset(s->redobj_mem, 0, reducer_bytes(kRedCap, 2)));
         reducer_bind(s->red_obj, s->redobj_mem, kRedCap, 2);
     }
     if (s->obj_pending) PET_CUDA(cudaStreamWaitEvent(st, s->ev_odone, 0));
-    PET_CUDA(cudaMemcpyAsync(s->fobj, s->f[s->cur], s->q_bytes, cudaMemcpyDeviceToDevice, st));
+    PET_CUDA(cudaMemcpyAsync(s->fobj, s->f[s->cur], s->tr ? 2 * s->q_bytes : s->q_bytes,
+                             cudaMemcpyDeviceToDevice, st));
     PET_CUDA(cudaEventRecord(s->ev_ofork, st));
     PET_CUDA(cudaStreamWaitEvent(s->ostream, s->ev_ofork, 0));
     FwdArgs fa;
@@ -950,10 +974,12 @@ static pet_status forward_any(const pet_geometry *g, int subset, const void *d_i
     const size_t esz = is_double ? 8 : 4;
     const size_t qb = (size_t)gd.N * gd.N * gd.Pp * esz, pb = (size_t)nv * gd.SB * gd.Pp * esz;
     void *scr = nullptr;
-    PET_TRY(geometry_scratch(g, qb + pb + 256, &scr));
-    void *img_i = scr, *proj_i = reinterpret_cast<char *>(scr) + ((qb + 255) / 256) * 256;
-    PET_TRY(to_internal_image(gd, d_img, img_i, is_double, is_double, st));
+    const bool tr = plane1_path(gd, is_double ? AR_FP64 : AR_KAHAN);
+    PET_TRY(geometry_scratch(g, (tr ? 2 * qb : qb) + pb + 256, &scr));
+    void *img_i = scr, *proj_i = reinterpret_cast<char *>(scr) + (((tr ? 2 * qb : qb) + 255) / 256) * 256;
     FwdArgs fa{};
+    if (tr) PET_TRY(plane_with_transpose(gd, d_img, img_i, reinterpret_cast<char *>(scr) + qb, st));
+    else PET_TRY(to_internal_image(gd, d_img, img_i, is_double, is_double, st));
     fa.g = gd;
     fa.slot0 = slot0;
     fa.nviews = nv;
@@ -1104,7 +1130,8 @@ static pet_status objective_any(const pet_geometry *g, const int32_t *d_counts,
         return fail(PET_ERR_INVALID, "pet_objective: NULL argument");
     cudaStream_t st = as_stream(stream);
     const GeoDev &gd = g->dev;
-    const size_t qb = ((size_t)gd.N * gd.N * gd.Pp * 4 + 255) / 256 * 256;
+    const bool tr = plane1_path(gd, AR_KAHAN);      // the image's transposed copy follows it
+    const size_t q4 = (size_t)gd.N * gd.N * gd.Pp * 4, qb = ((tr ? 2 : 1) * q4 + 255) / 256 * 256;
     const size_t sino = (size_t)gd.V * gd.SB * gd.Pp;
     const size_t sb = (sino * 4 + 255) / 256 * 256;
     void *scr = nullptr;
@@ -1113,7 +1140,8 @@ static pet_status objective_any(const pet_geometry *g, const int32_t *d_counts,
     void *img_i = base;
     int *cnt_i = reinterpret_cast<int *>(base + qb);
     float *gam_i = reinterpret_cast<float *>(base + qb + sb);
-    PET_TRY(to_internal_image(gd, d_img, img_i, 0, 0, st));
+    if (tr) PET_TRY(plane_with_transpose(gd, d_img, img_i, base + q4, st));
+    else PET_TRY(to_internal_image(gd, d_img, img_i, 0, 0, st));
     PET_TRY(to_internal_sino(gd, g->d_view_of_slot, 0, gd.V, d_counts, cnt_i, 0, 0, st));
     PET_TRY(to_internal_sino(gd, g->d_view_of_slot, 0, gd.V, d_gamma, gam_i, 1, 0, st));
     FwdArgs fa{};

@@ -7,6 +7,7 @@
 //     RDP value / gradient and nu maps.
 // Pixel-driven: one thread handles one pixel and one group of G planes; neighbours come
 // through L1; the gather's (pixel, view) weights are shared by all groups through shared memory.
+#include "image.cuh"
 #include "kernels.cuh"
 #include "profile.cuh"
 
@@ -18,171 +19,6 @@
 #endif
 
 namespace pet {
-
-// Loads the 3x3 in-plane neighbourhood of pixel (ix, iy) for one plane group.
-//   RG: gr_p = 2 sum_k (f_j - f_k)(gamma_R |f_j - f_k| + f_j + 3 f_k + 2 eps) / den^2
-//       (den = f_j + f_k + gamma_R |f_j - f_k| + eps; FP32 kernels use the fast reciprocal)
-//   MU: gx_p, gy_p of the Matlab-style gradient: central differences inside, one-sided at
-//       the edges (the missing side counts as the centre value)
-//   RV: rv_p = sum_k (f_j - f_k)^2 / den
-// z3: the neighbourhood is the 26 voxels around (ix, iy, plane) in the volume (neighbours
-// outside it are absent), and MU also gives gz_p, the gradient across the planes (central
-// inside, one-sided at the first and last plane, 0 for one plane).  Each position's plane group
-// is loaded with the planes just below and above it.
-template <int G, int AR, bool RG, bool MU, bool RV>
-__device__ __forceinline__ void stencil(const GeoDev &g, const typename ArithT<AR>::T *f, int grp,
-                                        int ix, int iy, typename ArithT<AR>::T gamma_r,
-                                        typename ArithT<AR>::T eps,
-                                        typename ArithT<AR>::T (&fc)[G],
-                                        typename ArithT<AR>::T (&gr)[G],
-                                        typename ArithT<AR>::T (&gx)[G],
-                                        typename ArithT<AR>::T (&gy)[G],
-                                        typename ArithT<AR>::T (&rv)[G],
-                                        bool z3 = false, typename ArithT<AR>::T *gz = nullptr)
-{
-    using T = typename ArithT<AR>::T;
-    const int N = g.N, Pp = g.Pp;
-    const T *base = f + grp * G;
-    const unsigned jc = (unsigned)iy * (unsigned)N + (unsigned)ix;   // images hold < 2^32 elements
-    load_group<G, T>(base + jc * (unsigned)Pp, fc);
-    const T hx = (ix > 0 && ix < N - 1) ? T(0.5) : T(1);
-    const T hy = (iy > 0 && iy < N - 1) ? T(0.5) : T(1);
-#pragma unroll
-    for (int p = 0; p < G; ++p) { gr[p] = T(0); gx[p] = T(0); gy[p] = T(0); rv[p] = T(0); }
-    if constexpr (MU) {
-        // a missing neighbour on one side is replaced by the centre value
-        const T sx = (ix == 0 ? -hx : T(0)) + (ix == N - 1 ? hx : T(0));
-        const T sy = (iy == 0 ? -hy : T(0)) + (iy == N - 1 ? hy : T(0));
-#pragma unroll
-        for (int p = 0; p < G; ++p) { gx[p] = sx * fc[p]; gy[p] = sy * fc[p]; }
-    }
-    // one (centre, neighbour) pair of Eq. RDP / Eq. gradRD
-    auto pair = [&](int p, T c, T k) {
-        const T d = c - k;
-        const T ad = d < T(0) ? -d : d;
-        const T den = c + k + gamma_r * ad + eps;
-        if constexpr (RG) {
-            const T num = d * (gamma_r * ad + c + T(3) * k + T(2) * eps);
-            if constexpr (AR == AR_FP64) gr[p] += num / (den * den);
-            else gr[p] += __fdividef(num, den * den);
-        }
-        if constexpr (RV) {
-            if constexpr (AR == AR_FP64) rv[p] += d * d / den;
-            else rv[p] += __fdividef(d * d, den);
-        }
-    };
-    const int z0 = grp * G;                  // plane of element 0 of the group
-#pragma unroll
-    for (int q = 0; q < 9; ++q) {
-        const int dx = q % 3 - 1, dy = q / 3 - 1;
-        if (q == 4 && !z3) continue;
-        if (!RG && !RV && dx != 0 && dy != 0) continue;    // gradient only: axial neighbours
-        const int x = ix + dx, y = iy + dy;
-        if (x < 0 || y < 0 || x >= N || y >= N) continue;
-        const unsigned jn = (unsigned)((int)jc + dy * N + dx) * (unsigned)Pp;
-        T fk[G];
-        if (q == 4) {
-#pragma unroll
-            for (int p = 0; p < G; ++p) fk[p] = fc[p];
-        } else {
-            load_group<G, T>(base + jn, fk);
-        }
-        if (z3) {
-            // the planes just below and above this position's group
-            const T lo = z0 > 0 ? f[jn + z0 - 1] : T(0);
-            const T hi = z0 + G < g.P ? f[jn + z0 + G] : T(0);
-#pragma unroll
-            for (int p = 0; p < G; ++p) {
-                const int z = z0 + p;
-                if (z >= g.P) continue;
-                if (RG || RV) {
-                    if (q != 4) pair(p, fc[p], fk[p]);
-                    if (z > 0) pair(p, fc[p], p > 0 ? fk[p - 1] : lo);
-                    if (z + 1 < g.P) pair(p, fc[p], p + 1 < G ? fk[p + 1] : hi);
-                }
-                if constexpr (MU) {
-                    if (q == 4 && gz) {
-                        const T dn = z > 0 ? (p > 0 ? fk[p - 1] : lo) : fc[p];
-                        const T up = z + 1 < g.P ? (p + 1 < G ? fk[p + 1] : hi) : fc[p];
-                        gz[p] = (z > 0 && z + 1 < g.P ? T(0.5) : T(1)) * (up - dn);
-                    }
-                }
-            }
-        } else if constexpr (RG && AR != AR_FP64 && G % 2 == 0) {
-            // packed FP32x2: two planes per instruction; 1/den^2 from the fast reciprocal
-            const float2 GR = make_float2(gamma_r, gamma_r), THREE = make_float2(3.f, 3.f);
-#pragma unroll
-            for (int p = 0; p < G; p += 2) {
-                const float2 c2 = make_float2(fc[p], fc[p + 1]), k2 = make_float2(fk[p], fk[p + 1]);
-                const float2 d = sub2(c2, k2);
-                const float2 ad = make_float2(fabsf(d.x), fabsf(d.y));
-                const float2 den = fma2(GR, ad, add2(add2(c2, k2), make_float2(eps, eps)));
-                const float2 t = fma2(GR, ad, fma2(THREE, k2, add2(c2, make_float2(2.f * eps, 2.f * eps))));
-                const float2 num = mul2(d, t);
-                const float2 den2 = mul2(den, den);
-                const float2 qq = make_float2(__fdividef(num.x, den2.x), __fdividef(num.y, den2.y));
-                gr[p] += qq.x;
-                gr[p + 1] += qq.y;
-            }
-        } else if constexpr (RG || RV) {
-#pragma unroll
-            for (int p = 0; p < G; ++p) pair(p, fc[p], fk[p]);
-        }
-        if constexpr (MU) {
-            if (q == 4) continue;
-            if (dy == 0) {
-                const T sgn = dx < 0 ? -hx : hx;
-#pragma unroll
-                for (int p = 0; p < G; ++p) gx[p] += sgn * fk[p];
-            } else if (dx == 0) {
-                const T sgn = dy < 0 ? -hy : hy;
-#pragma unroll
-                for (int p = 0; p < G; ++p) gy[p] += sgn * fk[p];
-            }
-        }
-    }
-    if constexpr (RG) {
-#pragma unroll
-        for (int p = 0; p < G; ++p) gr[p] *= T(2);
-    }
-}
-
-template <typename T>
-__device__ __forceinline__ T clampT(T v, T lo, T hi) { return v < lo ? lo : (v > hi ? hi : v); }
-
-template <typename T>
-__device__ __forceinline__ T fast_div(T a, T b)
-{
-    if constexpr (sizeof(T) == 8) return a / b;
-    else return __fdividef(a, b);
-}
-
-// |(gx, gy)|: FP32 kernels use x rsqrt(x) (two instructions, a few ulp)
-template <typename T>
-__device__ __forceinline__ T grad_norm(T gx, T gy)
-{
-    const T x = gx * gx + gy * gy;
-    if constexpr (sizeof(T) == 8) return sqrt(x);
-    else return x > 0.f ? x * rsqrtf(x) : 0.f;
-}
-
-// |(gx, gy, gz)|
-template <typename T>
-__device__ __forceinline__ T grad_norm3(T gx, T gy, T gz)
-{
-    const T x = gx * gx + gy * gy + gz * gz;
-    if constexpr (sizeof(T) == 8) return sqrt(x);
-    else return x > 0.f ? x * rsqrtf(x) : 0.f;
-}
-
-// mu = max(0.01, |grad f| / mean(f)); nu = P_{nu1}^{nu2}(mean(mu) / mu)
-template <typename T>
-__device__ __forceinline__ T nu_of(T gx, T gy, T gz, T inv_mean_f, T mean_mu, T nu1, T nu2)
-{
-    T mu = grad_norm3(gx, gy, gz) * inv_mean_f;
-    mu = mu < T(0.01) ? T(0.01) : mu;
-    return clampT<T>(fast_div(mean_mu, mu), nu1, nu2);
-}
 
 int sm_count();
 
@@ -583,11 +419,14 @@ __global__ void __launch_bounds__(256) image_kernel(const __grid_constant__ Imag
                                                     const Batch bt)
 {
     using T = typename ArithT<AR>::T;
-    const int total = total_vblocks(one, bt);
     __shared__ ImageArgs sh_args;
-    for (int vb = blockIdx.x; vb < total; vb += gridDim.x) {
-        int vloc, nv;
-        const ImageArgs &a = scan_args(one, bt, vb, vloc, nv, sh_args);
+    __shared__ double red_sh[1][32];
+    VblockRuns runs(total_vblocks(one, bt));
+    const ImageArgs *ap = nullptr;
+    int scan = -1, done = 0, vloc = 0, nv = 0;
+    for (int vb; (vb = runs.next()) >= 0;) {
+        if (scan_args_kept(one, bt, vb, vloc, nv, sh_args, scan, ap)) done = 0;
+        const ImageArgs &a = *ap;
         const GeoDev &g = a.g;
         const int N = g.N, NG = g.NG, Pp = g.Pp;
         const unsigned items = (unsigned)N * (unsigned)N * (unsigned)NG;    // < 2^32 (geometry limits)
@@ -648,7 +487,12 @@ __global__ void __launch_bounds__(256) image_kernel(const __grid_constant__ Imag
         }
         if constexpr (KIND == 0 || KIND == 1 || KIND == 4) {
             double v[1] = {(double)part};
-            grid_reduce<1>(v, a.red, a.result, vloc, nv);
+            reduce_partial<1>(v, a.red, vloc, red_sh);
+            ++done;
+            if (runs.ends() || vloc + 1 == nv) {
+                reduce_finish<1>(a.red, a.result, done, nv, red_sh);
+                done = 0;
+            }
         }
     }
 }
@@ -822,6 +666,7 @@ pet_status build_bp_table(pet_geometry *g, cudaStream_t st)
 // slots (and never more virtual blocks than the reducer has partial sums for).
 void update_shape(UpdateArgs &a, int arith)
 {
+    if (plane1_path(a.g, arith) && !a.tv) { update_shape_p1(a, arith); return; }
     const int TP = 256 / a.g.NG;
     const int ntiles = (a.g.N * a.g.N + TP - 1) / TP;
     const int sub = a.g.table, tof = a.g.T > 1;
@@ -833,14 +678,15 @@ void update_shape(UpdateArgs &a, int arith)
     a.nvb = (ntiles + a.tpv - 1) / a.tpv;
 }
 
-// items per thread: at most ~4 virtual blocks per SM (each ends in a block reduction) and never
-// more virtual blocks than reduction slots
+// items per thread: at most ~4 virtual blocks per SM (each ends in a block reduction; 2 for
+// single-plane images, of which a batch runs many) and never more virtual blocks than reduction
+// slots
 void image_shape(ImageArgs &a)
 {
     const long long items = (long long)a.g.N * a.g.N * a.g.NG;
     const long long nblk = (items + 255) / 256;
     const int cap = a.red.capacity > 0 ? a.red.capacity : (1 << 30);
-    const long long target = (long long)sm_count() * 4;
+    const long long target = (long long)sm_count() * (a.g.G == 1 ? 2 : 4);
     a.ipt = (int)std::max<long long>({1, (nblk + cap - 1) / cap, (nblk + target - 1) / target});
     a.nvb = (int)((nblk + a.ipt - 1) / a.ipt);
 }
@@ -887,7 +733,9 @@ static void update_dispatch(const UpdateArgs &a, const Batch &b, int arith, int 
 static pet_status update_any(const UpdateArgs &a, const Batch &b, int arith, int grid, cudaStream_t st)
 {
     LaunchScope ls(PET_K_UPDATE, st);
-    if (a.g.G == 1) {
+    if (plane1_path(a.g, arith) && !a.tv) {
+        update_p1_dispatch(a, b, arith, grid, st, false);
+    } else if (a.g.G == 1) {
         if (a.g.K <= 2) update_dispatch<1, 2>(a, b, arith, grid, st);
         else update_dispatch<1, 4>(a, b, arith, grid, st);
     } else {
