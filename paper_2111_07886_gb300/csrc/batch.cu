@@ -387,15 +387,11 @@ static pet_status solo_tick(pet_batch *b, BatchClass *c, int k, cudaStream_t st)
     pet_state *s = c->slot[k];
     SubiterPlan pl;
     plan_subiter(s, &pl, c->objective[k]);
-    if (pl.mu) {
-        PET_CUDA(cudaEventRecord(b->ev_fork, st));
-        PET_CUDA(cudaStreamWaitEvent(b->side, b->ev_fork, 0));
-        PET_TRY(launch_mu_sum(pl.mu_args, pl.arith, b->side));
-        PET_CUDA(cudaEventRecord(b->ev_join, b->side));
-    }
-    PET_TRY(launch_forward(pl.fwd, FWD_RATIO, pl.arith, st));
-    if (pl.mu) PET_CUDA(cudaStreamWaitEvent(st, b->ev_join, 0));
-    PET_TRY(launch_update(pl.upd, pl.arith, st));
+    PET_TRY(launch_subiter(pl, st, true, [](void *ctx, MuFork *mf) -> pet_status {
+        pet_batch *q = static_cast<pet_batch *>(ctx);
+        *mf = MuFork{q->side, q->ev_fork, q->ev_join};
+        return PET_OK;
+    }, b));
     if (pl.objective) {
         PET_TRY(launch_forward(pl.obj_fwd, FWD_OBJECTIVE, pl.arith, st));
         PET_TRY(launch_rdp_value(pl.obj_rdp, pl.arith, st));

@@ -171,4 +171,70 @@ __device__ __forceinline__ T nu_of(T gx, T gy, T gz, T inv_mean_f, T mean_mu, T 
     return clampT<T>(fast_div(mean_mu, mu), nu1, nu2);
 }
 
+// FP32 mu pass for 8-plane groups: sum over voxels of mu = max(0.01, |grad f| / mean(f))
+// (Matlab-style gradient: central differences inside, one-sided at the border, where the
+// missing neighbour is the centre value).  Thread layout of the update kernel (pixel x plane
+// group, TP = 256 / NG pixels per tile); a virtual block takes a.ipt tiles.
+__device__ __forceinline__ void mu_x8_vblock(const ImageArgs &a, int vloc, int nv)
+{
+    const GeoDev &g = a.g;
+    const int N = g.N, NG = g.NG, npix = N * N;
+    const unsigned Pp = (unsigned)g.Pp;
+    const int TP = 256 / NG;
+    const int pl = threadIdx.x / NG, grp = threadIdx.x % NG;
+    const int ntiles = (npix + TP - 1) / TP;
+    const float inv_mean_f = (float)((double)npix * g.P) / (float)*a.sum_f;
+    const float *f = reinterpret_cast<const float *>(a.f) + grp * 8;
+    const int nvalid = min(8, g.P - grp * 8);             // real planes of this group
+    float part = 0.f;
+    for (int tile = vloc * a.ipt; tile < min(ntiles, (vloc + 1) * a.ipt); ++tile) {
+        const int j = tile * TP + pl;
+        if (pl >= TP || j >= npix) continue;
+        const int ix = j % N, iy = j / N;
+        const unsigned jc = (unsigned)j;
+        f2x w_[4], e_[4], n_[4], s_[4];
+        load8x(f + (ix > 0 ? jc - 1 : jc) * Pp, w_);
+        load8x(f + (ix < N - 1 ? jc + 1 : jc) * Pp, e_);
+        load8x(f + (iy > 0 ? jc - N : jc) * Pp, n_);
+        load8x(f + (iy < N - 1 ? jc + N : jc) * Pp, s_);
+        const f2x HX = vsplat((ix > 0 && ix < N - 1) ? 0.5f : 1.f);
+        const f2x HY = vsplat((iy > 0 && iy < N - 1) ? 0.5f : 1.f);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const f2x gx = vmul(HX, vsub(e_[k], w_[k])), gy = vmul(HY, vsub(s_[k], n_[k]));
+            const f2x x2 = vfma(gx, gx, vmul(gy, gy));
+            float x0, x1, r0, r1;
+            vunpk(x2, x0, x1);
+            vunpk(vrsqrt(x2), r0, r1);
+            // |grad f|^2 below the smallest normal float (|grad f| < 1.1e-19, met on decayed
+            // backgrounds) counts as zero: mu = 0.01 there, and the flushed rsqrt would be inf
+            const float m0 = fmaxf(0.01f, x0 >= 1.17549435e-38f ? x0 * r0 * inv_mean_f : 0.f);
+            const float m1 = fmaxf(0.01f, x1 >= 1.17549435e-38f ? x1 * r1 * inv_mean_f : 0.f);
+            part += (2 * k < nvalid ? m0 : 0.f) + (2 * k + 1 < nvalid ? m1 : 0.f);
+        }
+    }
+    double v[1] = {(double)part};
+    grid_reduce<1>(v, a.red, a.result, vloc, nv);
+}
+
+// sum of mu for single-plane FP32 images: 256 a.ipt pixels of a virtual block
+__device__ __forceinline__ void mu_p1_vblock(const ImageArgs &a, int vloc, int nv)
+{
+    const GeoDev &g = a.g;
+    const int N = g.N, npix = N * N;
+    const float *f = reinterpret_cast<const float *>(a.f);
+    const float inv_mean_f = (float)npix / (float)*a.sum_f;
+    float part = 0.f;
+    for (int k = 0; k < a.ipt; ++k) {
+        const int j = (vloc * a.ipt + k) * 256 + (int)threadIdx.x;
+        if (j >= npix) break;
+        const int ix = j % N, iy = j / N;
+        float fc[1], gr[1], gx[1], gy[1], rv[1];
+        stencil<1, AR_FP32, false, true, false>(g, f, 0, ix, iy, 0.f, 0.f, fc, gr, gx, gy, rv);
+        part += fmaxf(0.01f, grad_norm3(gx[0], gy[0], 0.f) * inv_mean_f);
+    }
+    double v[1] = {(double)part};
+    grid_reduce<1>(v, a.red, a.result, vloc, nv);
+}
+
 }  // namespace pet

@@ -211,13 +211,13 @@ __device__ __forceinline__ f2x vrsqrt(f2x a)
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dependents_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
-// Host side: a launch of a 256-thread (kernel)(args, batch), with programmatic stream serialization
-// when `pdl` (the kernel then waits for the stream's previous kernel in grid_dependency_wait).
-template <typename K, typename A>
-static void launch_pdl(K kernel, int grid, cudaStream_t st, bool pdl, const A &a, const Batch &b)
+// Host side: a launch of 256-thread blocks, with programmatic stream serialization when `pdl` (the
+// kernel then waits for the stream's previous kernel in grid_dependency_wait).
+template <typename K, typename... A>
+static void launch_pdl(K kernel, int grid, cudaStream_t st, bool pdl, const A &...args)
 {
     if (!pdl) {
-        kernel<<<grid, 256, 0, st>>>(a, b);
+        kernel<<<grid, 256, 0, st>>>(args...);
         return;
     }
     cudaLaunchConfig_t cfg = {};
@@ -230,7 +230,7 @@ static void launch_pdl(K kernel, int grid, cudaStream_t st, bool pdl, const A &a
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, kernel, a, b);
+    cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
 // 16-byte asynchronous copy global -> shared (cp.async, cached in L2 only), its commit and the

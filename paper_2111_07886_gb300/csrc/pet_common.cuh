@@ -256,11 +256,17 @@ struct UpdateArgs {
 };
 // FP32 copies of the update's scalars (call after filling the double fields and g)
 void update_fp32_scalars(UpdateArgs &a);
-pet_status launch_update(const UpdateArgs &a, int arith, cudaStream_t st);
+// after_kernel: as for launch_forward, behind the projection of the same subiteration
+pet_status launch_update(const UpdateArgs &a, int arith, cudaStream_t st, bool after_kernel = false);
 void update_shape(UpdateArgs &a, int arith);               // fills tpv, nvb
 GeoDev update_geo(const GeoDev &g);                        // plane grouping of the update kernel
 pet_status launch_update_batch(const UpdateArgs &shape, const Batch &b, int arith,
                                cudaStream_t st);
+// stacks in FP32 with uniform bins and without TOF (update8.cu; launch_update forwards to these)
+bool update_x8_path(const GeoDev &g, int arith);
+const void *update_x8_fn(const UpdateArgs &a, int arith);
+void update_x8_dispatch(const UpdateArgs &a, const Batch &b, int arith, int grid, cudaStream_t st,
+                        bool pdl);
 // single-plane FP32 scans without TOF (plane1.cu; the calls above forward to these)
 bool plane1_path(const GeoDev &g, int arith);
 int plane1_pad();                                          // zero bins beside a row of w
@@ -299,6 +305,11 @@ void mu_shape(ImageArgs &a, int arith);                    // shape of the mu pa
 pet_status launch_mu_sum_batch(const ImageArgs &shape, const Batch &b, int arith, cudaStream_t st);
 pet_status launch_rdp_value_batch(const ImageArgs &shape, const Batch &b, int arith,
                                   cudaStream_t st);
+// the mu pass in the projection's launch, behind the stream's previous kernel: FP32 scans without
+// TOF, except stacks with the 3-D prior (whose pass is the generic image kernel)
+bool mu_joins_forward(const FwdArgs &a, const ImageArgs &mu, int arith);
+pet_status launch_forward_mu(const FwdArgs &a, const ImageArgs &mu, int arith, cudaStream_t st);
+void forward_mu_p1(const FwdArgs &a, const ImageArgs &m, int arith, cudaStream_t st);
 
 // per-scan reconstruction state (state.cu)
 }  // namespace pet
@@ -318,7 +329,8 @@ struct pet_state {
     void *invp_vox = nullptr;       // 1 / p_j per voxel [N*N][Pp] for diag(a) A (with mult)
     void *nu_frozen = nullptr;
     bool have_frozen = false;
-    void *tvmem = nullptr;          // TV variant: z, W, xbar, px, py (each q_bytes)
+    void *tvmem = nullptr;          // TV variant: z, W, xbar, px, py (each q_bytes) and, FP32, five
+                                    // more fields of the tiled proximal step
     double *sums = nullptr;         // [0..1] sum f (ping-pong), [2] sum mu, [3..5] objective
     double *objhist = nullptr;      // [(T+1) * 3] objective parts per outer iteration
     int objcap = 0;
@@ -352,6 +364,7 @@ struct TvArgs {
     void *xbar;                // extrapolated primal iterate
     const void *z, *w;         // z = f - W grad F_i and the metric W
     void *px, *py;             // dual variable (kept across subiterations)
+    void *x1, *x2, *xbar2, *px2, *py2;   // FP32: the passes' other fields (see tv_run_tiles)
     double b;                  // beta / M
     double t, U;               // P_t
     Reducer red;
@@ -375,6 +388,11 @@ struct SubiterPlan {
     ImageArgs obj_rdp;
 };
 void plan_subiter(pet_state *s, SubiterPlan *pl, bool with_objective);
+// the kernels of one planned subiteration on `st`; `fork` gives the side stream and the events for a
+// mu pass of its own (called only when one is needed)
+struct MuFork { cudaStream_t side; cudaEvent_t fork, join; };
+pet_status launch_subiter(const SubiterPlan &pl, cudaStream_t st, bool beside,
+                          pet_status (*fork)(void *, MuFork *), void *ctx);
 pet_status state_create_loaded(const pet_geometry *g, double sens, const int32_t *d_counts,
                                const float *d_gamma, const float *d_mult, const float *d_img,
                                const pet_params *p, cudaStream_t st, pet_state **out);

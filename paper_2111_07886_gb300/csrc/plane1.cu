@@ -184,6 +184,7 @@ template <int AR, int MODE, bool SUB>
 __global__ void __launch_bounds__(256, 4) fwd_kernel_p1(const __grid_constant__ FwdArgs one, const Batch bt)
 {
     grid_dependency_wait();                      // before any memory access
+    grid_dependents_launch();
     __shared__ float comb_s[256], comb_e[256];
     __shared__ FwdArgs sh_args;
     __shared__ double red_sh[2][32];
@@ -200,6 +201,19 @@ __global__ void __launch_bounds__(256, 4) fwd_kernel_p1(const __grid_constant__ 
                 done = 0;
             }
     }
+}
+
+// The subset projection and the mu pass in one launch (as fwd_mu_kernel)
+template <int AR, bool SUB>
+__global__ void __launch_bounds__(256, 4) fwd_mu_kernel_p1(const __grid_constant__ FwdArgs fwd,
+                                                           const __grid_constant__ ImageArgs mu, int nfwd)
+{
+    grid_dependency_wait();
+    grid_dependents_launch();
+    __shared__ float comb_s[256], comb_e[256];
+    const int vb = (int)blockIdx.x;
+    if (vb < nfwd) fwd_p1_vblock<AR, FWD_RATIO, SUB>(fwd, vb, comb_s, comb_e, nullptr);
+    else mu_p1_vblock(mu, vb - nfwd, mu.nvb);
 }
 
 // What a patch's (pixel, view) entries need of a view: x = t - h at the patch's first pixel relative
@@ -247,6 +261,7 @@ __global__ void __launch_bounds__(256, 4) update_kernel_p1(const __grid_constant
     __shared__ UpdateArgs sh_args;
     __shared__ double red_sh[1][32];
     __shared__ float part_sh[256];
+    grid_dependency_wait();
     grid_dependents_launch();
     VblockRuns runs(total_vblocks(one, bt));
     const UpdateArgs *ap = nullptr;
@@ -450,6 +465,18 @@ void forward_p1_dispatch(const FwdArgs &a, const Batch &b, int mode, int arith, 
     } else {
         if (arith == AR_KAHAN) fwd_p1_launch<AR_KAHAN, false>(a, b, mode, grid, st, pdl);
         else fwd_p1_launch<AR_FP32, false>(a, b, mode, grid, st, pdl);
+    }
+}
+
+void forward_mu_p1(const FwdArgs &a, const ImageArgs &m, int arith, cudaStream_t st)
+{
+    const int grid = a.nvb + m.nvb;
+    if (a.g.table) {
+        if (arith == AR_KAHAN) launch_pdl(fwd_mu_kernel_p1<AR_KAHAN, true>, grid, st, true, a, m, a.nvb);
+        else launch_pdl(fwd_mu_kernel_p1<AR_FP32, true>, grid, st, true, a, m, a.nvb);
+    } else {
+        if (arith == AR_KAHAN) launch_pdl(fwd_mu_kernel_p1<AR_KAHAN, false>, grid, st, true, a, m, a.nvb);
+        else launch_pdl(fwd_mu_kernel_p1<AR_FP32, false>, grid, st, true, a, m, a.nvb);
     }
 }
 

@@ -12,6 +12,7 @@
 #include <mutex>
 #include <vector>
 
+#include "image.cuh"
 #include "kernels.cuh"
 #include "profile.cuh"
 
@@ -32,11 +33,262 @@ namespace pet {
 // [c Lc, (c + 1) Lc) of its ray, Lc = ceil(nd / S), so that short subsets still fill the GPU; the
 // S partial sums of a (ray, group) are combined in chunk order through shared memory
 // (deterministic).  A persistent grid strides over the virtual blocks of one scan or a batch.
+template <int G, int AR, int MODE, bool SUB>
+__device__ __forceinline__ void fwd_vblock(const FwdArgs &a, int vloc, int nv,
+                                           typename ArithT<AR>::T *comb_s, typename ArithT<AR>::T *comb_e)
+{
+    static_assert(G == 8 || AR == AR_FP64, "single-plane FP32 scans run the kernels of plane1.cu");
+    using T = typename ArithT<AR>::T;
+    const GeoDev &g = a.g;
+    const int NG = g.NG, NB = g.NB, N = g.N, Pp = g.Pp, S = a.S, R = a.R;
+    const int nrays = a.nviews * NB;
+    constexpr bool kOrder = FWD_TILE_ORDER && (MODE != FWD_OBJECTIVE || FWD_TILE_ORDER > 1);
+    const int tpv_view = (NB + R - 1) / R;       // tiles of one view
+    const int ntiles = kOrder ? a.nviews * tpv_view : (nrays + R - 1) / R;
+    const bool lane_ok = (int)threadIdx.x < R * S * NG;
+    double obj[2] = {0.0, 0.0};
+    // with the centre-first order, virtual block v of a scan takes tiles v, v + nv, ...: a
+    // mix of long and short rays in every block (the objective mode's blocks hold several)
+    const int t_end = kOrder ? ntiles : min(ntiles, (vloc + 1) * a.tpv);
+    for (int tile = kOrder ? vloc : vloc * a.tpv; tile < t_end; tile += kOrder ? nv : 1) {
+    const int grp = threadIdx.x % NG;
+    const int c = (threadIdx.x / NG) % S;
+    const int rl = threadIdx.x / (NG * S);
+    // centre-first order: tile rank t -> (view, tile of the view) with the view's tiles
+    // taken from its centre outwards (c, c + 1, c - 1, c + 2, ...; c the lower middle), so
+    // that the longest rays run first and the launch ends on short ones
+    const int tr = kOrder ? tile / a.nviews : 0;
+    const int tb = (tpv_view - 1) / 2 + ((tr & 1) ? (tr + 1) / 2 : -(tr / 2));
+    const int bin = tb * R + rl;
+    // subset-local ray index u * NB + b
+    const int ray = kOrder ? (tile % a.nviews) * NB + bin : tile * R + rl;
+    const bool live = lane_ok && (kOrder ? bin < NB : ray < nrays);
+    GroupSum<G, AR> acc;
+    acc.zero();
+    if (live) {
+        const int slot = a.slot0 + ray / NB;
+        const ViewGeo &vw = g.views[slot];
+        const RayGeo &rg = g.rays[(size_t)a.slot0 * NB + ray];
+        const int ds = vw.xdrive ? 1 : N;        // pixel stride along the driving axis
+        const int cs = vw.xdrive ? N : 1;        // pixel stride along the cross axis
+        const T *img = reinterpret_cast<const T *>(a.img) + (size_t)grp * G;
+        const int Lc = (rg.nd + S - 1) / S;
+        const int k0 = c * Lc, k1 = min(rg.nd, k0 + Lc);
+        // sub-rays of the bin (SUB instantiations only; the others walk its centre line)
+        const int nsr = SUB ? g.R : 1;
+        if constexpr (AR == AR_FP64) {
+            const double step = vw.step, ast = fabs(vw.step), L = vw.L, im = vw.inv_minor;
+            for (int sr = 0; sr < nsr; ++sr)
+            for (int k = k0; k < k1; ++k) {
+                const int d = rg.d0 + k;
+                const double lo = fma((double)k, step, rg.lo + (2 * sr + 1 - nsr) * (SUB ? rg.sh : vw.half));
+                const double hi = lo + ast;
+                const double f0 = floor(lo), f1 = floor(hi);
+                const int r0 = (int)f0, r1 = (int)f1;
+                double l1 = (r1 != r0) ? (hi - f1) * im : 0.0;
+                double l0 = L - l1;
+                const bool ok0 = (unsigned)r0 < (unsigned)N, ok1 = (unsigned)r1 < (unsigned)N;
+                l0 = ok0 ? l0 : 0.0;
+                l1 = ok1 ? l1 : 0.0;
+                T x0[G], x1[G];
+                load_group<G, T>(img + (unsigned)(d * ds + (ok0 ? r0 : 0) * cs) * (unsigned)Pp, x0);
+                load_group<G, T>(img + (unsigned)(d * ds + (ok1 ? r1 : 0) * cs) * (unsigned)Pp, x1);
+                acc.add2terms(l0, x0, l1, x1);
+            }
+        } else if constexpr (G == 8 && FWD_FAST) {
+            // FP32 pairs, as below, with three changes: the fraction of the cross coordinate
+            // is read from its top 23 bits as the mantissa of a float in [1, 2) (no integer-
+            // to-float conversion), the pixel offsets advance incrementally along the driving
+            // axis, and the compensated sum takes blocks of 8 steps summed by FMAs (one
+            // compensated step per block instead of one per driving step)
+            const long long stp = vw.stepq, ast = vw.absstepq;
+            const float L = vw.Lf, imb = vw.inv_minorf;
+            const float *imf = reinterpret_cast<const float *>(img);
+            const unsigned dstep = (unsigned)ds * (unsigned)Pp, cstep = (unsigned)cs * (unsigned)Pp;
+            f2x sm[4], er[4], bl[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) { sm[q] = 0ull; er[q] = 0ull; bl[q] = 0ull; }
+            auto merge = [&]() {
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    if constexpr (AR == AR_KAHAN) {
+                        const f2x y = vadd(bl[q], er[q]);
+                        const f2x t = vadd(sm[q], y);
+                        er[q] = vsub(y, vsub(t, sm[q]));
+                        sm[q] = t;
+                    } else {
+                        sm[q] = vadd(sm[q], bl[q]);
+                    }
+                    bl[q] = 0ull;
+                }
+            };
+            int nb = 0;
+            for (int sr = 0; sr < nsr; ++sr) {
+            unsigned base = (unsigned)(rg.d0 + k0) * dstep;
+            long long lo = rg.loq + (long long)(2 * sr + 1 - nsr) * (SUB ? rg.shq : vw.halfq) + (long long)k0 * stp;
+            for (int k = k0; k < k1; ++k) {
+                const long long hi = lo + ast;
+                const int r0 = (int)(lo >> 32), r1 = (int)(hi >> 32);
+                const bool cross = r1 != r0;
+                const bool ok0 = (unsigned)r0 < (unsigned)N;
+                const bool ok1 = cross && (unsigned)r1 < (unsigned)N;
+                const float fr = __uint_as_float(0x3F800000u | ((unsigned)hi >> 9)) - 1.f;
+                const float t1 = cross ? fr * imb : 0.f;
+                const float l1 = ok1 ? t1 : 0.f;
+                const float l0 = ok0 ? L - t1 : 0.f;
+                const unsigned o0 = base + (ok0 ? (unsigned)r0 * cstep : 0u);
+                const unsigned o1 = base + (ok1 ? (unsigned)r1 * cstep : 0u);
+                f2x x0[4], x1[4];
+                load8x(imf + o0, x0);
+                load8x_if(imf + o1, ok1, x1);
+                const f2x W0 = vsplat(l0), W1 = vsplat(l1);
+#pragma unroll
+                for (int q = 0; q < 4; ++q) bl[q] = vfma(W1, x1[q], vfma(W0, x0[q], bl[q]));
+                if (++nb == 8) { merge(); nb = 0; }
+                lo += stp;
+                base += dstep;
+            }
+            }
+            merge();
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                float a0, a1, b0, b1;
+                vunpk(sm[q], a0, a1);
+                vunpk(er[q], b0, b1);
+                acc.set(2 * q, a0, b0);
+                acc.set(2 * q + 1, a1, b1);
+            }
+        } else if constexpr (G == 8) {
+            // FP32 pairs; the second pixel of a step is read only when the line crosses
+            // into it (l1 > 0), on about |slope| of the steps
+            const long long stp = vw.stepq, ast = vw.absstepq;
+            const float L = vw.Lf, im = vw.inv_minorf * kQ32;
+            const float *imf = reinterpret_cast<const float *>(img);
+            f2x sm[4], er[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) { sm[q] = 0ull; er[q] = 0ull; }
+            for (int sr = 0; sr < nsr; ++sr) {
+            long long lo = rg.loq + (long long)(2 * sr + 1 - nsr) * (SUB ? rg.shq : vw.halfq) + (long long)k0 * stp;
+            for (int k = k0; k < k1; ++k) {
+                const int d = rg.d0 + k;
+                const long long hi = lo + ast;
+                const int r0 = (int)(lo >> 32), r1 = (int)(hi >> 32);
+                const bool ok0 = (unsigned)r0 < (unsigned)N;
+                const bool ok1 = r1 != r0 && (unsigned)r1 < (unsigned)N;
+                const float l1 = ok1 ? __uint2float_rn((unsigned)(hi & 0xFFFFFFFFLL)) * im : 0.f;
+                const float l0 = ok0 ? L - (r1 != r0 ? __uint2float_rn((unsigned)(hi & 0xFFFFFFFFLL)) * im : 0.f) : 0.f;
+                f2x x0[4], x1[4];
+                load8x(imf + (unsigned)(d * ds + (ok0 ? r0 : 0) * cs) * (unsigned)Pp, x0);
+                load8x_if(imf + (unsigned)(d * ds + (ok1 ? r1 : 0) * cs) * (unsigned)Pp, ok1, x1);
+                const f2x W0 = vsplat(l0), W1 = vsplat(l1);
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    if constexpr (AR == AR_KAHAN) {
+                        const f2x y = vfma(W1, x1[q], vfma(W0, x0[q], er[q]));
+                        const f2x t = vadd(sm[q], y);
+                        er[q] = vsub(y, vsub(t, sm[q]));
+                        sm[q] = t;
+                    } else {
+                        sm[q] = vfma(W1, x1[q], vfma(W0, x0[q], sm[q]));
+                    }
+                }
+                lo += stp;
+            }
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                float a0, a1, b0, b1;
+                vunpk(sm[q], a0, a1);
+                vunpk(er[q], b0, b1);
+                acc.set(2 * q, a0, b0);
+                acc.set(2 * q + 1, a1, b1);
+            }
+        }
+    }
+    // combine the S chunks of each (ray, group) in chunk order
+    T tot[G];
+    if (S > 1) {
+        __syncthreads();
+#pragma unroll
+        for (int p = 0; p < G; ++p) {
+            comb_s[p * 256 + threadIdx.x] = acc.s_at(p);
+            comb_e[p * 256 + threadIdx.x] = acc.e_at(p);
+        }
+        __syncthreads();
+#pragma unroll
+        for (int p = 0; p < G; ++p) {
+            T s0 = acc.s_at(p), e0 = acc.e_at(p);
+            if (c == 0 && lane_ok) {            // idle lanes (>= R S NG) have no chunks
+                for (int cc = 1; cc < S; ++cc) {
+                    const int o = p * 256 + (rl * S + cc) * NG + grp;
+                    if constexpr (AR == AR_KAHAN) {
+                        const T y = comb_s[o] + (comb_e[o] + e0);
+                        const T t = s0 + y;
+                        e0 = y - (t - s0);
+                        s0 = t;
+                    } else {
+                        s0 += comb_s[o];
+                    }
+                }
+            }
+            tot[p] = s0 + e0;
+        }
+    } else {
+#pragma unroll
+        for (int p = 0; p < G; ++p) tot[p] = acc.value(p);
+    }
+    if (live && c == 0) {
+        const size_t o = (size_t)ray * Pp + (size_t)grp * G;
+        const T scale = (T)g.scale;
+        if constexpr (MODE == FWD_PLAIN) {
+            T y[G];
+#pragma unroll
+            for (int p = 0; p < G; ++p) y[p] = scale * tot[p];
+            store_group<G, T>(reinterpret_cast<T *>(a.out) + o, y);
+        } else {
+            int cnt[G];
+            float gam[G];
+            load_group_i<G>(a.counts + o, cnt);
+            load_group<G, float>(a.gamma + o, gam);
+            // per-bin detection factors: the system matrix is diag(a) A, so the mean is
+            // a_i (A f)_i + gamma_i and the backprojected ratio carries a_i (a_i = 1, exact
+            // in the products, without factors)
+            const float *mp = a.mult ? a.mult + o : nullptr;
+            if constexpr (MODE == FWD_RATIO) {
+                T w[G];
+#pragma unroll
+                for (int p = 0; p < G; ++p) {
+                    const T m = mp ? (T)__ldg(mp + p) : T(1);
+                    const T y = scale * (tot[p] * m) + (T)gam[p];
+                    w[p] = (grp * G + p < g.P) ? m * (T(1) - (T)cnt[p] / y) : T(0);
+                }
+                store_group<G, T>(reinterpret_cast<T *>(a.out) + o, w);
+            } else {
+                // the likelihood terms in FP64 in every mode: ln((double) Af + gamma)
+                T s_af = T(0);
+                double s_gl = 0.0;
+#pragma unroll
+                for (int p = 0; p < G; ++p) {
+                    if (grp * G + p < g.P) {
+                        const T af = scale * (mp ? tot[p] * (T)__ldg(mp + p) : tot[p]);
+                        s_af += af;
+                        if (cnt[p] != 0) s_gl += (double)cnt[p] * log((double)af + (double)gam[p]);
+                    }
+                }
+                obj[0] += (double)s_af;
+                obj[1] += s_gl;
+            }
+        }
+    }
+    }  // tiles of this virtual block
+    if constexpr (MODE == FWD_OBJECTIVE) grid_reduce<2>(obj, a.red, a.result, vloc, nv);
+}
+
 template <int G, int AR, int MODE, bool SUB = false>
 __global__ void __launch_bounds__(256, 3) fwd_kernel(const __grid_constant__ FwdArgs one, const Batch bt)
 {
     grid_dependency_wait();                      // before any memory access
-    static_assert(G == 8 || AR == AR_FP64, "single-plane FP32 scans run the kernels of plane1.cu");
+    grid_dependents_launch();                    // the update may be scheduled behind this kernel
     using T = typename ArithT<AR>::T;
     __shared__ T comb_s[256 * G];
     __shared__ T comb_e[256 * G];
@@ -45,250 +297,26 @@ __global__ void __launch_bounds__(256, 3) fwd_kernel(const __grid_constant__ Fwd
     for (int vb = blockIdx.x; vb < total; vb += gridDim.x) {
         int vloc, nv;
         const FwdArgs &a = scan_args(one, bt, vb, vloc, nv, sh_args);
-        const GeoDev &g = a.g;
-        const int NG = g.NG, NB = g.NB, N = g.N, Pp = g.Pp, S = a.S, R = a.R;
-        const int nrays = a.nviews * NB;
-        constexpr bool kOrder = FWD_TILE_ORDER && (MODE != FWD_OBJECTIVE || FWD_TILE_ORDER > 1);
-        const int tpv_view = (NB + R - 1) / R;       // tiles of one view
-        const int ntiles = kOrder ? a.nviews * tpv_view : (nrays + R - 1) / R;
-        const bool lane_ok = (int)threadIdx.x < R * S * NG;
-        double obj[2] = {0.0, 0.0};
-        // with the centre-first order, virtual block v of a scan takes tiles v, v + nv, ...: a
-        // mix of long and short rays in every block (the objective mode's blocks hold several)
-        const int t_end = kOrder ? ntiles : min(ntiles, (vloc + 1) * a.tpv);
-        for (int tile = kOrder ? vloc : vloc * a.tpv; tile < t_end; tile += kOrder ? nv : 1) {
-        const int grp = threadIdx.x % NG;
-        const int c = (threadIdx.x / NG) % S;
-        const int rl = threadIdx.x / (NG * S);
-        // centre-first order: tile rank t -> (view, tile of the view) with the view's tiles
-        // taken from its centre outwards (c, c + 1, c - 1, c + 2, ...; c the lower middle), so
-        // that the longest rays run first and the launch ends on short ones
-        const int tr = kOrder ? tile / a.nviews : 0;
-        const int tb = (tpv_view - 1) / 2 + ((tr & 1) ? (tr + 1) / 2 : -(tr / 2));
-        const int bin = tb * R + rl;
-        // subset-local ray index u * NB + b
-        const int ray = kOrder ? (tile % a.nviews) * NB + bin : tile * R + rl;
-        const bool live = lane_ok && (kOrder ? bin < NB : ray < nrays);
-        GroupSum<G, AR> acc;
-        acc.zero();
-        if (live) {
-            const int slot = a.slot0 + ray / NB;
-            const ViewGeo &vw = g.views[slot];
-            const RayGeo &rg = g.rays[(size_t)a.slot0 * NB + ray];
-            const int ds = vw.xdrive ? 1 : N;        // pixel stride along the driving axis
-            const int cs = vw.xdrive ? N : 1;        // pixel stride along the cross axis
-            const T *img = reinterpret_cast<const T *>(a.img) + (size_t)grp * G;
-            const int Lc = (rg.nd + S - 1) / S;
-            const int k0 = c * Lc, k1 = min(rg.nd, k0 + Lc);
-            // sub-rays of the bin (SUB instantiations only; the others walk its centre line)
-            const int nsr = SUB ? g.R : 1;
-            if constexpr (AR == AR_FP64) {
-                const double step = vw.step, ast = fabs(vw.step), L = vw.L, im = vw.inv_minor;
-                for (int sr = 0; sr < nsr; ++sr)
-                for (int k = k0; k < k1; ++k) {
-                    const int d = rg.d0 + k;
-                    const double lo = fma((double)k, step, rg.lo + (2 * sr + 1 - nsr) * (SUB ? rg.sh : vw.half));
-                    const double hi = lo + ast;
-                    const double f0 = floor(lo), f1 = floor(hi);
-                    const int r0 = (int)f0, r1 = (int)f1;
-                    double l1 = (r1 != r0) ? (hi - f1) * im : 0.0;
-                    double l0 = L - l1;
-                    const bool ok0 = (unsigned)r0 < (unsigned)N, ok1 = (unsigned)r1 < (unsigned)N;
-                    l0 = ok0 ? l0 : 0.0;
-                    l1 = ok1 ? l1 : 0.0;
-                    T x0[G], x1[G];
-                    load_group<G, T>(img + (unsigned)(d * ds + (ok0 ? r0 : 0) * cs) * (unsigned)Pp, x0);
-                    load_group<G, T>(img + (unsigned)(d * ds + (ok1 ? r1 : 0) * cs) * (unsigned)Pp, x1);
-                    acc.add2terms(l0, x0, l1, x1);
-                }
-            } else if constexpr (G == 8 && FWD_FAST) {
-                // FP32 pairs, as below, with three changes: the fraction of the cross coordinate
-                // is read from its top 23 bits as the mantissa of a float in [1, 2) (no integer-
-                // to-float conversion), the pixel offsets advance incrementally along the driving
-                // axis, and the compensated sum takes blocks of 8 steps summed by FMAs (one
-                // compensated step per block instead of one per driving step)
-                const long long stp = vw.stepq, ast = vw.absstepq;
-                const float L = vw.Lf, imb = vw.inv_minorf;
-                const float *imf = reinterpret_cast<const float *>(img);
-                const unsigned dstep = (unsigned)ds * (unsigned)Pp, cstep = (unsigned)cs * (unsigned)Pp;
-                f2x sm[4], er[4], bl[4];
-#pragma unroll
-                for (int q = 0; q < 4; ++q) { sm[q] = 0ull; er[q] = 0ull; bl[q] = 0ull; }
-                auto merge = [&]() {
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        if constexpr (AR == AR_KAHAN) {
-                            const f2x y = vadd(bl[q], er[q]);
-                            const f2x t = vadd(sm[q], y);
-                            er[q] = vsub(y, vsub(t, sm[q]));
-                            sm[q] = t;
-                        } else {
-                            sm[q] = vadd(sm[q], bl[q]);
-                        }
-                        bl[q] = 0ull;
-                    }
-                };
-                int nb = 0;
-                for (int sr = 0; sr < nsr; ++sr) {
-                unsigned base = (unsigned)(rg.d0 + k0) * dstep;
-                long long lo = rg.loq + (long long)(2 * sr + 1 - nsr) * (SUB ? rg.shq : vw.halfq) + (long long)k0 * stp;
-                for (int k = k0; k < k1; ++k) {
-                    const long long hi = lo + ast;
-                    const int r0 = (int)(lo >> 32), r1 = (int)(hi >> 32);
-                    const bool cross = r1 != r0;
-                    const bool ok0 = (unsigned)r0 < (unsigned)N;
-                    const bool ok1 = cross && (unsigned)r1 < (unsigned)N;
-                    const float fr = __uint_as_float(0x3F800000u | ((unsigned)hi >> 9)) - 1.f;
-                    const float t1 = cross ? fr * imb : 0.f;
-                    const float l1 = ok1 ? t1 : 0.f;
-                    const float l0 = ok0 ? L - t1 : 0.f;
-                    const unsigned o0 = base + (ok0 ? (unsigned)r0 * cstep : 0u);
-                    const unsigned o1 = base + (ok1 ? (unsigned)r1 * cstep : 0u);
-                    f2x x0[4], x1[4];
-                    load8x(imf + o0, x0);
-                    load8x_if(imf + o1, ok1, x1);
-                    const f2x W0 = vsplat(l0), W1 = vsplat(l1);
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) bl[q] = vfma(W1, x1[q], vfma(W0, x0[q], bl[q]));
-                    if (++nb == 8) { merge(); nb = 0; }
-                    lo += stp;
-                    base += dstep;
-                }
-                }
-                merge();
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    float a0, a1, b0, b1;
-                    vunpk(sm[q], a0, a1);
-                    vunpk(er[q], b0, b1);
-                    acc.set(2 * q, a0, b0);
-                    acc.set(2 * q + 1, a1, b1);
-                }
-            } else if constexpr (G == 8) {
-                // FP32 pairs; the second pixel of a step is read only when the line crosses
-                // into it (l1 > 0), on about |slope| of the steps
-                const long long stp = vw.stepq, ast = vw.absstepq;
-                const float L = vw.Lf, im = vw.inv_minorf * kQ32;
-                const float *imf = reinterpret_cast<const float *>(img);
-                f2x sm[4], er[4];
-#pragma unroll
-                for (int q = 0; q < 4; ++q) { sm[q] = 0ull; er[q] = 0ull; }
-                for (int sr = 0; sr < nsr; ++sr) {
-                long long lo = rg.loq + (long long)(2 * sr + 1 - nsr) * (SUB ? rg.shq : vw.halfq) + (long long)k0 * stp;
-                for (int k = k0; k < k1; ++k) {
-                    const int d = rg.d0 + k;
-                    const long long hi = lo + ast;
-                    const int r0 = (int)(lo >> 32), r1 = (int)(hi >> 32);
-                    const bool ok0 = (unsigned)r0 < (unsigned)N;
-                    const bool ok1 = r1 != r0 && (unsigned)r1 < (unsigned)N;
-                    const float l1 = ok1 ? __uint2float_rn((unsigned)(hi & 0xFFFFFFFFLL)) * im : 0.f;
-                    const float l0 = ok0 ? L - (r1 != r0 ? __uint2float_rn((unsigned)(hi & 0xFFFFFFFFLL)) * im : 0.f) : 0.f;
-                    f2x x0[4], x1[4];
-                    load8x(imf + (unsigned)(d * ds + (ok0 ? r0 : 0) * cs) * (unsigned)Pp, x0);
-                    load8x_if(imf + (unsigned)(d * ds + (ok1 ? r1 : 0) * cs) * (unsigned)Pp, ok1, x1);
-                    const f2x W0 = vsplat(l0), W1 = vsplat(l1);
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        if constexpr (AR == AR_KAHAN) {
-                            const f2x y = vfma(W1, x1[q], vfma(W0, x0[q], er[q]));
-                            const f2x t = vadd(sm[q], y);
-                            er[q] = vsub(y, vsub(t, sm[q]));
-                            sm[q] = t;
-                        } else {
-                            sm[q] = vfma(W1, x1[q], vfma(W0, x0[q], sm[q]));
-                        }
-                    }
-                    lo += stp;
-                }
-                }
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    float a0, a1, b0, b1;
-                    vunpk(sm[q], a0, a1);
-                    vunpk(er[q], b0, b1);
-                    acc.set(2 * q, a0, b0);
-                    acc.set(2 * q + 1, a1, b1);
-                }
-            }
-        }
-        // combine the S chunks of each (ray, group) in chunk order
-        T tot[G];
-        if (S > 1) {
-            __syncthreads();
-#pragma unroll
-            for (int p = 0; p < G; ++p) {
-                comb_s[p * 256 + threadIdx.x] = acc.s_at(p);
-                comb_e[p * 256 + threadIdx.x] = acc.e_at(p);
-            }
-            __syncthreads();
-#pragma unroll
-            for (int p = 0; p < G; ++p) {
-                T s0 = acc.s_at(p), e0 = acc.e_at(p);
-                if (c == 0 && lane_ok) {            // idle lanes (>= R S NG) have no chunks
-                    for (int cc = 1; cc < S; ++cc) {
-                        const int o = p * 256 + (rl * S + cc) * NG + grp;
-                        if constexpr (AR == AR_KAHAN) {
-                            const T y = comb_s[o] + (comb_e[o] + e0);
-                            const T t = s0 + y;
-                            e0 = y - (t - s0);
-                            s0 = t;
-                        } else {
-                            s0 += comb_s[o];
-                        }
-                    }
-                }
-                tot[p] = s0 + e0;
-            }
-        } else {
-#pragma unroll
-            for (int p = 0; p < G; ++p) tot[p] = acc.value(p);
-        }
-        if (live && c == 0) {
-            const size_t o = (size_t)ray * Pp + (size_t)grp * G;
-            const T scale = (T)g.scale;
-            if constexpr (MODE == FWD_PLAIN) {
-                T y[G];
-#pragma unroll
-                for (int p = 0; p < G; ++p) y[p] = scale * tot[p];
-                store_group<G, T>(reinterpret_cast<T *>(a.out) + o, y);
-            } else {
-                int cnt[G];
-                float gam[G];
-                load_group_i<G>(a.counts + o, cnt);
-                load_group<G, float>(a.gamma + o, gam);
-                // per-bin detection factors: the system matrix is diag(a) A, so the mean is
-                // a_i (A f)_i + gamma_i and the backprojected ratio carries a_i (a_i = 1, exact
-                // in the products, without factors)
-                const float *mp = a.mult ? a.mult + o : nullptr;
-                if constexpr (MODE == FWD_RATIO) {
-                    T w[G];
-#pragma unroll
-                    for (int p = 0; p < G; ++p) {
-                        const T m = mp ? (T)__ldg(mp + p) : T(1);
-                        const T y = scale * (tot[p] * m) + (T)gam[p];
-                        w[p] = (grp * G + p < g.P) ? m * (T(1) - (T)cnt[p] / y) : T(0);
-                    }
-                    store_group<G, T>(reinterpret_cast<T *>(a.out) + o, w);
-                } else {
-                    // the likelihood terms in FP64 in every mode: ln((double) Af + gamma)
-                    T s_af = T(0);
-                    double s_gl = 0.0;
-#pragma unroll
-                    for (int p = 0; p < G; ++p) {
-                        if (grp * G + p < g.P) {
-                            const T af = scale * (mp ? tot[p] * (T)__ldg(mp + p) : tot[p]);
-                            s_af += af;
-                            if (cnt[p] != 0) s_gl += (double)cnt[p] * log((double)af + (double)gam[p]);
-                        }
-                    }
-                    obj[0] += (double)s_af;
-                    obj[1] += s_gl;
-                }
-            }
-        }
-        }  // tiles of this virtual block
-        if constexpr (MODE == FWD_OBJECTIVE) grid_reduce<2>(obj, a.red, a.result, vloc, nv);
+        fwd_vblock<G, AR, MODE, SUB>(a, vloc, nv, comb_s, comb_e);
     }
+}
+
+// The subset projection and the mu pass of one scan (8-plane groups, FP32, in-plane prior) in one
+// launch: blocks below nfwd project, the others run the mu pass.  Both only read f, and the mu
+// pass's short blocks come last and fill the projection's tail; as a launch of its own on a side
+// stream it cost a fork and a join of events per subiteration and kept the update from being
+// scheduled behind the projection.
+template <int AR, bool SUB>
+__global__ void __launch_bounds__(256, 3) fwd_mu_kernel(const __grid_constant__ FwdArgs fwd,
+                                                        const __grid_constant__ ImageArgs mu, int nfwd)
+{
+    grid_dependency_wait();
+    grid_dependents_launch();
+    __shared__ float comb_s[256 * 8];
+    __shared__ float comb_e[256 * 8];
+    const int vb = (int)blockIdx.x;
+    if (vb < nfwd) fwd_vblock<8, AR, FWD_RATIO, SUB>(fwd, vb, nfwd, comb_s, comb_e);
+    else mu_x8_vblock(mu, vb - nfwd, mu.nvb);
 }
 
 template <int G, int AR>
@@ -418,6 +446,35 @@ pet_status launch_forward(const FwdArgs &a0, int mode, int arith, cudaStream_t s
     else fwd_dispatch<8>(a, b, mode, arith, grid, st, after_kernel);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "fwd_kernel launch");
+    return PET_OK;
+}
+
+bool mu_joins_forward(const FwdArgs &a, const ImageArgs &mu, int arith)
+{
+    return arith != AR_FP64 && a.g.T == 1 && (a.g.G == 1 || !mu.z3);
+}
+
+pet_status launch_forward_mu(const FwdArgs &a0, const ImageArgs &m0, int arith, cudaStream_t st)
+{
+    FwdArgs a = a0;
+    ImageArgs m = m0;
+    forward_shape(a, FWD_RATIO, arith);
+    mu_shape(m, arith);
+    LaunchScope ls(PET_K_FORWARD_RATIO, st);
+    if (a.g.G == 1) {
+        forward_mu_p1(a, m, arith, st);
+    } else {
+        const int grid = a.nvb + m.nvb;
+        if (a.g.table) {
+            if (arith == AR_KAHAN) launch_pdl(fwd_mu_kernel<AR_KAHAN, true>, grid, st, true, a, m, a.nvb);
+            else launch_pdl(fwd_mu_kernel<AR_FP32, true>, grid, st, true, a, m, a.nvb);
+        } else {
+            if (arith == AR_KAHAN) launch_pdl(fwd_mu_kernel<AR_KAHAN, false>, grid, st, true, a, m, a.nvb);
+            else launch_pdl(fwd_mu_kernel<AR_FP32, false>, grid, st, true, a, m, a.nvb);
+        }
+    }
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return cuda_fail(e, "fwd_mu_kernel launch");
     return PET_OK;
 }
 

@@ -14,9 +14,6 @@
 #ifndef UPDATE_G1_BLOCKS
 #define UPDATE_G1_BLOCKS 4      // resident blocks per SM the single-plane update kernel is built for
 #endif
-#ifndef UPDATE_X8_BLOCKS
-#define UPDATE_X8_BLOCKS 3      // resident blocks per SM the packed update kernel is built for
-#endif
 
 namespace pet {
 
@@ -54,7 +51,8 @@ __global__ void __launch_bounds__(256, G == 1 ? UPDATE_G1_BLOCKS : 3) update_ker
 {
     using T = typename ArithT<AR>::T;
     __shared__ BpTable<KC, AR> tb;
-    grid_dependents_launch();                    // as in update_kernel_x8
+    grid_dependency_wait();                      // as in update_kernel_x8
+    grid_dependents_launch();
     const int total = total_vblocks(one, bt);
     __shared__ UpdateArgs sh_args;
     for (int vb = blockIdx.x; vb < total; vb += gridDim.x) {
@@ -158,214 +156,6 @@ __global__ void __launch_bounds__(256, G == 1 ? UPDATE_G1_BLOCKS : 3) update_ker
                 store_group<G, T>(reinterpret_cast<T *>(a.zbuf) + o, out);
                 store_group<G, T>(reinterpret_cast<T *>(a.wbuf) + o, wv);
             }
-        }
-        double v[1] = {(double)part};
-        grid_reduce<1>(v, a.red, a.sum_fout, vloc, nv);
-    }
-}
-
-// FP32 update for 8-plane groups held as four f32x2 pairs.  Same step as update_kernel, with:
-//   - the 3x3 stencil loading every neighbour with missing ones (image border) replaced by the
-//     centre value: their RDP term is exactly zero (d = 0) and the Matlab-style gradient becomes
-//     the one-sided difference, as in the generic stencil;
-//   - the RDP pair term written as d (den + 2 f_k + eps) / den^2 (the numerator
-//     gamma_R |d| + f_j + 3 f_k + 2 eps equals den + 2 f_k + eps), from one reciprocal of den;
-//   - nu = P_{nu1}^{nu2}(mean(mu) / mu) from 1 / mu = min(100, mean(f) / |grad f|);
-//   - the step folded into two per-plane constants before the gather,
-//     f^{k,i} = P_t(A + B b) with A = f - c (beta/M) grad R, B = -c scale, c = lambda alpha nu S,
-//     so that only A, B and the sums of b = A_i^T w stay live across the gather.
-template <int KC, int AR>
-__global__ void __launch_bounds__(256, UPDATE_X8_BLOCKS) update_kernel_x8(
-    const __grid_constant__ UpdateArgs one, const Batch bt)
-{
-    static_assert(AR != AR_FP64, "FP32 arithmetic only");
-    // 16 KB of (pixel, view) entries: the rest of the SM's shared memory stays L1 for the gather
-    using Table = BpTable<KC, AR, 1024 / (KC > 2 ? 2 : 1)>;
-    __shared__ Table tb;
-    // the next subiteration's projection (launched after this kernel with programmatic stream
-    // serialization) may be scheduled as this kernel's blocks retire; it waits for completion
-    grid_dependents_launch();
-    const int total = total_vblocks(one, bt);
-    __shared__ UpdateArgs sh_args;
-    for (int vb = blockIdx.x; vb < total; vb += gridDim.x) {
-        int vloc, nv;
-        const UpdateArgs &a = scan_args(one, bt, vb, vloc, nv, sh_args);
-        const GeoDev &g = a.g;
-        const int N = g.N, NG = g.NG, npix = N * N;
-        const unsigned Pp = (unsigned)g.Pp;
-        const int TP = 256 / NG;
-        const int pl = threadIdx.x / NG, grp = threadIdx.x % NG;
-        const int VC = max(1, min(a.nviews, Table::CAP / TP));
-        const bool dyn = a.nu_mode == 1 || a.nu_mode == 2;
-        const double q = (double)npix * g.P;
-        // per-scan scalars in FP32 (an FP64 division per thread is costly at GB300's FP64 rate)
-        const float mean_f = dyn ? (float)*a.sum_f / (float)q : 1.f;
-        const float mean_mu = dyn ? (float)*a.sum_mu / (float)q : 1.f;
-        const float U = a.fs_U, tt = a.fs_t;
-        // eps >= 1e-30 keeps 1/den finite, so that a zero-difference term stays exactly zero
-        const float eps = fmaxf(a.fs_eps, 1e-30f);
-        const float *f = reinterpret_cast<const float *>(a.f) + grp * 8;
-        const float *w = reinterpret_cast<const float *>(a.w) + grp * 8;
-        const float *invp = reinterpret_cast<const float *>(a.invp);
-        const int ntiles = (npix + TP - 1) / TP;
-        // the subset's precomputed entries (one contiguous block per tile) when two tiles' entries
-        // fit the table: double-buffered, the next tile's block copied with cp.async while this
-        // tile is gathered and the next one's stencil runs (one barrier per tile)
-        const bool pre = a.bptab && 2 * a.nviews * TP <= Table::CAP;
-        const int t0 = vloc * a.tpv, t1 = min(ntiles, (vloc + 1) * a.tpv);
-        auto copy_tile = [&](int tile) {
-            const int tbytes = a.nviews * TP * (int)sizeof(typename Table::E);
-            const char *src = static_cast<const char *>(a.bptab) + (size_t)tile * tbytes;
-            char *dst = reinterpret_cast<char *>(tb.e) + ((tile - t0) & 1) * tbytes;
-            for (int o = threadIdx.x * 16; o < tbytes; o += 256 * 16) cp_async16(dst + o, src + o);
-            cp_async_commit();
-        };
-        if (pre && t0 < t1) copy_tile(t0);
-        float part = 0.f;
-        for (int tile = t0; tile < t1; ++tile) {
-            const int j0 = tile * TP, j = j0 + pl;
-            const bool active = pl < TP && j < npix;
-            f2x A[4], B[4];
-            if (active) {
-                const int ix = j % N, iy = j / N;
-                const unsigned jc = (unsigned)j;
-                const unsigned xm = ix > 0 ? jc - 1 : jc, xp = ix < N - 1 ? jc + 1 : jc;
-                const unsigned ym = iy > 0 ? jc - N : jc, yp = iy < N - 1 ? jc + N : jc;
-                const f2x GR = vsplat(a.fs_gamma_r), EP = vsplat(eps), TWO = vsplat(2.f);
-                f2x c[4], ce[4], gr[4], g2[4], nb0[4], nb1[4];
-                load8x(f + jc * Pp, c);
-#pragma unroll
-                for (int k = 0; k < 4; ++k) { ce[k] = vadd(c[k], EP); gr[k] = 0ull; }
-                auto rdp = [&](const f2x(&x)[4]) {
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        const f2x d = vsub(c[k], x[k]);
-                        const f2x den = vfma(GR, vabs(d), vadd(ce[k], x[k]));
-                        const f2x num = vadd(den, vfma(TWO, x[k], EP));
-                        const f2x r = vrcp(den);
-                        gr[k] = vfma(vmul(d, vmul(num, r)), r, gr[k]);
-                    }
-                };
-                // axial neighbours: RDP terms and the Matlab-style gradient
-                load8x(f + xm * Pp, nb0);
-                load8x(f + xp * Pp, nb1);
-                rdp(nb0);
-                rdp(nb1);
-                if (dyn) {
-                    const f2x HX = vsplat((ix > 0 && ix < N - 1) ? 0.5f : 1.f);
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        const f2x t = vmul(HX, vsub(nb1[k], nb0[k]));
-                        g2[k] = vmul(t, t);
-                    }
-                }
-                load8x(f + ym * Pp, nb0);
-                load8x(f + yp * Pp, nb1);
-                rdp(nb0);
-                rdp(nb1);
-                f2x nu[4];
-                if (dyn) {
-                    const f2x HY = vsplat((iy > 0 && iy < N - 1) ? 0.5f : 1.f);
-                    const float nu1 = a.fs_nu1, nu2 = a.fs_nu2;
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        const f2x t = vmul(HY, vsub(nb1[k], nb0[k]));
-                        float r0, r1;
-                        vunpk(vrsqrt(vfma(t, t, g2[k])), r0, r1);
-                        // 1 / mu = 1 / max(0.01, |grad f| / mean f) = min(100, mean f / |grad f|)
-                        r0 = fminf(100.f, r0 * mean_f);
-                        r1 = fminf(100.f, r1 * mean_f);
-                        nu[k] = vpk(fminf(fmaxf(mean_mu * r0, nu1), nu2),
-                                    fminf(fmaxf(mean_mu * r1, nu1), nu2));
-                    }
-                    if (a.nu_mode == 2)
-                        store8x(reinterpret_cast<float *>(a.nu_frozen) + jc * Pp + grp * 8, nu);
-                } else if (a.nu_mode == 3) {
-                    load8x(reinterpret_cast<const float *>(a.nu_frozen) + jc * Pp + grp * 8, nu);
-                } else {
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) nu[k] = vsplat(1.f);
-                }
-                // diagonal neighbours
-                const unsigned dm = iy > 0 ? jc - N : jc, dp = iy < N - 1 ? jc + N : jc;
-                load8x(f + (ix > 0 && iy > 0 ? dm - 1 : jc) * Pp, nb0);
-                load8x(f + (ix < N - 1 && iy > 0 ? dm + 1 : jc) * Pp, nb1);
-                rdp(nb0);
-                rdp(nb1);
-                load8x(f + (ix > 0 && iy < N - 1 ? dp - 1 : jc) * Pp, nb0);
-                load8x(f + (ix < N - 1 && iy < N - 1 ? dp + 1 : jc) * Pp, nb1);
-                rdp(nb0);
-                rdp(nb1);
-                // c = lambda alpha nu S, S = min(f, U - f) / p;  A = f - c (beta/M) 2 gr;  B = -c scale
-                const f2x NK = vsplat(-a.fs_lam * invp[j] * a.fs_ips);
-                const f2x BM = vsplat(2.f * a.fs_bm), SC = vsplat(a.fs_scale);
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    float c0, c1;
-                    vunpk(c[k], c0, c1);
-                    const f2x S = vpk(fminf(c0, U - c0), fminf(c1, U - c1));
-                    const f2x cn = vmul(vmul(nu[k], S), NK);
-                    A[k] = vfma(cn, vmul(BM, gr[k]), c[k]);
-                    B[k] = vmul(cn, SC);
-                }
-            }
-            // gather backprojection b = A_i^T w with the tile's shared (pixel, view) weights
-            f2x sm[4], er[4];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) { sm[k] = 0ull; er[k] = 0ull; }
-            for (int u0 = 0; u0 < a.nviews; u0 += VC) {
-                const int nvc = min(VC, a.nviews - u0);
-                if (pre) {
-                    cp_async_wait_all();             // this tile's block (this thread's part)
-                    __syncthreads();                 // all parts; the previous gather is done
-                    if (tile + 1 < t1) copy_tile(tile + 1);
-                } else {
-                    __syncthreads();
-                    bp_fill<KC, AR>(g, a.slot0, u0, nvc, j0, TP, tb);
-                    __syncthreads();
-                }
-                if (!active) continue;
-                const typename Table::E *te = tb.e + (pre ? ((tile - t0) & 1) * a.nviews * TP : 0);
-                for (int uu = 0; uu < nvc; ++uu) {
-                    const typename Table::E ent = te[uu * TP + pl];
-                    const float *row = w + ent.off;
-#pragma unroll
-                    for (int kb = 0; kb < KC; kb += 2) {
-                        f2x x0[4], x1[4];
-                        load8x(row + kb * Pp, x0);
-                        load8x(row + (kb + 1) * Pp, x1);
-                        const f2x W0 = vsplat(ent.w[kb]), W1 = vsplat(ent.w[kb + 1]);
-#pragma unroll
-                        for (int k = 0; k < 4; ++k) {
-                            if constexpr (AR == AR_KAHAN) {
-                                const f2x y = vfma(W1, x1[k], vfma(W0, x0[k], er[k]));
-                                const f2x t = vadd(sm[k], y);
-                                er[k] = vsub(y, vsub(t, sm[k]));
-                                sm[k] = t;
-                            } else {
-                                sm[k] = vfma(W1, x1[k], vfma(W0, x0[k], sm[k]));
-                            }
-                        }
-                    }
-                }
-            }
-            if (!active) continue;
-            // step and clamp P_t
-            f2x out[4];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const f2x b = AR == AR_KAHAN ? vadd(sm[k], er[k]) : sm[k];
-                float f0, f1;
-                vunpk(vfma(B[k], b, A[k]), f0, f1);
-                f0 = f0 <= 0.f ? tt : (f0 >= U ? U - tt : f0);
-                f1 = f1 <= 0.f ? tt : (f1 >= U ? U - tt : f1);
-                const int p0 = grp * 8 + 2 * k;
-                f0 = p0 < g.P ? f0 : 0.f;
-                f1 = p0 + 1 < g.P ? f1 : 0.f;
-                part += f0 + f1;
-                out[k] = vpk(f0, f1);
-            }
-            store8x(reinterpret_cast<float *>(a.fout) + (unsigned)j * Pp + grp * 8, out);
         }
         double v[1] = {(double)part};
         grid_reduce<1>(v, a.red, a.sum_fout, vloc, nv);
@@ -497,10 +287,7 @@ __global__ void __launch_bounds__(256) image_kernel(const __grid_constant__ Imag
     }
 }
 
-// FP32 mu pass for 8-plane groups: sum over voxels of mu = max(0.01, |grad f| / mean(f))
-// (Matlab-style gradient: central differences inside, one-sided at the border, where the
-// missing neighbour is the centre value).  Thread layout of the update kernel (pixel x plane
-// group, TP = 256 / NG pixels per tile); a virtual block takes a.ipt tiles.
+// The mu pass alone (batches, and scans whose pass does not join the projection).
 __global__ void __launch_bounds__(256) mu_kernel_x8(const __grid_constant__ ImageArgs one, const Batch bt)
 {
     const int total = total_vblocks(one, bt);
@@ -508,44 +295,7 @@ __global__ void __launch_bounds__(256) mu_kernel_x8(const __grid_constant__ Imag
     for (int vb = blockIdx.x; vb < total; vb += gridDim.x) {
         int vloc, nv;
         const ImageArgs &a = scan_args(one, bt, vb, vloc, nv, sh_args);
-        const GeoDev &g = a.g;
-        const int N = g.N, NG = g.NG, npix = N * N;
-        const unsigned Pp = (unsigned)g.Pp;
-        const int TP = 256 / NG;
-        const int pl = threadIdx.x / NG, grp = threadIdx.x % NG;
-        const int ntiles = (npix + TP - 1) / TP;
-        const float inv_mean_f = (float)((double)npix * g.P) / (float)*a.sum_f;
-        const float *f = reinterpret_cast<const float *>(a.f) + grp * 8;
-        const int nvalid = min(8, g.P - grp * 8);             // real planes of this group
-        float part = 0.f;
-        for (int tile = vloc * a.ipt; tile < min(ntiles, (vloc + 1) * a.ipt); ++tile) {
-            const int j = tile * TP + pl;
-            if (pl >= TP || j >= npix) continue;
-            const int ix = j % N, iy = j / N;
-            const unsigned jc = (unsigned)j;
-            f2x w_[4], e_[4], n_[4], s_[4];
-            load8x(f + (ix > 0 ? jc - 1 : jc) * Pp, w_);
-            load8x(f + (ix < N - 1 ? jc + 1 : jc) * Pp, e_);
-            load8x(f + (iy > 0 ? jc - N : jc) * Pp, n_);
-            load8x(f + (iy < N - 1 ? jc + N : jc) * Pp, s_);
-            const f2x HX = vsplat((ix > 0 && ix < N - 1) ? 0.5f : 1.f);
-            const f2x HY = vsplat((iy > 0 && iy < N - 1) ? 0.5f : 1.f);
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const f2x gx = vmul(HX, vsub(e_[k], w_[k])), gy = vmul(HY, vsub(s_[k], n_[k]));
-                const f2x x2 = vfma(gx, gx, vmul(gy, gy));
-                float x0, x1, r0, r1;
-                vunpk(x2, x0, x1);
-                vunpk(vrsqrt(x2), r0, r1);
-                // |grad f|^2 below the smallest normal float (|grad f| < 1.1e-19, met on decayed
-                // backgrounds) counts as zero: mu = 0.01 there, and the flushed rsqrt would be inf
-                const float m0 = fmaxf(0.01f, x0 >= 1.17549435e-38f ? x0 * r0 * inv_mean_f : 0.f);
-                const float m1 = fmaxf(0.01f, x1 >= 1.17549435e-38f ? x1 * r1 * inv_mean_f : 0.f);
-                part += (2 * k < nvalid ? m0 : 0.f) + (2 * k + 1 < nvalid ? m1 : 0.f);
-            }
-        }
-        double v[1] = {(double)part};
-        grid_reduce<1>(v, a.red, a.result, vloc, nv);
+        mu_x8_vblock(a, vloc, nv);
     }
 }
 
@@ -557,7 +307,7 @@ GeoDev update_geo(const GeoDev &g) { return g; }
 int resident_blocks(const void *fn);
 
 template <int G, int KC>
-static const void *update_fn(int arith, int z3 = 0, int sub = 0, int tof = 0)
+static const void *update_fn(int arith, int sub, int tof)
 {
     if (tof && sub) {                            // TOF on ring-sampled bins: KC = 4
         if (arith == AR_FP32) return (const void *)update_kernel<G, 4, AR_FP32, true, true>;
@@ -574,91 +324,11 @@ static const void *update_fn(int arith, int z3 = 0, int sub = 0, int tof = 0)
         if (arith == AR_KAHAN) return (const void *)update_kernel<G, 4, AR_KAHAN, true>;
         return (const void *)update_kernel<G, 4, AR_FP64, true>;
     }
-    if constexpr (G == 8) {
-        if (z3 && arith == AR_FP32) return (const void *)update_kernel<G, KC, AR_FP32>;
-        if (z3 && arith == AR_KAHAN) return (const void *)update_kernel<G, KC, AR_KAHAN>;
-        if (arith == AR_FP32) return (const void *)update_kernel_x8<KC, AR_FP32>;
-        if (arith == AR_KAHAN) return (const void *)update_kernel_x8<KC, AR_KAHAN>;
-    } else {
+    if constexpr (G == 1) {                      // single-plane FP32: the TV variant only
         if (arith == AR_FP32) return (const void *)update_kernel<G, KC, AR_FP32>;
         if (arith == AR_KAHAN) return (const void *)update_kernel<G, KC, AR_KAHAN>;
     }
     return (const void *)update_kernel<G, KC, AR_FP64>;
-}
-
-// Entries of update_kernel_x8's (pixel, view) table for one subset, computed once per geometry:
-// entry e = (tile t, view u, pixel pl of the tile) is bp_entry(pixel t TP + pl, view u), in the
-// kernel's shared-memory order, so that one tile's entries are one contiguous block.  bp_entry
-// has no arithmetic that differs between the FP32 kernels (the FP32 and FP32 + Kahan tables are
-// the same bits as those the kernel computes).
-template <int KC>
-__global__ void __launch_bounds__(256) bp_table_kernel(const __grid_constant__ GeoDev g, int slot0,
-                                                      int nviews, int TP, long long nent, void *out)
-{
-    using E = typename BpTable<KC, AR_KAHAN, 1024 / (KC > 2 ? 2 : 1)>::E;
-    const long long per = (long long)nviews * TP;
-    const int npix = g.N * g.N;
-    for (long long e = blockIdx.x * 256LL + threadIdx.x; e < nent; e += (long long)gridDim.x * 256) {
-        const long long tile = e / per;
-        const int r = (int)(e - tile * per);
-        const int uu = r / TP, pl = r - uu * TP;
-        const long long j = tile * TP + pl;
-        const bool in = j < npix;
-        reinterpret_cast<E *>(out)[e] = bp_entry<KC, AR_KAHAN, 1024 / (KC > 2 ? 2 : 1)>(
-            g, slot0, uu, in, in ? (int)(j % g.N) : 0, in ? (int)(j / g.N) : 0);
-    }
-}
-
-// The packed update kernel runs for 8-plane groups with uniform bins and without TOF; its table
-// holds 1024 (KC = 2) or 512 (KC = 4) entries of 16 or 32 bytes, two tiles' worth when copied.
-size_t bp_table_bytes_bound(const pet_geometry_desc &d)
-{
-    if (d.nplanes <= 1 || d.subrays > 1 || d.ring_mm > 0 || d.tof_bins > 1) return 0;
-    const long long NG = (d.nplanes + 7) / 8, TP = 256 / NG;
-    const long long npix = (long long)d.n * d.n, ntiles = (npix + TP - 1) / TP;
-    const long long vmax = (d.nviews + d.nsubsets - 1) / d.nsubsets;
-    if (TP < 1 || 2 * vmax * TP > 1024) return 0;
-    return (size_t)(ntiles * d.nviews * TP * 32);
-}
-
-pet_status build_bp_table(pet_geometry *g, cudaStream_t st)
-{
-    const GeoDev &gd = g->dev;
-    g->bptab_off.clear();
-    if (gd.G != 8 || gd.table || gd.T > 1) return PET_OK;
-    const int KC = gd.K <= 2 ? 2 : 4;
-    const int CAP = KC > 2 ? 512 : 1024;
-    const int TP = 256 / gd.NG;
-    if (TP < 1) return PET_OK;
-    const size_t esz = KC > 2 ? sizeof(BpTable<4, AR_KAHAN, 512>::E) : sizeof(BpTable<2, AR_KAHAN, 1024>::E);
-    const long long ntiles = ((long long)gd.N * gd.N + TP - 1) / TP;
-    std::vector<size_t> off(gd.M);
-    size_t total = 0;
-    for (int i = 0; i < gd.M; ++i) {
-        const int nv = g->voff[i + 1] - g->voff[i];
-        if (2 * nv * TP > CAP) return PET_OK;       // the kernel computes this geometry's entries
-        off[i] = total;
-        total += (size_t)ntiles * nv * TP * esz;
-    }
-    if (total == 0) return PET_OK;
-    void *tab = nullptr;
-    PET_CUDA(dev_malloc(&tab, total));
-    for (int i = 0; i < gd.M; ++i) {
-        const int nv = g->voff[i + 1] - g->voff[i];
-        const long long nent = ntiles * nv * TP;
-        const int grid = (int)std::min<long long>((nent + 255) / 256, (long long)sm_count() * 16);
-        char *out = static_cast<char *>(tab) + off[i];
-        if (KC == 2) bp_table_kernel<2><<<grid, 256, 0, st>>>(gd, g->voff[i], nv, TP, nent, out);
-        else bp_table_kernel<4><<<grid, 256, 0, st>>>(gd, g->voff[i], nv, TP, nent, out);
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) {
-            cudaFree(tab);
-            return cuda_fail(e, "bp_table_kernel launch");
-        }
-    }
-    g->d_bptab = tab;                                // set together with the offsets
-    g->bptab_off = off;
-    return PET_OK;
 }
 
 // Pixel tiles per virtual block: each virtual block ends in a block reduction and a grid-wide
@@ -670,9 +340,9 @@ void update_shape(UpdateArgs &a, int arith)
     const int TP = 256 / a.g.NG;
     const int ntiles = (a.g.N * a.g.N + TP - 1) / TP;
     const int sub = a.g.table, tof = a.g.T > 1;
-    const void *fn = a.g.G == 1 ? (a.g.K <= 2 ? update_fn<1, 2>(arith, 0, sub, tof) : update_fn<1, 4>(arith, 0, sub, tof))
-                                : (a.g.K <= 2 ? update_fn<8, 2>(arith, a.z3 || a.tv || a.vox, sub, tof)
-                                              : update_fn<8, 4>(arith, a.z3 || a.tv || a.vox, sub, tof));
+    const void *fn = update_x8_path(a.g, arith) ? update_x8_fn(a, arith)
+                     : a.g.G == 1 ? (a.g.K <= 2 ? update_fn<1, 2>(arith, sub, tof) : update_fn<1, 4>(arith, sub, tof))
+                                  : (a.g.K <= 2 ? update_fn<8, 2>(arith, sub, tof) : update_fn<8, 4>(arith, sub, tof));
     const int slots = sm_count() * resident_blocks(fn);
     a.tpv = std::max({1, (ntiles + a.red.capacity - 1) / a.red.capacity, (ntiles + slots - 1) / slots});
     a.nvb = (ntiles + a.tpv - 1) / a.tpv;
@@ -694,70 +364,65 @@ void image_shape(ImageArgs &a)
 static int persistent_grid(int nvb) { return std::max(1, std::min(nvb, sm_count() * 8)); }
 
 template <int G, int KC>
-static void update_dispatch(const UpdateArgs &a, const Batch &b, int arith, int grid, cudaStream_t st)
+static void update_dispatch(const UpdateArgs &a, const Batch &b, int arith, int grid, cudaStream_t st,
+                            bool pdl)
 {
     if (a.g.T > 1 && a.g.table) {                // TOF on ring-sampled bins: KC = 4
-        if (arith == AR_FP32) update_kernel<G, 4, AR_FP32, true, true><<<grid, 256, 0, st>>>(a, b);
-        else if (arith == AR_KAHAN) update_kernel<G, 4, AR_KAHAN, true, true><<<grid, 256, 0, st>>>(a, b);
-        else update_kernel<G, 4, AR_FP64, true, true><<<grid, 256, 0, st>>>(a, b);
+        if (arith == AR_FP32) launch_pdl(update_kernel<G, 4, AR_FP32, true, true>, grid, st, pdl, a, b);
+        else if (arith == AR_KAHAN) launch_pdl(update_kernel<G, 4, AR_KAHAN, true, true>, grid, st, pdl, a, b);
+        else launch_pdl(update_kernel<G, 4, AR_FP64, true, true>, grid, st, pdl, a, b);
         return;
     }
     if (a.g.T > 1) {                             // TOF geometries: generic kernel
-        if (arith == AR_FP32) update_kernel<G, KC, AR_FP32, false, true><<<grid, 256, 0, st>>>(a, b);
-        else if (arith == AR_KAHAN) update_kernel<G, KC, AR_KAHAN, false, true><<<grid, 256, 0, st>>>(a, b);
-        else update_kernel<G, KC, AR_FP64, false, true><<<grid, 256, 0, st>>>(a, b);
+        if (arith == AR_FP32) launch_pdl(update_kernel<G, KC, AR_FP32, false, true>, grid, st, pdl, a, b);
+        else if (arith == AR_KAHAN) launch_pdl(update_kernel<G, KC, AR_KAHAN, false, true>, grid, st, pdl, a, b);
+        else launch_pdl(update_kernel<G, KC, AR_FP64, false, true>, grid, st, pdl, a, b);
         return;
     }
     if (a.g.table) {                             // sub-ray / ring geometries: KC = 4, generic kernel
-        if (arith == AR_FP32) update_kernel<G, 4, AR_FP32, true><<<grid, 256, 0, st>>>(a, b);
-        else if (arith == AR_KAHAN) update_kernel<G, 4, AR_KAHAN, true><<<grid, 256, 0, st>>>(a, b);
-        else update_kernel<G, 4, AR_FP64, true><<<grid, 256, 0, st>>>(a, b);
+        if (arith == AR_FP32) launch_pdl(update_kernel<G, 4, AR_FP32, true>, grid, st, pdl, a, b);
+        else if (arith == AR_KAHAN) launch_pdl(update_kernel<G, 4, AR_KAHAN, true>, grid, st, pdl, a, b);
+        else launch_pdl(update_kernel<G, 4, AR_FP64, true>, grid, st, pdl, a, b);
         return;
     }
-    if constexpr (G == 8) {
-        // the packed kernel has the in-plane RDP step and p per pixel only; the 3-D prior, the
-        // TV variant and scans with detection factors (p per voxel) run the generic kernel
-        const bool gen = a.z3 || a.tv || a.vox;
-        if (gen && arith == AR_FP32) update_kernel<G, KC, AR_FP32><<<grid, 256, 0, st>>>(a, b);
-        else if (gen && arith == AR_KAHAN) update_kernel<G, KC, AR_KAHAN><<<grid, 256, 0, st>>>(a, b);
-        else if (arith == AR_FP32) update_kernel_x8<KC, AR_FP32><<<grid, 256, 0, st>>>(a, b);
-        else if (arith == AR_KAHAN) update_kernel_x8<KC, AR_KAHAN><<<grid, 256, 0, st>>>(a, b);
-        else update_kernel<G, KC, AR_FP64><<<grid, 256, 0, st>>>(a, b);
-    } else {
-        if (arith == AR_FP32) update_kernel<G, KC, AR_FP32><<<grid, 256, 0, st>>>(a, b);
-        else if (arith == AR_KAHAN) update_kernel<G, KC, AR_KAHAN><<<grid, 256, 0, st>>>(a, b);
-        else update_kernel<G, KC, AR_FP64><<<grid, 256, 0, st>>>(a, b);
+    if constexpr (G == 1) {                      // single-plane FP32: the TV variant only
+        if (arith == AR_FP32) return launch_pdl(update_kernel<G, KC, AR_FP32>, grid, st, pdl, a, b);
+        if (arith == AR_KAHAN) return launch_pdl(update_kernel<G, KC, AR_KAHAN>, grid, st, pdl, a, b);
     }
+    launch_pdl(update_kernel<G, KC, AR_FP64>, grid, st, pdl, a, b);
 }
 
-static pet_status update_any(const UpdateArgs &a, const Batch &b, int arith, int grid, cudaStream_t st)
+static pet_status update_any(const UpdateArgs &a, const Batch &b, int arith, int grid, cudaStream_t st,
+                            bool pdl)
 {
     LaunchScope ls(PET_K_UPDATE, st);
     if (plane1_path(a.g, arith) && !a.tv) {
-        update_p1_dispatch(a, b, arith, grid, st, false);
+        update_p1_dispatch(a, b, arith, grid, st, pdl);
+    } else if (update_x8_path(a.g, arith)) {
+        update_x8_dispatch(a, b, arith, grid, st, pdl);
     } else if (a.g.G == 1) {
-        if (a.g.K <= 2) update_dispatch<1, 2>(a, b, arith, grid, st);
-        else update_dispatch<1, 4>(a, b, arith, grid, st);
+        if (a.g.K <= 2) update_dispatch<1, 2>(a, b, arith, grid, st, pdl);
+        else update_dispatch<1, 4>(a, b, arith, grid, st, pdl);
     } else {
-        if (a.g.K <= 2) update_dispatch<8, 2>(a, b, arith, grid, st);
-        else update_dispatch<8, 4>(a, b, arith, grid, st);
+        if (a.g.K <= 2) update_dispatch<8, 2>(a, b, arith, grid, st, pdl);
+        else update_dispatch<8, 4>(a, b, arith, grid, st, pdl);
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "update_kernel launch");
     return PET_OK;
 }
 
-pet_status launch_update(const UpdateArgs &a0, int arith, cudaStream_t st)
+pet_status launch_update(const UpdateArgs &a0, int arith, cudaStream_t st, bool after_kernel)
 {
     UpdateArgs a = a0;
     update_shape(a, arith);
     update_fp32_scalars(a);
-    return update_any(a, Batch{nullptr, nullptr, 0, 0}, arith, persistent_grid(a.nvb), st);
+    return update_any(a, Batch{nullptr, nullptr, 0, 0}, arith, persistent_grid(a.nvb), st, after_kernel);
 }
 
 pet_status launch_update_batch(const UpdateArgs &shape, const Batch &b, int arith, cudaStream_t st)
 {
-    return update_any(shape, b, arith, b.grid, st);
+    return update_any(shape, b, arith, b.grid, st, false);
 }
 
 template <int G, int KC>

@@ -1,0 +1,406 @@
+// The FP32 update of stacks (8-plane groups): one packed kernel for the in-plane and the 3-D prior,
+// 1/p per pixel or per voxel, and the TV variant, and its precomputed backprojection entries.
+#include "kernels.cuh"
+#include "profile.cuh"
+
+#ifndef UPDATE_X8_BLOCKS
+#define UPDATE_X8_BLOCKS 3      // resident blocks per SM the packed update kernel is built for
+#endif
+
+namespace pet {
+
+int sm_count();
+constexpr int X8_Z3 = 1, X8_VOX = 2, X8_TV = 4;
+
+// FP32 update for 8-plane groups held as four f32x2 pairs.  Same step as update_kernel, with:
+//   - the 3x3 stencil loading every neighbour with missing ones (image border) replaced by the
+//     centre value: their RDP term is exactly zero (d = 0) and the Matlab-style gradient becomes
+//     the one-sided difference, as in the generic stencil;
+//   - the RDP pair term written as d (den + 2 f_k + eps) / den^2 (the numerator
+//     gamma_R |d| + f_j + 3 f_k + 2 eps equals den + 2 f_k + eps), from one reciprocal of den;
+//   - nu = P_{nu1}^{nu2}(mean(mu) / mu) from 1 / mu = min(100, mean(f) / |grad f|);
+//   - the step folded into two per-plane constants before the gather,
+//     f^{k,i} = P_t(A + B b) with A = f - c (beta/M) grad R, B = -c scale, c = lambda alpha nu S,
+//     so that only A, B and the sums of b = A_i^T w stay live across the gather.
+// FL: X8_Z3, the 3-D prior: RDP over the 26 neighbours and nu from the 3-D gradient (each in-plane
+// position's group is used as it is and shifted by one plane up and down); X8_VOX, 1/p per voxel
+// (scans with per-bin detection factors); X8_TV, the TV variant (no RDP term, the unclamped z and
+// the metric W written for the proximal step).
+template <int KC, int AR, int FL>
+__global__ void __launch_bounds__(256, FL & X8_Z3 ? 2 : UPDATE_X8_BLOCKS) update_kernel_x8(
+    const __grid_constant__ UpdateArgs one, const Batch bt)
+{
+    static_assert(AR != AR_FP64, "FP32 arithmetic only");
+    // 16 KB of (pixel, view) entries: the rest of the SM's shared memory stays L1 for the gather
+    using Table = BpTable<KC, AR, 1024 / (KC > 2 ? 2 : 1)>;
+    __shared__ Table tb;
+    // launched behind the projection (see launch_update): nothing is read before it has completed
+    grid_dependency_wait();
+    // the next subiteration's projection (launched after this kernel with programmatic stream
+    // serialization) may be scheduled as this kernel's blocks retire; it waits for completion
+    grid_dependents_launch();
+    const int total = total_vblocks(one, bt);
+    __shared__ UpdateArgs sh_args;
+    for (int vb = blockIdx.x; vb < total; vb += gridDim.x) {
+        int vloc, nv;
+        const UpdateArgs &a = scan_args(one, bt, vb, vloc, nv, sh_args);
+        const GeoDev &g = a.g;
+        const int N = g.N, NG = g.NG, npix = N * N;
+        const unsigned Pp = (unsigned)g.Pp;
+        const int TP = 256 / NG;
+        const int pl = threadIdx.x / NG, grp = threadIdx.x % NG;
+        const int VC = max(1, min(a.nviews, Table::CAP / TP));
+        const bool dyn = a.nu_mode == 1 || a.nu_mode == 2;
+        const double q = (double)npix * g.P;
+        // per-scan scalars in FP32 (an FP64 division per thread is costly at GB300's FP64 rate)
+        const float mean_f = dyn ? (float)*a.sum_f / (float)q : 1.f;
+        const float mean_mu = dyn ? (float)*a.sum_mu / (float)q : 1.f;
+        const float U = a.fs_U, tt = a.fs_t;
+        // eps >= 1e-30 keeps 1/den finite, so that a zero-difference term stays exactly zero
+        const float eps = fmaxf(a.fs_eps, 1e-30f);
+        const float *f = reinterpret_cast<const float *>(a.f) + grp * 8;
+        const float *w = reinterpret_cast<const float *>(a.w) + grp * 8;
+        const float *invp = reinterpret_cast<const float *>(a.invp);
+        const int ntiles = (npix + TP - 1) / TP;
+        // the subset's precomputed entries (one contiguous block per tile) when two tiles' entries
+        // fit the table: double-buffered, the next tile's block copied with cp.async while this
+        // tile is gathered and the next one's stencil runs (one barrier per tile)
+        const bool pre = a.bptab && 2 * a.nviews * TP <= Table::CAP;
+        const int t0 = vloc * a.tpv, t1 = min(ntiles, (vloc + 1) * a.tpv);
+        auto copy_tile = [&](int tile) {
+            const int tbytes = a.nviews * TP * (int)sizeof(typename Table::E);
+            const char *src = static_cast<const char *>(a.bptab) + (size_t)tile * tbytes;
+            char *dst = reinterpret_cast<char *>(tb.e) + ((tile - t0) & 1) * tbytes;
+            for (int o = threadIdx.x * 16; o < tbytes; o += 256 * 16) cp_async16(dst + o, src + o);
+            cp_async_commit();
+        };
+        if (pre && t0 < t1) copy_tile(t0);
+        float part = 0.f;
+        for (int tile = t0; tile < t1; ++tile) {
+            const int j0 = tile * TP, j = j0 + pl;
+            const bool active = pl < TP && j < npix;
+            f2x A[4], B[4];
+            if (active) {
+                const int ix = j % N, iy = j / N;
+                const unsigned jc = (unsigned)j;
+                const unsigned xm = ix > 0 ? jc - 1 : jc, xp = ix < N - 1 ? jc + 1 : jc;
+                const unsigned ym = iy > 0 ? jc - N : jc, yp = iy < N - 1 ? jc + N : jc;
+                constexpr bool Z3 = FL & X8_Z3, VOX = FL & X8_VOX, TV = FL & X8_TV;
+                const f2x GR = vsplat(a.fs_gamma_r), EP = vsplat(eps), TWO = vsplat(2.f);
+                f2x c[4], ce[4], gr[4], g2[4], nb0[4], nb1[4];
+                load8x(f + jc * Pp, c);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) { ce[k] = vadd(c[k], EP); gr[k] = 0ull; }
+                auto rdp = [&](const f2x(&x)[4]) {
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const f2x d = vsub(c[k], x[k]);
+                        const f2x den = vfma(GR, vabs(d), vadd(ce[k], x[k]));
+                        const f2x num = vadd(den, vfma(TWO, x[k], EP));
+                        const f2x r = vrcp(den);
+                        gr[k] = vfma(vmul(d, vmul(num, r)), r, gr[k]);
+                    }
+                };
+                // 3-D: the planes z - 1 (dn) and z + 1 (up) of a position's group x; a missing plane
+                // counts as the centre pixel's own value (its term is then exactly zero)
+                const int nlive = g.P - grp * 8;             // real planes from this group on
+                auto shifted = [&](const f2x(&x)[4], unsigned jn, f2x(&dn)[4], f2x(&up)[4]) {
+                    float v[8], cv[8];
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        vunpk(x[k], v[2 * k], v[2 * k + 1]);
+                        vunpk(c[k], cv[2 * k], cv[2 * k + 1]);
+                    }
+                    const float lo = grp > 0 ? __ldg(f + jn * Pp - 1) : cv[0];
+                    const float hi = nlive > 8 ? __ldg(f + jn * Pp + 8) : cv[7];
+                    float u8[8];
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) u8[q] = q + 1 < nlive ? (q < 7 ? v[q + 1] : hi) : cv[q];
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        dn[k] = vpk(k ? v[2 * k - 1] : lo, v[2 * k]);
+                        up[k] = vpk(u8[2 * k], u8[2 * k + 1]);
+                    }
+                };
+                // the RDP terms of one in-plane position (3-D: with the planes beside it)
+                auto position = [&](const f2x(&x)[4], unsigned jn, bool there) {
+                    if constexpr (TV) return;
+                    rdp(x);
+                    if constexpr (Z3) {
+                        if (!there) return;
+                        f2x dn[4], up[4];
+                        shifted(x, jn, dn, up);
+                        rdp(dn);
+                        rdp(up);
+                    }
+                };
+                // axial neighbours: RDP terms and the Matlab-style gradient
+                load8x(f + xm * Pp, nb0);
+                load8x(f + xp * Pp, nb1);
+                position(nb0, xm, ix > 0);
+                position(nb1, xp, ix < N - 1);
+                if (dyn) {
+                    const f2x HX = vsplat((ix > 0 && ix < N - 1) ? 0.5f : 1.f);
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const f2x t = vmul(HX, vsub(nb1[k], nb0[k]));
+                        g2[k] = vmul(t, t);
+                    }
+                }
+                load8x(f + ym * Pp, nb0);
+                load8x(f + yp * Pp, nb1);
+                position(nb0, ym, iy > 0);
+                position(nb1, yp, iy < N - 1);
+                if constexpr (Z3) {
+                    // the centre column: two neighbours, and the gradient across the planes
+                    f2x dn[4], up[4];
+                    shifted(c, jc, dn, up);
+                    rdp(dn);
+                    rdp(up);
+                    if (dyn) {
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            const int z0 = grp * 8 + 2 * k;
+                            const f2x HZ = vpk(z0 > 0 && z0 + 1 < g.P ? 0.5f : 1.f, z0 + 2 < g.P ? 0.5f : 1.f);
+                            const f2x t = vmul(HZ, vsub(up[k], dn[k]));
+                            g2[k] = vfma(t, t, g2[k]);
+                        }
+                    }
+                }
+                f2x nu[4];
+                if (dyn) {
+                    const f2x HY = vsplat((iy > 0 && iy < N - 1) ? 0.5f : 1.f);
+                    const float nu1 = a.fs_nu1, nu2 = a.fs_nu2;
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const f2x t = vmul(HY, vsub(nb1[k], nb0[k]));
+                        float r0, r1;
+                        vunpk(vrsqrt(vfma(t, t, g2[k])), r0, r1);
+                        // 1 / mu = 1 / max(0.01, |grad f| / mean f) = min(100, mean f / |grad f|)
+                        r0 = fminf(100.f, r0 * mean_f);
+                        r1 = fminf(100.f, r1 * mean_f);
+                        nu[k] = vpk(fminf(fmaxf(mean_mu * r0, nu1), nu2),
+                                    fminf(fmaxf(mean_mu * r1, nu1), nu2));
+                    }
+                    if (a.nu_mode == 2)
+                        store8x(reinterpret_cast<float *>(a.nu_frozen) + jc * Pp + grp * 8, nu);
+                } else if (a.nu_mode == 3) {
+                    load8x(reinterpret_cast<const float *>(a.nu_frozen) + jc * Pp + grp * 8, nu);
+                } else {
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) nu[k] = vsplat(1.f);
+                }
+                // diagonal neighbours
+                if constexpr (!TV) {
+                    const unsigned dm = iy > 0 ? jc - N : jc, dp = iy < N - 1 ? jc + N : jc;
+                    const bool xl = ix > 0, xr = ix < N - 1, yl = iy > 0, yr = iy < N - 1;
+                    const unsigned j0_ = xl && yl ? dm - 1 : jc, j1_ = xr && yl ? dm + 1 : jc;
+                    const unsigned j2_ = xl && yr ? dp - 1 : jc, j3_ = xr && yr ? dp + 1 : jc;
+                    load8x(f + j0_ * Pp, nb0);
+                    load8x(f + j1_ * Pp, nb1);
+                    position(nb0, j0_, xl && yl);
+                    position(nb1, j1_, xr && yl);
+                    load8x(f + j2_ * Pp, nb0);
+                    load8x(f + j3_ * Pp, nb1);
+                    position(nb0, j2_, xl && yr);
+                    position(nb1, j3_, xr && yr);
+                }
+                // c = lambda alpha nu S, S = min(f, U - f) / p;  A = f - c (beta/M) 2 gr;  B = -c scale
+                f2x NK[4];
+                if constexpr (VOX) {
+                    load8x(invp + jc * Pp + grp * 8, NK);
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) NK[k] = vmul(NK[k], vsplat(-a.fs_lam * a.fs_ips));
+                } else {
+                    NK[0] = vsplat(-a.fs_lam * invp[j] * a.fs_ips);
+                    NK[1] = NK[2] = NK[3] = NK[0];
+                }
+                const f2x BM = vsplat(2.f * a.fs_bm), SC = vsplat(a.fs_scale);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    float c0, c1;
+                    vunpk(c[k], c0, c1);
+                    const f2x S = vpk(fminf(c0, U - c0), fminf(c1, U - c1));
+                    const f2x cn = vmul(vmul(nu[k], S), NK[k]);
+                    if constexpr (TV) {
+                        A[k] = c[k];
+                        float w0, w1;
+                        vunpk(cn, w0, w1);
+                        nb0[k] = vpk(2 * k < nlive ? -w0 : 1.f, 2 * k + 1 < nlive ? -w1 : 1.f);
+                    } else {
+                        A[k] = vfma(cn, vmul(BM, gr[k]), c[k]);
+                    }
+                    B[k] = vmul(cn, SC);
+                }
+                if constexpr (TV) store8x(reinterpret_cast<float *>(a.wbuf) + jc * Pp + grp * 8, nb0);
+            }
+            // gather backprojection b = A_i^T w with the tile's shared (pixel, view) weights
+            f2x sm[4], er[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) { sm[k] = 0ull; er[k] = 0ull; }
+            for (int u0 = 0; u0 < a.nviews; u0 += VC) {
+                const int nvc = min(VC, a.nviews - u0);
+                if (pre) {
+                    cp_async_wait_all();             // this tile's block (this thread's part)
+                    __syncthreads();                 // all parts; the previous gather is done
+                    if (tile + 1 < t1) copy_tile(tile + 1);
+                } else {
+                    __syncthreads();
+                    bp_fill<KC, AR>(g, a.slot0, u0, nvc, j0, TP, tb);
+                    __syncthreads();
+                }
+                if (!active) continue;
+                const typename Table::E *te = tb.e + (pre ? ((tile - t0) & 1) * a.nviews * TP : 0);
+                for (int uu = 0; uu < nvc; ++uu) {
+                    const typename Table::E ent = te[uu * TP + pl];
+                    const float *row = w + ent.off;
+#pragma unroll
+                    for (int kb = 0; kb < KC; kb += 2) {
+                        f2x x0[4], x1[4];
+                        load8x(row + kb * Pp, x0);
+                        load8x(row + (kb + 1) * Pp, x1);
+                        const f2x W0 = vsplat(ent.w[kb]), W1 = vsplat(ent.w[kb + 1]);
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            if constexpr (AR == AR_KAHAN) {
+                                const f2x y = vfma(W1, x1[k], vfma(W0, x0[k], er[k]));
+                                const f2x t = vadd(sm[k], y);
+                                er[k] = vsub(y, vsub(t, sm[k]));
+                                sm[k] = t;
+                            } else {
+                                sm[k] = vfma(W1, x1[k], vfma(W0, x0[k], sm[k]));
+                            }
+                        }
+                    }
+                }
+            }
+            if (!active) continue;
+            // step and clamp P_t
+            f2x out[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const f2x b = AR == AR_KAHAN ? vadd(sm[k], er[k]) : sm[k];
+                float f0, f1;
+                vunpk(vfma(B[k], b, A[k]), f0, f1);
+                if constexpr (!(FL & X8_TV)) {
+                    f0 = f0 <= 0.f ? tt : (f0 >= U ? U - tt : f0);
+                    f1 = f1 <= 0.f ? tt : (f1 >= U ? U - tt : f1);
+                }
+                const int p0 = grp * 8 + 2 * k;
+                f0 = p0 < g.P ? f0 : 0.f;
+                f1 = p0 + 1 < g.P ? f1 : 0.f;
+                part += f0 + f1;
+                out[k] = vpk(f0, f1);
+            }
+            store8x(reinterpret_cast<float *>(a.fout) + (unsigned)j * Pp + grp * 8, out);
+            if constexpr (FL & X8_TV)
+                store8x(reinterpret_cast<float *>(a.zbuf) + (unsigned)j * Pp + grp * 8, out);
+        }
+        double v[1] = {(double)part};
+        grid_reduce<1>(v, a.red, a.sum_fout, vloc, nv);
+    }
+}
+
+// Entries of update_kernel_x8's (pixel, view) table for one subset, computed once per geometry:
+// entry e = (tile t, view u, pixel pl of the tile) is bp_entry(pixel t TP + pl, view u), in the
+// kernel's shared-memory order, so that one tile's entries are one contiguous block.  bp_entry
+// has no arithmetic that differs between the FP32 kernels (the FP32 and FP32 + Kahan tables are
+// the same bits as those the kernel computes).
+template <int KC>
+__global__ void __launch_bounds__(256) bp_table_kernel(const __grid_constant__ GeoDev g, int slot0,
+                                                      int nviews, int TP, long long nent, void *out)
+{
+    using E = typename BpTable<KC, AR_KAHAN, 1024 / (KC > 2 ? 2 : 1)>::E;
+    const long long per = (long long)nviews * TP;
+    const int npix = g.N * g.N;
+    for (long long e = blockIdx.x * 256LL + threadIdx.x; e < nent; e += (long long)gridDim.x * 256) {
+        const long long tile = e / per;
+        const int r = (int)(e - tile * per);
+        const int uu = r / TP, pl = r - uu * TP;
+        const long long j = tile * TP + pl;
+        const bool in = j < npix;
+        reinterpret_cast<E *>(out)[e] = bp_entry<KC, AR_KAHAN, 1024 / (KC > 2 ? 2 : 1)>(
+            g, slot0, uu, in, in ? (int)(j % g.N) : 0, in ? (int)(j / g.N) : 0);
+    }
+}
+
+// The packed update kernel runs for 8-plane groups with uniform bins and without TOF; its table
+// holds 1024 (KC = 2) or 512 (KC = 4) entries of 16 or 32 bytes, two tiles' worth when copied.
+size_t bp_table_bytes_bound(const pet_geometry_desc &d)
+{
+    if (d.nplanes <= 1 || d.subrays > 1 || d.ring_mm > 0 || d.tof_bins > 1) return 0;
+    const long long NG = (d.nplanes + 7) / 8, TP = 256 / NG;
+    const long long npix = (long long)d.n * d.n, ntiles = (npix + TP - 1) / TP;
+    const long long vmax = (d.nviews + d.nsubsets - 1) / d.nsubsets;
+    if (TP < 1 || 2 * vmax * TP > 1024) return 0;
+    return (size_t)(ntiles * d.nviews * TP * 32);
+}
+
+pet_status build_bp_table(pet_geometry *g, cudaStream_t st)
+{
+    const GeoDev &gd = g->dev;
+    g->bptab_off.clear();
+    if (gd.G != 8 || gd.table || gd.T > 1) return PET_OK;
+    const int KC = gd.K <= 2 ? 2 : 4;
+    const int CAP = KC > 2 ? 512 : 1024;
+    const int TP = 256 / gd.NG;
+    if (TP < 1) return PET_OK;
+    const size_t esz = KC > 2 ? sizeof(BpTable<4, AR_KAHAN, 512>::E) : sizeof(BpTable<2, AR_KAHAN, 1024>::E);
+    const long long ntiles = ((long long)gd.N * gd.N + TP - 1) / TP;
+    std::vector<size_t> off(gd.M);
+    size_t total = 0;
+    for (int i = 0; i < gd.M; ++i) {
+        const int nv = g->voff[i + 1] - g->voff[i];
+        if (2 * nv * TP > CAP) return PET_OK;       // the kernel computes this geometry's entries
+        off[i] = total;
+        total += (size_t)ntiles * nv * TP * esz;
+    }
+    if (total == 0) return PET_OK;
+    void *tab = nullptr;
+    PET_CUDA(dev_malloc(&tab, total));
+    for (int i = 0; i < gd.M; ++i) {
+        const int nv = g->voff[i + 1] - g->voff[i];
+        const long long nent = ntiles * nv * TP;
+        const int grid = (int)std::min<long long>((nent + 255) / 256, (long long)sm_count() * 16);
+        char *out = static_cast<char *>(tab) + off[i];
+        if (KC == 2) bp_table_kernel<2><<<grid, 256, 0, st>>>(gd, g->voff[i], nv, TP, nent, out);
+        else bp_table_kernel<4><<<grid, 256, 0, st>>>(gd, g->voff[i], nv, TP, nent, out);
+        cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) {
+            cudaFree(tab);
+            return cuda_fail(e, "bp_table_kernel launch");
+        }
+    }
+    g->d_bptab = tab;                                // set together with the offsets
+    g->bptab_off = off;
+    return PET_OK;
+}
+
+// Stacks in FP32 with uniform bins and no TOF run the packed kernel.
+bool update_x8_path(const GeoDev &g, int arith)
+{
+    return g.G == 8 && arith != AR_FP64 && !g.table && g.T == 1;
+}
+
+template <int KC, int AR>
+static auto x8_fn(const UpdateArgs &a) -> void (*)(const UpdateArgs, const Batch)
+{
+    if (a.tv) return a.vox ? update_kernel_x8<KC, AR, X8_TV | X8_VOX> : update_kernel_x8<KC, AR, X8_TV>;
+    if (a.z3) return a.vox ? update_kernel_x8<KC, AR, X8_Z3 | X8_VOX> : update_kernel_x8<KC, AR, X8_Z3>;
+    return a.vox ? update_kernel_x8<KC, AR, X8_VOX> : update_kernel_x8<KC, AR, 0>;
+}
+
+static auto x8_any(const UpdateArgs &a, int arith)
+{
+    if (a.g.K <= 2) return arith == AR_KAHAN ? x8_fn<2, AR_KAHAN>(a) : x8_fn<2, AR_FP32>(a);
+    return arith == AR_KAHAN ? x8_fn<4, AR_KAHAN>(a) : x8_fn<4, AR_FP32>(a);
+}
+
+const void *update_x8_fn(const UpdateArgs &a, int arith) { return (const void *)x8_any(a, arith); }
+
+void update_x8_dispatch(const UpdateArgs &a, const Batch &b, int arith, int grid, cudaStream_t st, bool pdl)
+{
+    launch_pdl(x8_any(a, arith), grid, st, pdl, a, b);
+}
+
+}  // namespace pet

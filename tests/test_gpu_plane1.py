@@ -35,7 +35,7 @@ GEOMS = [
 def test_single_plane_against_oracle(geom):
     N, V, NB, M, rho, R = geom
     w = synth.Workload("p1", N, 1, 4.0, V, NB, 4.0 * rho, M, 3e6, "ellipses2d",
-                       synth.AlgoParams(iterations=2, beta=0.05, **synth.P2_WORKLOAD), seed=N + V, subrays=R)
+                       synth.AlgoParams(iterations=3, beta=0.05, **synth.P2_WORKLOAD), seed=N + V, subrays=R)
     scan = synth.make_scan(w)
     g, og = pet.Geometry.from_dict(w.geometry(), scan["sens"]), oracle.geom_from(w.geometry(), scan["sens"])
     x = np.asarray(synth.random_image((1, N, N), seed=V), np.float32)
