@@ -1,0 +1,153 @@
+// FP32 stand-alone backprojection of stacks with uniform bins (no TOF), two by two pixels per thread.
+//
+// A thread that gathers one pixel reads KC = 2 rows per view and group, 14.5 GB of L1 reads for all
+// 288 views of a 256 x 256 x 89 stack, and 634 us were spent on them.  The lines of one view that
+// meet a 2 x 2 block of pixels are at most KQ = 3 neighbouring bins (4 for bins below 0.94
+// pixels), so a thread that holds the four pixels' sums reads 3 rows where four threads read 8.
+// Its (block, view) entries hold the rows' offset and the KQ x 4 lengths, as pairs (w, w) for the
+// f32x2 FMAs, in shared memory; tiles are about square, so that a view's rows are shared in both
+// directions.  Sums: a view is added by FMAs onto the compensation term, and every fourth view one
+// compensated step moves it into the sum (no registers beyond those of a plain compensated sum).
+#include "kernels.cuh"
+#include "profile.cuh"
+
+namespace pet {
+
+int sm_count();
+
+template <int KQ> struct __align__(16) QuadEntry {
+    f2x w[KQ * 4];             // [bin][pixel], pixel = 2 dy + dx
+    unsigned off, pad[3];
+};
+constexpr int QUAD_BYTES = 32 * 1024;
+
+// One entry: pixels (x, y), (x + 1, y), (x, y + 1), (x + 1, y + 1) against view u of the subset.
+template <int KQ>
+__device__ __forceinline__ void quad_entry(const GeoDev &g, int slot0, int u, int x, int y, QuadEntry<KQ> &e)
+{
+    int b0[4], first = 0x7fffffff;
+    float wk[4][2];
+#pragma unroll
+    for (int p = 0; p < 4; ++p) {
+        const int px = x + (p & 1), py = y + (p >> 1);
+        b0[p] = 0;
+        wk[p][0] = wk[p][1] = 0.f;
+        if (px < g.N && py < g.N) {
+            bp_weights<2, AR_KAHAN>(g, g.views[slot0 + u], slot0 + u, px, py, b0[p], wk[p]);
+            first = min(first, b0[p]);
+        }
+    }
+    const int bc = min(max(first, 0), g.NB - KQ);      // all KQ rows of the entry exist
+    e.off = ((unsigned)u * (unsigned)g.NB + (unsigned)bc) * (unsigned)g.Pp;
+#pragma unroll
+    for (int k = 0; k < KQ; ++k)
+#pragma unroll
+        for (int p = 0; p < 4; ++p) {
+            const int s = bc + k - b0[p];
+            e.w[k * 4 + p] = vsplat(s == 0 ? wk[p][0] : (s == 1 ? wk[p][1] : 0.f));
+        }
+}
+
+template <int KQ, int AR>
+__global__ void __launch_bounds__(256, 2) back_quad_kernel(const __grid_constant__ BackArgs a)
+{
+    using E = QuadEntry<KQ>;
+    constexpr int CAP = QUAD_BYTES / (int)sizeof(E);
+    __shared__ E tb[CAP];
+    const GeoDev &g = a.g;
+    const int N = g.N, NG = g.NG, TP = min(256 / NG, CAP);
+    int ty = 1;
+    while ((ty + 1) * (ty + 1) <= TP) ++ty;
+    const int tx = TP / ty, nq = tx * ty;                             // blocks of a tile
+    const int ntx = (N + 2 * tx - 1) / (2 * tx), ntiles = ntx * ((N + 2 * ty - 1) / (2 * ty));
+    const int q = threadIdx.x / NG, grp = threadIdx.x - q * NG, qy = q / tx, qx = q - qy * tx;
+    const int VC = min(a.nviews, CAP / nq);
+    const unsigned Pp = (unsigned)g.Pp;
+    const float *proj = reinterpret_cast<const float *>(a.proj) + grp * 8;
+    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+        const int x0 = (tile % ntx) * 2 * tx, y0 = (tile / ntx) * 2 * ty;
+        const int x = x0 + 2 * qx, y = y0 + 2 * qy;
+        const bool active = q < nq && x < N && y < N;
+        f2x sm[4][4], er[4][4];
+#pragma unroll
+        for (int p = 0; p < 4; ++p)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) sm[p][k] = er[p][k] = 0ull;
+        auto merge = [&]() {
+#pragma unroll
+            for (int p = 0; p < 4; ++p)
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    if constexpr (AR == AR_KAHAN) {
+                        const f2x t = vadd(sm[p][k], er[p][k]);
+                        er[p][k] = vsub(er[p][k], vsub(t, sm[p][k]));
+                        sm[p][k] = t;
+                    }
+                }
+        };
+        for (int u0 = 0; u0 < a.nviews; u0 += VC) {
+            const int nvc = min(VC, a.nviews - u0);
+            __syncthreads();
+            for (int i = threadIdx.x; i < nq * nvc; i += 256) {
+                const int uu = i / nq, b = i - uu * nq, by = b / tx;
+                quad_entry<KQ>(g, a.slot0, u0 + uu, x0 + 2 * (b - by * tx), y0 + 2 * by, tb[i]);
+            }
+            __syncthreads();
+            if (!active) continue;
+            for (int uu = 0; uu < nvc; ++uu) {
+                const E &e = tb[uu * nq + q];
+                const float *row = proj + e.off;
+#pragma unroll
+                for (int b = 0; b < KQ; ++b) {
+                    f2x v[4];
+                    load8x(row + b * Pp, v);
+                    const ulonglong2 w01 = reinterpret_cast<const ulonglong2 *>(e.w)[2 * b];
+                    const ulonglong2 w23 = reinterpret_cast<const ulonglong2 *>(e.w)[2 * b + 1];
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        er[0][k] = vfma(w01.x, v[k], er[0][k]);
+                        er[1][k] = vfma(w01.y, v[k], er[1][k]);
+                        er[2][k] = vfma(w23.x, v[k], er[2][k]);
+                        er[3][k] = vfma(w23.y, v[k], er[3][k]);
+                    }
+                }
+                if ((uu & 3) == 3) merge();
+            }
+            merge();
+        }
+        if (!active) continue;
+        const float scale = (float)g.scale;
+#pragma unroll
+        for (int p = 0; p < 4; ++p) {
+            const int px = x + (p & 1), py = y + (p >> 1);
+            if (px >= N || py >= N) continue;
+            float o[8];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) vunpk(vadd(sm[p][k], er[p][k]), o[2 * k], o[2 * k + 1]);
+#pragma unroll
+            for (int c = 0; c < 8; ++c) o[c] = grp * 8 + c < g.P ? scale * o[c] : 0.f;
+            store_group<8, float>(reinterpret_cast<float *>(a.img) + ((unsigned)(py * N + px) * Pp + grp * 8), o);
+        }
+    }
+}
+
+// Stacks in FP32 whose 2 x 2 pixel blocks meet at most four bins of a view.
+bool back_quad_path(const BackArgs &a, int arith)
+{
+    return a.proj && a.g.G == 8 && arith != AR_FP64 && !a.g.table && a.g.T == 1 && a.g.K <= 2 && a.g.KQ <= 4 &&
+           a.g.NG <= 256;
+}
+
+void back_quad_dispatch(const BackArgs &a, int arith, cudaStream_t st)
+{
+    const int grid = sm_count() * 2;
+    if (a.g.KQ <= 3) {
+        if (arith == AR_KAHAN) back_quad_kernel<3, AR_KAHAN><<<grid, 256, 0, st>>>(a);
+        else back_quad_kernel<3, AR_FP32><<<grid, 256, 0, st>>>(a);
+    } else {
+        if (arith == AR_KAHAN) back_quad_kernel<4, AR_KAHAN><<<grid, 256, 0, st>>>(a);
+        else back_quad_kernel<4, AR_FP32><<<grid, 256, 0, st>>>(a);
+    }
+}
+
+}  // namespace pet

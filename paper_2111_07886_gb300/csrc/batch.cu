@@ -39,7 +39,8 @@ struct BatchClass {
     int z3 = 0;                               // 3-D prior (the generic update and mu kernels)
     int sub = 0;                              // sub-ray geometry (the sub-ray update kernel)
     int vox = 0;                              // detection factors: p per voxel (generic update)
-    int tof = 0;                              // TOF geometries (the TOF projector and gather)
+    int tof = 0;                              // TOF geometries (the TOF projector and gather):
+                                              // 1, or 2 for those of tof_fwd_stack
     int cap = 0;                              // scan slots of this class
     std::vector<pet_state *> slot;            // nullptr = empty
     std::vector<bool> objective;              // per slot: plan objectives
@@ -153,7 +154,7 @@ extern "C" void pet_batch_destroy(pet_batch *b)
 static pet_status class_for(pet_batch *b, pet_state *s, BatchClass **out)
 {
     const int G = s->g->dev.G, arith = s->arith, KC = kc_of(s), z3 = s->prm.rdp_3d;
-    const int sub = s->g->dev.table, vox = s->attn ? 1 : 0, tof = s->g->dev.T > 1 ? 1 : 0;
+    const int sub = s->g->dev.table, vox = s->attn ? 1 : 0, tof = s->g->dev.T > 1 ? 1 + s->g->dev.tofk : 0;
     for (BatchClass *c : b->classes)
         if (c->G == G && c->arith == arith && c->KC == KC && c->z3 == z3 && c->sub == sub &&
             c->vox == vox && c->tof == tof) {
@@ -279,6 +280,7 @@ static pet_status class_launches(pet_batch *b, BatchClass *c, const BatchClass::
     fs.g.K = c->KC;
     fs.g.R = c->sub ? 2 : 1;                  // selects the sub-ray (table-driven) projector
     fs.g.table = c->sub;
+    fs.g.tofk = c->tof == 2;
     fs.g.T = c->tof ? 2 : 1;                  // selects the TOF projector (the count comes per scan)
     UpdateArgs us{};
     us.g.G = c->G;

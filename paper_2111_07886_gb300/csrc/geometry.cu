@@ -134,7 +134,7 @@ static pet_status build_tables(pet_geometry *g, std::vector<ViewGeo> &views,
     g->voff[M] = V;
     views.resize(V);
     rays.resize((size_t)V * NB);
-    int K = 1;
+    int K = 1, KQ = 1;
     for (int u = 0; u < V; ++u) {
         const int v = g->view_of_slot[u];
         const double th = (double)v * 3.14159265358979323846 / (double)V;
@@ -205,6 +205,7 @@ static pet_status build_tables(pet_geometry *g, std::vector<ViewGeo> &views,
         if (ring) K = std::max(K, (int)floor(2.0 * (0.5 * (ac + as)) / wmin) + 3);
         else if (R == 1) K = std::max(K, (int)floor(2.0 * vg.h) + 1);
         else K = std::max(K, (int)floor(2.0 * (vg.h + 0.5 - 0.5 / R)) + 2);
+        KQ = std::max(KQ, (int)floor(4.0 * vg.h) + 1);
         views[u] = vg;
         // driving steps the line at offset r meets the image (+- one step of margin)
         auto range = [&](double r, long long &dlo, long long &dhi, double &LO0) {
@@ -254,6 +255,7 @@ static pet_status build_tables(pet_geometry *g, std::vector<ViewGeo> &views,
     }
     // sub-ray and ring kernels are built for 4 candidates
     g->dev.K = (R > 1 || ring) ? std::max(K, 3) : K;
+    g->dev.KQ = KQ;
     g->dev.R = R;
     g->dev.ring = ring ? 1 : 0;
     g->dev.table = (R > 1 || ring) ? 1 : 0;
@@ -297,6 +299,8 @@ static pet_status geometry_init(pet_geometry *g, cudaStream_t st)
     } else {
         gd.tof_d = gd.tof_k = gd.tof_w = 0.0;
     }
+    gd.tof_hw = gd.T > 1 ? std::min(gd.T, (int)floor(std::min(64.0, 2.0 * gd.tof_w / gd.tof_d)) + 2) : 0;
+    gd.tofk = gd.T > 1 && gd.G == 8 && tof_stack_shape(gd.NG, gd.T) ? 1 : 0;
     gd.tof_df = (float)gd.tof_d; gd.tof_kf = (float)gd.tof_k; gd.tof_wf = (float)gd.tof_w;
     PET_CUDA(dev_malloc(&g->d_views, sizeof(ViewGeo) * views.size()));
     PET_CUDA(dev_malloc(&g->d_rays, sizeof(RayGeo) * rays.size()));

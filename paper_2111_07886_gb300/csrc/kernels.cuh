@@ -335,6 +335,14 @@ template <int G, int AR> struct GroupSum {
         }
     }
 
+    // s_p += w x_p (FP64)
+    __device__ __forceinline__ void add1term(T w, const T (&x)[G])
+    {
+        static_assert(AR == AR_FP64, "FP64 sums only");
+#pragma unroll
+        for (int p = 0; p < G; ++p) s2[p] = fma(w, x[p], s2[p]);
+    }
+
     // scalar-weight-only form (sensitivity: x == 1)
     __device__ __forceinline__ void add_scalar(T y0)
     {
@@ -1014,17 +1022,24 @@ __device__ __forceinline__ const A &scan_args(const A &one, const Batch &b, int 
     return sh;
 }
 
-// scan_args for a block that takes consecutive virtual blocks: `cur` is the scan whose arguments
-// `sh` holds (-1: none); the copy, and its two barriers, are made only when the scan changes.
-// Returns true when it changed.
+// scan_args for a block that takes consecutive virtual blocks: the scan whose arguments `sh` holds and
+// its virtual blocks [begin, end) are kept, so that the search of the prefix table and the copy with
+// its two barriers are made only when the scan changes.
+struct KeptScan {
+    int begin = 0, end = -1;
+};
+// Returns true when the scan changed.  Every thread of the block must call it with the same vb.
 template <class A>
 __device__ __forceinline__ bool scan_args_kept(const A &one, const Batch &b, int vb, int &local, int &count,
-                                               A &sh, int &cur, const A *&out)
+                                               A &sh, KeptScan &kept, const A *&out)
 {
+    if (vb >= kept.begin && vb < kept.end) {
+        local = vb - kept.begin;
+        return false;
+    }
     const A *src = scan_of(one, b, vb, local, count);
-    const int scan = b.nscans == 0 ? 0 : (int)(src - reinterpret_cast<const A *>(b.args));
-    if (scan == cur) return false;
-    cur = scan;
+    kept.begin = vb - local;
+    kept.end = kept.begin + count;
     out = &one;
     if (b.nscans == 0) return true;
     __syncthreads();                                  // the previous virtual block is done with sh
@@ -1039,12 +1054,13 @@ __device__ __forceinline__ bool scan_args_kept(const A &one, const Batch &b, int
 }
 
 // The virtual blocks of one block of a persistent grid: runs of consecutive ones (a run mostly stays
-// within one scan, whose arguments and reduction ticket are then handled once), about eight runs
-// per block so that blocks with cheap and with costly scans even out.
+// within one scan, whose arguments and reduction ticket are then handled once), about three runs
+// per block so that blocks with cheap and with costly scans even out (one contiguous range per
+// block left a third of the cycles idle, eight runs paid a ticket per virtual block).
 struct VblockRuns {
     int total, len, base, at;
     __device__ __forceinline__ explicit VblockRuns(int n)
-        : total(n), len(max(1, n / ((int)gridDim.x * 8))), base((int)blockIdx.x * len), at(0) {}
+        : total(n), len(max(1, n / ((int)gridDim.x * 3))), base((int)blockIdx.x * len), at(0) {}
     // the next virtual block, -1 when there is none
     __device__ __forceinline__ int next()
     {

@@ -115,6 +115,7 @@ struct RayGeo {
 struct GeoDev {
     int N, P, Pp, G, NG;      // image side, planes, padded planes, group size, groups
     int V, NB, M, K;          // views, bins, subsets, max candidate bins per view in the gather
+    int KQ;                   // max lines of one view that meet a 2 x 2 block of pixels
     int tuneS;                // forward projector chunks per ray picked by pet_autotune (0: heuristic)
     int R;                    // sub-rays per bin (1: one line); scale includes the 1 / R
     int ring;                 // 1: bins sampled like a detector ring's lines (table-driven)
@@ -127,6 +128,8 @@ struct GeoDev {
     double rho;               // bin spacing / pixel size
     double tof_d, tof_k, tof_w;   // TOF bin width, 1 / (sigma sqrt 2), window half-width
     float tof_df, tof_kf, tof_wf; //   (pixel units; h_t < 1e-12 beyond the window)
+    int tof_hw;               // at most this many TOF bins lie within the window of a position
+    int tofk;                 // 1: the FP32 projections run tof_fwd_stack (see geometry_init)
     long long offq;           // half a sub-ray spacing in bin units, Q32.32 (2^32 / (2 R))
     double scale;             // sens * pixel_mm
     const ViewGeo *views;     // [V] in subset order
@@ -207,6 +210,7 @@ enum Arith { AR_FP32 = 0, AR_KAHAN = 1, AR_FP64 = 2 };
 pet_status launch_forward(const FwdArgs &a, int mode, int arith, cudaStream_t st,
                           bool after_kernel = false);
 void forward_shape(FwdArgs &a, int mode, int arith);      // fills S, R, tpv, nvb
+bool tof_stack_shape(int NG, int T);   // the shapes tof_fwd_stack is for
 // time-of-flight geometries (g.T > 1; launch_forward / forward_shape forward to these)
 pet_status launch_forward_tof(const FwdArgs &a, int mode, int arith, cudaStream_t st);
 pet_status launch_forward_tof_batch(const FwdArgs &shape, const Batch &b, int mode, int arith,
@@ -224,6 +228,8 @@ struct BackArgs {
 };
 
 pet_status launch_back(const BackArgs &a, int arith, cudaStream_t st);
+bool back_quad_path(const BackArgs &a, int arith);      // back8.cu
+void back_quad_dispatch(const BackArgs &a, int arith, cudaStream_t st);
 
 struct UpdateArgs {
     GeoDev g;
@@ -262,8 +268,9 @@ void update_shape(UpdateArgs &a, int arith);               // fills tpv, nvb
 GeoDev update_geo(const GeoDev &g);                        // plane grouping of the update kernel
 pet_status launch_update_batch(const UpdateArgs &shape, const Batch &b, int arith,
                                cudaStream_t st);
-// stacks in FP32 with uniform bins and without TOF (update8.cu; launch_update forwards to these)
-bool update_x8_path(const GeoDev &g, int arith);
+// stacks in FP32 with uniform bins (update8.cu; launch_update forwards to these)
+bool update_x8_path(const UpdateArgs &a, int arith);
+int update_x8_tiles(const UpdateArgs &a);
 const void *update_x8_fn(const UpdateArgs &a, int arith);
 void update_x8_dispatch(const UpdateArgs &a, const Batch &b, int arith, int grid, cudaStream_t st,
                         bool pdl);

@@ -190,9 +190,10 @@ __global__ void __launch_bounds__(256, 4) fwd_kernel_p1(const __grid_constant__ 
     __shared__ double red_sh[2][32];
     VblockRuns runs(total_vblocks(one, bt));
     const FwdArgs *a = nullptr;
-    int scan = -1, done = 0, vloc = 0, nv = 0;
+    int done = 0, vloc = 0, nv = 0;
+    KeptScan kept;
     for (int vb; (vb = runs.next()) >= 0;) {
-        if (scan_args_kept(one, bt, vb, vloc, nv, sh_args, scan, a)) done = 0;
+        if (scan_args_kept(one, bt, vb, vloc, nv, sh_args, kept, a)) done = 0;
         fwd_p1_vblock<AR, MODE, SUB>(*a, vloc, comb_s, comb_e, red_sh);
         ++done;
         if constexpr (MODE == FWD_OBJECTIVE)
@@ -244,6 +245,132 @@ __device__ __forceinline__ void p1_neighbour(const float *f, int N, int ix, int 
     else if (q < 4) gy += (float)dy * fk;
 }
 
+// The patches of one virtual block that fall to warp `wid`; returns this lane's sum of new pixels.
+template <int KC, int AR, bool SUB, int C>
+__device__ __forceinline__ float p1_patches(const UpdateArgs &a, P1View *vt, int vloc, int wid, int lane,
+                                            float inv_mean_f, float mean_mu)
+{
+    const GeoDev &g = a.g;
+    const int N = g.N, NB = g.NB, npix = N * N, stride = NB + 2 * P1_PAD;
+    const bool dyn = a.nu_mode == 1 || a.nu_mode == 2;
+    constexpr int PX = 32 / C, TX = C == 1 ? 8 : (C == 8 ? 2 : 4), TY = PX / TX;
+    const int c = lane / PX, pl = lane - c * PX, py = pl / TX, px = pl - py * TX;
+    const int ntx = (N + TX - 1) / TX, npatch = ntx * ((N + TY - 1) / TY);
+    const float *w = reinterpret_cast<const float *>(a.w);
+    const float *f = reinterpret_cast<const float *>(a.f);
+    const float U = a.fs_U, tt = a.fs_t, scale = a.fs_scale;
+    float part = 0.f;
+    for (int k = 0; k < a.tpv; ++k) {
+        const int patch = (vloc * a.tpv + k) * 8 + wid;
+        if (patch >= npatch) break;
+        const int x0 = (patch % ntx) * TX, y0 = (patch / ntx) * TY;
+        const int ix = x0 + px, iy = y0 + py, j = iy * N + ix;
+        const bool active = ix < N && iy < N;
+        // stencil
+        float fc = 0.f, gr = 0.f, gx = 0.f, gy = 0.f;
+        if (active) {
+            fc = __ldg(f + j);
+#pragma unroll
+            for (int q8 = 0; q8 < 8 / C; ++q8) {
+                const int q = q8 * C + c;
+                p1_neighbour(f, N, ix, iy, q, fc, a.fs_gamma_r, a.fs_eps, gr, gx, gy);
+            }
+        }
+#pragma unroll
+        for (int o = PX; o < 32; o *= 2) {
+            gr += __shfl_xor_sync(0xffffffffu, gr, o);
+            gx += __shfl_xor_sync(0xffffffffu, gx, o);
+            gy += __shfl_xor_sync(0xffffffffu, gy, o);
+        }
+        // gather
+        float s = 0.f, e = 0.f;
+        // the general entry: sub-ray bins, and views along an axis (membership from the forward
+        // walk's own coordinates)
+        auto any_view = [&](int u) {
+            int b0;
+            float wk[KC];
+            bp_weights<KC, AR, SUB>(g, g.views[a.slot0 + u], a.slot0 + u, ix, iy, b0, wk);
+            const float *row = w + (size_t)u * stride + P1_PAD;
+            float y = 0.f;
+#pragma unroll
+            for (int q = 0; q < KC; ++q) y = fmaf(wk[q], __ldg(row + min(max(b0 + q, 0), NB - 1)), y);
+            p1_add<AR>(y, s, e);
+        };
+        if constexpr (SUB) {
+            if (active)
+                for (int u = c; u < a.nviews; u += C) any_view(u);
+        } else {
+            for (int u0 = 0; u0 < a.nviews; u0 += P1_VIEWS) {
+                const int nvc = min(P1_VIEWS, a.nviews - u0);
+                bool axis = false;
+                __syncwarp();
+                if (lane < nvc) {
+                    const ViewGeo &vw = g.views[a.slot0 + u0 + lane];
+                    const long long xq = vw.t0q - vw.hq + (long long)x0 * vw.cxq + (long long)y0 * vw.cyq;
+                    axis = vw.axis;
+                    P1View v;
+                    v.bin = (int)(xq >> 32);
+                    v.x = (int)(((unsigned)xq >> 6) + (((unsigned)xq >> 5) & 1u));
+                    v.cx = (int)((vw.cxq + 32) >> 6);
+                    v.cy = (int)((vw.cyq + 32) >> 6);
+                    v.row = (unsigned)(u0 + lane) * (unsigned)stride + P1_PAD;
+                    v.h2 = 2.f * vw.hf;
+                    v.ws = axis ? 0.f : vw.wslopef;
+                    v.L = axis ? 0.f : vw.Lf;
+                    vt[lane] = v;
+                }
+                const unsigned axes = __ballot_sync(0xffffffffu, axis);
+                __syncwarp();
+                if (!active) continue;
+#pragma unroll 4
+                for (int u = c; u < nvc; u += C) {
+                    const P1View v = vt[u];
+                    const int x = v.x + px * v.cx + py * v.cy;
+                    const int up = (x + 0x3FFFFFF) >> 26;                            // ceil
+                    const float e0 = (float)((up << 26) - x) * 1.4901161193847656e-8f;   // b0 - (t - h)
+                    const int b0 = min(max(v.bin + up, -P1_PAD), NB + P1_PAD - KC);
+                    const float *row = w + (v.row + (unsigned)b0);
+                    float y = fminf(v.L, fmaxf(0.f, fminf(e0, v.h2 - e0)) * v.ws) * __ldg(row);
+#pragma unroll
+                    for (int q = 1; q < KC; ++q) {
+                        // KC = 2 holds geometries with 2 h < 2: the rising side ends before bin 1
+                        const float r = v.h2 - (e0 + (float)q), d = KC == 2 ? r : fminf(e0 + (float)q, r);
+                        y = fmaf(fminf(v.L, fmaxf(0.f, d) * v.ws), __ldg(row + q), y);
+                    }
+                    p1_add<AR>(y, s, e);
+                }
+                if (axes)
+                    for (int u = c; u < nvc; u += C)
+                        if (axes >> u & 1) any_view(u0 + u);
+            }
+        }
+        const float mine = s + e;
+#pragma unroll
+        for (int cc = 1; cc < C; ++cc) p1_add<AR>(__shfl_sync(0xffffffffu, mine, cc * PX + pl), s, e);
+        // step
+        if (c == 0 && active) {
+            float nu = 1.f;
+            if (a.nu_mode == 3) {
+                nu = __ldg(reinterpret_cast<const float *>(a.nu_frozen) + j);
+            } else if (dyn) {
+                // central differences inside, one-sided at the border
+                gx *= ix > 0 && ix < N - 1 ? 0.5f : 1.f;
+                gy *= iy > 0 && iy < N - 1 ? 0.5f : 1.f;
+                nu = nu_of<float>(gx, gy, 0.f, inv_mean_f, mean_mu, a.fs_nu1, a.fs_nu2);
+                if (a.nu_mode == 2) reinterpret_cast<float *>(a.nu_frozen)[j] = nu;
+            }
+            const float ip = __ldg(reinterpret_cast<const float *>(a.invp) + j) * a.fs_ips;
+            const float coef = a.fs_lam * nu * ((fc < 0.5f * U ? fc : U - fc) * ip);
+            float ft = fc - coef * (scale * (s + e) + a.fs_bm * (2.f * gr));
+            ft = ft <= 0.f ? tt : (ft >= U ? U - tt : ft);
+            part += ft;
+            reinterpret_cast<float *>(a.fout)[j] = ft;
+            reinterpret_cast<float *>(a.fout)[npix + ix * N + iy] = ft;   // the transposed copy
+        }
+    }
+    return part;
+}
+
 // f^{k,i} = P_t(f - lambda_k alpha_{k,i} nu S(f) (A_i^T w + (beta/M) grad R(f))) for one plane.
 // A warp works alone, without block barriers: it takes a patch of 32 / C pixels (8 x 4, 4 x 4,
 // 4 x 2 or 2 x 2, so that one view's bins are a few sectors of the row of w) with C lanes per
@@ -255,7 +382,7 @@ __device__ __forceinline__ void p1_neighbour(const float *f, int N, int ix, int 
 // the sinogram needs no test per bin.  A virtual block is 8 warps x a.tpv patches; only its sum
 // ends in barriers.
 template <int KC, int AR, bool SUB>
-__global__ void __launch_bounds__(256, 4) update_kernel_p1(const __grid_constant__ UpdateArgs one, const Batch bt)
+__global__ void __launch_bounds__(256, SUB ? 3 : 4) update_kernel_p1(const __grid_constant__ UpdateArgs one, const Batch bt)
 {
     __shared__ __align__(16) P1View views[SUB ? 1 : 8][P1_VIEWS];
     __shared__ UpdateArgs sh_args;
@@ -265,14 +392,15 @@ __global__ void __launch_bounds__(256, 4) update_kernel_p1(const __grid_constant
     grid_dependents_launch();
     VblockRuns runs(total_vblocks(one, bt));
     const UpdateArgs *ap = nullptr;
-    int scan = -1, done = 0, vloc = 0, nv = 0;
+    int done = 0, vloc = 0, nv = 0;
+    KeptScan kept;
     float inv_mean_f = 1.f, mean_mu = 1.f;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     for (int vb; (vb = runs.next()) >= 0;) {
-        const bool fresh = scan_args_kept(one, bt, vb, vloc, nv, sh_args, scan, ap);
+        const bool fresh = scan_args_kept(one, bt, vb, vloc, nv, sh_args, kept, ap);
         const UpdateArgs &a = *ap;
         const GeoDev &g = a.g;
-        const int N = g.N, NB = g.NB, npix = N * N, C = a.C, stride = NB + 2 * P1_PAD;
+        const int npix = g.N * g.N;
         const bool dyn = a.nu_mode == 1 || a.nu_mode == 2;
         if (fresh) {
             done = 0;
@@ -281,116 +409,13 @@ __global__ void __launch_bounds__(256, 4) update_kernel_p1(const __grid_constant
                 mean_mu = (float)*a.sum_mu / (float)npix;
             }
         }
-        const int PX = 32 / C, TX = C == 1 ? 8 : (C == 8 ? 2 : 4), TY = PX / TX;
-        const int c = lane / PX, pl = lane - c * PX, py = pl / TX, px = pl - py * TX;
-        const int ntx = (N + TX - 1) / TX, npatch = ntx * ((N + TY - 1) / TY);
-        const float *w = reinterpret_cast<const float *>(a.w);
-        const float *f = reinterpret_cast<const float *>(a.f);
-        const float U = a.fs_U, tt = a.fs_t, scale = a.fs_scale;
         float part = 0.f;
-        for (int k = 0; k < a.tpv; ++k) {
-            const int patch = (vloc * a.tpv + k) * 8 + wid;
-            if (patch >= npatch) break;
-            const int x0 = (patch % ntx) * TX, y0 = (patch / ntx) * TY;
-            const int ix = x0 + px, iy = y0 + py, j = iy * N + ix;
-            const bool active = ix < N && iy < N;
-            // stencil
-            float fc = 0.f, gr = 0.f, gx = 0.f, gy = 0.f;
-            if (active) {
-                fc = __ldg(f + j);
-                for (int q = c; q < 8; q += C)
-                    p1_neighbour(f, N, ix, iy, q, fc, a.fs_gamma_r, a.fs_eps, gr, gx, gy);
-            }
-            for (int o = PX; o < 32; o *= 2) {
-                gr += __shfl_xor_sync(0xffffffffu, gr, o);
-                gx += __shfl_xor_sync(0xffffffffu, gx, o);
-                gy += __shfl_xor_sync(0xffffffffu, gy, o);
-            }
-            // gather
-            float s = 0.f, e = 0.f;
-            // the general entry: sub-ray bins, and views along an axis (membership from the forward
-            // walk's own coordinates)
-            auto any_view = [&](int u) {
-                int b0;
-                float wk[KC];
-                bp_weights<KC, AR, SUB>(g, g.views[a.slot0 + u], a.slot0 + u, ix, iy, b0, wk);
-                const float *row = w + (size_t)u * stride + P1_PAD;
-                float y = 0.f;
-#pragma unroll
-                for (int q = 0; q < KC; ++q) y = fmaf(wk[q], __ldg(row + min(max(b0 + q, 0), NB - 1)), y);
-                p1_add<AR>(y, s, e);
-            };
-            if constexpr (SUB) {
-                if (active)
-                    for (int u = c; u < a.nviews; u += C) any_view(u);
-            } else {
-                P1View *vt = views[wid];
-                for (int u0 = 0; u0 < a.nviews; u0 += P1_VIEWS) {
-                    const int nvc = min(P1_VIEWS, a.nviews - u0);
-                    bool axis = false;
-                    __syncwarp();
-                    if (lane < nvc) {
-                        const ViewGeo &vw = g.views[a.slot0 + u0 + lane];
-                        const long long xq = vw.t0q - vw.hq + (long long)x0 * vw.cxq + (long long)y0 * vw.cyq;
-                        axis = vw.axis;
-                        P1View v;
-                        v.bin = (int)(xq >> 32);
-                        v.x = (int)(((unsigned)xq >> 6) + (((unsigned)xq >> 5) & 1u));
-                        v.cx = (int)((vw.cxq + 32) >> 6);
-                        v.cy = (int)((vw.cyq + 32) >> 6);
-                        v.row = (unsigned)(u0 + lane) * (unsigned)stride + P1_PAD;
-                        v.h2 = 2.f * vw.hf;
-                        v.ws = axis ? 0.f : vw.wslopef;
-                        v.L = axis ? 0.f : vw.Lf;
-                        vt[lane] = v;
-                    }
-                    const unsigned axes = __ballot_sync(0xffffffffu, axis);
-                    __syncwarp();
-                    if (!active) continue;
-#pragma unroll 4
-                    for (int u = c; u < nvc; u += C) {
-                        const P1View v = vt[u];
-                        const int x = v.x + px * v.cx + py * v.cy;
-                        const int up = (x + 0x3FFFFFF) >> 26;                            // ceil
-                        const float e0 = (float)((up << 26) - x) * 1.4901161193847656e-8f;   // b0 - (t - h)
-                        const int b0 = min(max(v.bin + up, -P1_PAD), NB + P1_PAD - KC);
-                        const float *row = w + (v.row + (unsigned)b0);
-                        float y = fminf(v.L, fmaxf(0.f, fminf(e0, v.h2 - e0)) * v.ws) * __ldg(row);
-#pragma unroll
-                        for (int q = 1; q < KC; ++q) {
-                            // KC = 2 holds geometries with 2 h < 2: the rising side ends before bin 1
-                            const float r = v.h2 - (e0 + (float)q), d = KC == 2 ? r : fminf(e0 + (float)q, r);
-                            y = fmaf(fminf(v.L, fmaxf(0.f, d) * v.ws), __ldg(row + q), y);
-                        }
-                        p1_add<AR>(y, s, e);
-                    }
-                    if (axes)
-                        for (int u = c; u < nvc; u += C)
-                            if (axes >> u & 1) any_view(u0 + u);
-                }
-            }
-            const float mine = s + e;
-            for (int cc = 1; cc < C; ++cc) p1_add<AR>(__shfl_sync(0xffffffffu, mine, cc * PX + pl), s, e);
-            // step
-            if (c == 0 && active) {
-                float nu = 1.f;
-                if (a.nu_mode == 3) {
-                    nu = __ldg(reinterpret_cast<const float *>(a.nu_frozen) + j);
-                } else if (dyn) {
-                    // central differences inside, one-sided at the border
-                    gx *= ix > 0 && ix < N - 1 ? 0.5f : 1.f;
-                    gy *= iy > 0 && iy < N - 1 ? 0.5f : 1.f;
-                    nu = nu_of<float>(gx, gy, 0.f, inv_mean_f, mean_mu, a.fs_nu1, a.fs_nu2);
-                    if (a.nu_mode == 2) reinterpret_cast<float *>(a.nu_frozen)[j] = nu;
-                }
-                const float ip = __ldg(reinterpret_cast<const float *>(a.invp) + j) * a.fs_ips;
-                const float coef = a.fs_lam * nu * ((fc < 0.5f * U ? fc : U - fc) * ip);
-                float ft = fc - coef * (scale * (s + e) + a.fs_bm * (2.f * gr));
-                ft = ft <= 0.f ? tt : (ft >= U ? U - tt : ft);
-                part += ft;
-                reinterpret_cast<float *>(a.fout)[j] = ft;
-                reinterpret_cast<float *>(a.fout)[npix + ix * N + iy] = ft;   // the transposed copy
-            }
+        P1View *vt = views[SUB ? 0 : wid];
+        switch (a.C) {
+        case 1: part = p1_patches<KC, AR, SUB, 1>(a, vt, vloc, wid, lane, inv_mean_f, mean_mu); break;
+        case 2: part = p1_patches<KC, AR, SUB, 2>(a, vt, vloc, wid, lane, inv_mean_f, mean_mu); break;
+        case 4: part = p1_patches<KC, AR, SUB, 4>(a, vt, vloc, wid, lane, inv_mean_f, mean_mu); break;
+        default: part = p1_patches<KC, AR, SUB, 8>(a, vt, vloc, wid, lane, inv_mean_f, mean_mu);
         }
         // the block's 256 partial sums, added in FP64 by one warp (the FP64 pipe is narrow)
         part_sh[threadIdx.x] = part;
@@ -426,13 +451,15 @@ static const void *fwd_p1_fn(int mode, int sub)
                                : (const void *)fwd_kernel_p1<AR, FWD_OBJECTIVE, false>;
 }
 
-// Chunks per ray: enough threads for one wave of 2048 per SM, at least 8 driving steps each.
+// Chunks per ray: enough threads for one wave of 2048 per SM, at least 16 driving steps each (8 for
+// sub-ray bins, whose steps are about ten times the work).
 void forward_shape_p1(FwdArgs &a, int mode, int arith)
 {
     const long long nrays = (long long)a.nviews * a.g.NB;
     const long long want = (long long)sm_count() * 2048;
+    const int least = a.g.table ? 8 : 16;
     int S = 1;
-    while (S < P1_MAX_CHUNKS && nrays * S < want && a.g.N / (2 * S) >= 8) S *= 2;
+    while (S < P1_MAX_CHUNKS && nrays * S < want && a.g.N / (2 * S) >= least) S *= 2;
     if (a.g.tuneS > 0 && mode != FWD_OBJECTIVE) S = a.g.tuneS;
     a.S = S;
     a.R = 256 / S;

@@ -28,12 +28,20 @@
 
 namespace pet {
 
+constexpr int Q52_MAX_N = 1024;  // image sides whose FP64 walk keeps its positions in Q11.52
+
 // Thread layout: a virtual block is R rays x S chunks x NG plane groups (thread = (ray * S +
 // chunk) * NG + group; threads beyond R S NG idle).  Chunk c walks driving steps
 // [c Lc, (c + 1) Lc) of its ray, Lc = ceil(nd / S), so that short subsets still fill the GPU; the
 // S partial sums of a (ray, group) are combined in chunk order through shared memory
 // (deterministic).  A persistent grid strides over the virtual blocks of one scan or a batch.
-template <int G, int AR, int MODE, bool SUB>
+// U (FP32): driving steps whose loads are issued together.  Two fit three blocks per SM, four take 128
+// registers and two blocks: more loads in flight per thread, fewer threads.  Four are faster on long
+// chunks (all views of 256 x 256 x 89, S = 1: 570 us, two 613, one 665) and where the tiles do not
+// fill three blocks per SM anyway (one iteration of 200 x 200 x 24: 914 us, two 1030); two on the short
+// chunks of a subset split over many tiles (256 x 256 x 89, S = 7: 2759 us an iteration, four 2943).
+// The sums are the same bits.
+template <int G, int AR, int MODE, bool SUB, int U>
 __device__ __forceinline__ void fwd_vblock(const FwdArgs &a, int vloc, int nv,
                                            typename ArithT<AR>::T *comb_s, typename ArithT<AR>::T *comb_e)
 {
@@ -78,6 +86,37 @@ __device__ __forceinline__ void fwd_vblock(const FwdArgs &a, int vloc, int nv,
         const int nsr = SUB ? g.R : 1;
         if constexpr (AR == AR_FP64) {
             const double step = vw.step, ast = fabs(vw.step), L = vw.L, im = vw.inv_minor;
+            if (N <= Q52_MAX_N && (!SUB || nsr * fabs(rg.sh) < 256.0)) {      // |lo| < 2^11
+                // The FP64 pipe (two lanes per SM and cycle) is what this walk waits for, so the
+                // positions are kept in Q11.52 integers, as exact as the doubles at these sizes,
+                // and a lane takes one pixel per turn (the step's second pixel only where the line
+                // crosses into it): 11 FP64 operations per pixel of 8 planes instead of 25 per step.
+                const long long stq = __double2ll_rn(step * 4503599627370496.0), aq = stq < 0 ? -stq : stq;
+                for (int sr = 0; sr < nsr; ++sr) {
+                    const double lo0 = rg.lo + (2 * sr + 1 - nsr) * (SUB ? rg.sh : vw.half);
+                    long long lo = __double2ll_rn(fma((double)k0, step, lo0) * 4503599627370496.0);
+                    bool second = false;
+                    for (int k = k0; k < k1;) {
+                        const long long hi = lo + aq;
+                        const int r0 = (int)(lo >> 52), r1 = (int)(hi >> 52);
+                        const bool cross = r1 != r0;
+                        const double frac = __longlong_as_double(0x3FF0000000000000LL | (hi & 0xFFFFFFFFFFFFFLL)) - 1.0;
+                        const double l1 = cross ? frac * im : 0.0;
+                        const int r = second ? r1 : r0;
+                        const double l = second ? l1 : L - l1;
+                        if ((unsigned)r < (unsigned)N) {
+                            T x[G];
+                            load_group<G, T>(img + (unsigned)((rg.d0 + k) * ds + r * cs) * (unsigned)Pp, x);
+                            acc.add1term(l, x);
+                        }
+                        second = cross && !second;
+                        if (!second) {
+                            ++k;
+                            lo += stq;
+                        }
+                    }
+                }
+            } else
             for (int sr = 0; sr < nsr; ++sr)
             for (int k = k0; k < k1; ++k) {
                 const int d = rg.d0 + k;
@@ -126,27 +165,54 @@ __device__ __forceinline__ void fwd_vblock(const FwdArgs &a, int vloc, int nv,
             for (int sr = 0; sr < nsr; ++sr) {
             unsigned base = (unsigned)(rg.d0 + k0) * dstep;
             long long lo = rg.loq + (long long)(2 * sr + 1 - nsr) * (SUB ? rg.shq : vw.halfq) + (long long)k0 * stp;
-            for (int k = k0; k < k1; ++k) {
+            // U steps at a time (their loads are issued together, the sums in step order)
+            int k = k0;
+            auto prep = [&](unsigned &o0, unsigned &o1, bool &ok1, float &l0, float &l1) {
                 const long long hi = lo + ast;
                 const int r0 = (int)(lo >> 32), r1 = (int)(hi >> 32);
                 const bool cross = r1 != r0;
                 const bool ok0 = (unsigned)r0 < (unsigned)N;
-                const bool ok1 = cross && (unsigned)r1 < (unsigned)N;
+                ok1 = cross && (unsigned)r1 < (unsigned)N;
                 const float fr = __uint_as_float(0x3F800000u | ((unsigned)hi >> 9)) - 1.f;
                 const float t1 = cross ? fr * imb : 0.f;
-                const float l1 = ok1 ? t1 : 0.f;
-                const float l0 = ok0 ? L - t1 : 0.f;
-                const unsigned o0 = base + (ok0 ? (unsigned)r0 * cstep : 0u);
-                const unsigned o1 = base + (ok1 ? (unsigned)r1 * cstep : 0u);
+                l1 = ok1 ? t1 : 0.f;
+                l0 = ok0 ? L - t1 : 0.f;
+                o0 = base + (ok0 ? (unsigned)r0 * cstep : 0u);
+                o1 = base + (ok1 ? (unsigned)r1 * cstep : 0u);
+                lo += stp;
+                base += dstep;
+            };
+            for (; k + U <= k1; k += U) {
+                f2x x0[U][4], x1[U][4];
+                float l0[U], l1[U];
+#pragma unroll
+                for (int i = 0; i < U; ++i) {
+                    unsigned o0, o1;
+                    bool ok1;
+                    prep(o0, o1, ok1, l0[i], l1[i]);
+                    load8x(imf + o0, x0[i]);
+                    load8x_if(imf + o1, ok1, x1[i]);
+                }
+#pragma unroll
+                for (int i = 0; i < U; ++i) {
+                    const f2x W0 = vsplat(l0[i]), W1 = vsplat(l1[i]);
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) bl[q] = vfma(W1, x1[i][q], vfma(W0, x0[i][q], bl[q]));
+                    if (++nb == 8) { merge(); nb = 0; }
+                }
+            }
+            for (; k < k1; ++k) {
                 f2x x0[4], x1[4];
+                float l0, l1;
+                unsigned o0, o1;
+                bool ok1;
+                prep(o0, o1, ok1, l0, l1);
                 load8x(imf + o0, x0);
                 load8x_if(imf + o1, ok1, x1);
                 const f2x W0 = vsplat(l0), W1 = vsplat(l1);
 #pragma unroll
                 for (int q = 0; q < 4; ++q) bl[q] = vfma(W1, x1[q], vfma(W0, x0[q], bl[q]));
                 if (++nb == 8) { merge(); nb = 0; }
-                lo += stp;
-                base += dstep;
             }
             }
             merge();
@@ -284,8 +350,8 @@ __device__ __forceinline__ void fwd_vblock(const FwdArgs &a, int vloc, int nv,
     if constexpr (MODE == FWD_OBJECTIVE) grid_reduce<2>(obj, a.red, a.result, vloc, nv);
 }
 
-template <int G, int AR, int MODE, bool SUB = false>
-__global__ void __launch_bounds__(256, 3) fwd_kernel(const __grid_constant__ FwdArgs one, const Batch bt)
+template <int G, int AR, int MODE, bool SUB = false, int U = 2>
+__global__ void __launch_bounds__(256, U == 4 ? 2 : 3) fwd_kernel(const __grid_constant__ FwdArgs one, const Batch bt)
 {
     grid_dependency_wait();                      // before any memory access
     grid_dependents_launch();                    // the update may be scheduled behind this kernel
@@ -297,7 +363,7 @@ __global__ void __launch_bounds__(256, 3) fwd_kernel(const __grid_constant__ Fwd
     for (int vb = blockIdx.x; vb < total; vb += gridDim.x) {
         int vloc, nv;
         const FwdArgs &a = scan_args(one, bt, vb, vloc, nv, sh_args);
-        fwd_vblock<G, AR, MODE, SUB>(a, vloc, nv, comb_s, comb_e);
+        fwd_vblock<G, AR, MODE, SUB, U>(a, vloc, nv, comb_s, comb_e);
     }
 }
 
@@ -306,8 +372,8 @@ __global__ void __launch_bounds__(256, 3) fwd_kernel(const __grid_constant__ Fwd
 // pass's short blocks come last and fill the projection's tail; as a launch of its own on a side
 // stream it cost a fork and a join of events per subiteration and kept the update from being
 // scheduled behind the projection.
-template <int AR, bool SUB>
-__global__ void __launch_bounds__(256, 3) fwd_mu_kernel(const __grid_constant__ FwdArgs fwd,
+template <int AR, bool SUB, int U>
+__global__ void __launch_bounds__(256, U == 4 ? 2 : 3) fwd_mu_kernel(const __grid_constant__ FwdArgs fwd,
                                                         const __grid_constant__ ImageArgs mu, int nfwd)
 {
     grid_dependency_wait();
@@ -315,8 +381,18 @@ __global__ void __launch_bounds__(256, 3) fwd_mu_kernel(const __grid_constant__ 
     __shared__ float comb_s[256 * 8];
     __shared__ float comb_e[256 * 8];
     const int vb = (int)blockIdx.x;
-    if (vb < nfwd) fwd_vblock<8, AR, FWD_RATIO, SUB>(fwd, vb, nfwd, comb_s, comb_e);
+    if (vb < nfwd) fwd_vblock<8, AR, FWD_RATIO, SUB, U>(fwd, vb, nfwd, comb_s, comb_e);
     else mu_x8_vblock(mu, vb - nfwd, mu.nvb);
+}
+
+int sm_count();
+
+// U of a stack's projection (see fwd_vblock), from its launch shape; batched launches (N = 0 here) take 2.
+static int fwd_steps(const FwdArgs &a)
+{
+    if (a.g.N == 0 || a.S < 1 || a.R < 1) return 2;
+    const long long tiles = (long long)a.nviews * ((a.g.NB + a.R - 1) / a.R);
+    return a.g.N / a.S >= 128 || tiles <= 2LL * sm_count() ? 4 : 2;
 }
 
 template <int G, int AR>
@@ -328,6 +404,14 @@ static void fwd_dispatch_mode(const FwdArgs &a, const Batch &b, int mode, int gr
         else if (mode == FWD_RATIO) launch_pdl(fwd_kernel<G, AR, FWD_RATIO, true>, grid, st, pdl, a, b);
         else launch_pdl(fwd_kernel<G, AR, FWD_OBJECTIVE, true>, grid, st, pdl, a, b);
         return;
+    }
+    if constexpr (G == 8 && AR != AR_FP64) {
+        if (fwd_steps(a) == 4) {
+            if (mode == FWD_PLAIN) launch_pdl(fwd_kernel<G, AR, FWD_PLAIN, false, 4>, grid, st, pdl, a, b);
+            else if (mode == FWD_RATIO) launch_pdl(fwd_kernel<G, AR, FWD_RATIO, false, 4>, grid, st, pdl, a, b);
+            else launch_pdl(fwd_kernel<G, AR, FWD_OBJECTIVE, false, 4>, grid, st, pdl, a, b);
+            return;
+        }
     }
     if (mode == FWD_PLAIN) launch_pdl(fwd_kernel<G, AR, FWD_PLAIN>, grid, st, pdl, a, b);
     else if (mode == FWD_RATIO) launch_pdl(fwd_kernel<G, AR, FWD_RATIO>, grid, st, pdl, a, b);
@@ -421,7 +505,8 @@ void forward_shape(FwdArgs &a, int mode, int arith)
     if (mode == FWD_OBJECTIVE) {
         // each virtual block ends in a block reduction and a grid-wide ticket: one wave of them
         const void *fn = a.g.G == 1 ? fwd_fn_g<1>(mode, arith, a.g.table) : fwd_fn_g<8>(mode, arith, a.g.table);
-        const long long slots = (long long)sm_count() * resident_blocks(fn);
+        const bool four = a.g.G == 8 && arith != AR_FP64 && !a.g.table && fwd_steps(a) == 4;
+        const long long slots = (long long)sm_count() * (four ? 2 : resident_blocks(fn));
         long long tpv = (ntiles + slots - 1) / slots;
         if (a.red.capacity > 0) tpv = std::max(tpv, (ntiles + a.red.capacity - 1) / a.red.capacity);
         a.tpv = (int)std::max(1LL, tpv);
@@ -466,11 +551,14 @@ pet_status launch_forward_mu(const FwdArgs &a0, const ImageArgs &m0, int arith, 
     } else {
         const int grid = a.nvb + m.nvb;
         if (a.g.table) {
-            if (arith == AR_KAHAN) launch_pdl(fwd_mu_kernel<AR_KAHAN, true>, grid, st, true, a, m, a.nvb);
-            else launch_pdl(fwd_mu_kernel<AR_FP32, true>, grid, st, true, a, m, a.nvb);
+            if (arith == AR_KAHAN) launch_pdl(fwd_mu_kernel<AR_KAHAN, true, 2>, grid, st, true, a, m, a.nvb);
+            else launch_pdl(fwd_mu_kernel<AR_FP32, true, 2>, grid, st, true, a, m, a.nvb);
+        } else if (fwd_steps(a) == 4) {
+            if (arith == AR_KAHAN) launch_pdl(fwd_mu_kernel<AR_KAHAN, false, 4>, grid, st, true, a, m, a.nvb);
+            else launch_pdl(fwd_mu_kernel<AR_FP32, false, 4>, grid, st, true, a, m, a.nvb);
         } else {
-            if (arith == AR_KAHAN) launch_pdl(fwd_mu_kernel<AR_KAHAN, false>, grid, st, true, a, m, a.nvb);
-            else launch_pdl(fwd_mu_kernel<AR_FP32, false>, grid, st, true, a, m, a.nvb);
+            if (arith == AR_KAHAN) launch_pdl(fwd_mu_kernel<AR_KAHAN, false, 2>, grid, st, true, a, m, a.nvb);
+            else launch_pdl(fwd_mu_kernel<AR_FP32, false, 2>, grid, st, true, a, m, a.nvb);
         }
     }
     cudaError_t e = cudaGetLastError();

@@ -213,9 +213,10 @@ __global__ void __launch_bounds__(256) image_kernel(const __grid_constant__ Imag
     __shared__ double red_sh[1][32];
     VblockRuns runs(total_vblocks(one, bt));
     const ImageArgs *ap = nullptr;
-    int scan = -1, done = 0, vloc = 0, nv = 0;
+    int done = 0, vloc = 0, nv = 0;
+    KeptScan kept;
     for (int vb; (vb = runs.next()) >= 0;) {
-        if (scan_args_kept(one, bt, vb, vloc, nv, sh_args, scan, ap)) done = 0;
+        if (scan_args_kept(one, bt, vb, vloc, nv, sh_args, kept, ap)) done = 0;
         const ImageArgs &a = *ap;
         const GeoDev &g = a.g;
         const int N = g.N, NG = g.NG, Pp = g.Pp;
@@ -338,9 +339,9 @@ void update_shape(UpdateArgs &a, int arith)
 {
     if (plane1_path(a.g, arith) && !a.tv) { update_shape_p1(a, arith); return; }
     const int TP = 256 / a.g.NG;
-    const int ntiles = (a.g.N * a.g.N + TP - 1) / TP;
+    const int ntiles = update_x8_path(a, arith) ? update_x8_tiles(a) : (a.g.N * a.g.N + TP - 1) / TP;
     const int sub = a.g.table, tof = a.g.T > 1;
-    const void *fn = update_x8_path(a.g, arith) ? update_x8_fn(a, arith)
+    const void *fn = update_x8_path(a, arith) ? update_x8_fn(a, arith)
                      : a.g.G == 1 ? (a.g.K <= 2 ? update_fn<1, 2>(arith, sub, tof) : update_fn<1, 4>(arith, sub, tof))
                                   : (a.g.K <= 2 ? update_fn<8, 2>(arith, sub, tof) : update_fn<8, 4>(arith, sub, tof));
     const int slots = sm_count() * resident_blocks(fn);
@@ -398,7 +399,7 @@ static pet_status update_any(const UpdateArgs &a, const Batch &b, int arith, int
     LaunchScope ls(PET_K_UPDATE, st);
     if (plane1_path(a.g, arith) && !a.tv) {
         update_p1_dispatch(a, b, arith, grid, st, pdl);
-    } else if (update_x8_path(a.g, arith)) {
+    } else if (update_x8_path(a, arith)) {
         update_x8_dispatch(a, b, arith, grid, st, pdl);
     } else if (a.g.G == 1) {
         if (a.g.K <= 2) update_dispatch<1, 2>(a, b, arith, grid, st, pdl);
@@ -457,7 +458,9 @@ pet_status launch_back(const BackArgs &a, int arith, cudaStream_t st)
     const int ntiles = (a.g.N * a.g.N + TP - 1) / TP;
     const int grid = persistent_grid(ntiles);
     LaunchScope ls(PET_K_OTHER, st);
-    if (a.g.G == 1) {
+    if (back_quad_path(a, arith)) {
+        back_quad_dispatch(a, arith, st);
+    } else if (a.g.G == 1) {
         if (a.g.K <= 2) back_dispatch<1, 2>(a, arith, grid, st);
         else back_dispatch<1, 4>(a, arith, grid, st);
     } else {

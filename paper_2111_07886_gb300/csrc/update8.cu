@@ -1,16 +1,102 @@
 // The FP32 update of stacks (8-plane groups): one packed kernel for the in-plane and the 3-D prior,
 // 1/p per pixel or per voxel, and the TV variant, and its precomputed backprojection entries.
+#include <math.h>
+
 #include "kernels.cuh"
 #include "profile.cuh"
-
-#ifndef UPDATE_X8_BLOCKS
-#define UPDATE_X8_BLOCKS 3      // resident blocks per SM the packed update kernel is built for
-#endif
 
 namespace pet {
 
 int sm_count();
-constexpr int X8_Z3 = 1, X8_VOX = 2, X8_TV = 4;
+constexpr int X8_Z3 = 1, X8_VOX = 2, X8_TV = 4, X8_TOF = 8;
+
+// TOF: a (pixel, view) entry is X8_HD words (row offset, first TOF bin | count << 8, KC lengths) and
+// h_t for up to g.tof_hw TOF bins; X8_TOF_WORDS of them in shared memory.  A tile is a TX x TY patch,
+// as square as 256 / NG pixels allow: a view's rows [bin][T] of a patch overlap in two directions.
+constexpr int X8_TOF_WORDS = 6144;
+struct X8Patch { int tx, ty, es; };
+template <int KC>
+static __host__ __device__ __forceinline__ X8Patch x8_patch(const GeoDev &g)
+{
+    X8Patch p;
+    p.es = (KC <= 2 ? 4 : 8) + (g.tof_hw + 3) / 4 * 4;
+    int n = 256 / g.NG;
+    if (n > X8_TOF_WORDS / p.es) n = X8_TOF_WORDS / p.es;
+    p.ty = 1;
+    while ((p.ty + 1) * (p.ty + 1) <= n) ++p.ty;
+    p.tx = n / p.ty;
+    return p;
+}
+
+// One TOF entry of pixel (ix, iy) and view u of the subset: the row offset and lengths of bp_entry,
+// the TOF bins whose centre lies within the kernel's window of the pixel's position along the view's
+// lines, and h_t of each (each bin edge's erfc evaluated once; the tail form of tof_h).
+template <int KC, int AR>
+__device__ __forceinline__ void tof_entry(const GeoDev &g, int slot0, int u, int ix, int iy, float *out)
+{
+    const bool in = ix < g.N && iy < g.N;
+    const auto ent = bp_entry<KC, AR, 0>(g, slot0, u, in, ix, iy);
+    const ViewGeo &vw = g.views[slot0 + u];
+    const float tau = vw.tau0f + (float)ix * vw.tauxf + (float)iy * vw.tauyf;
+    const float d = g.tof_df, kk = g.tof_kf, W = g.tof_wf;
+    const float tc = tau / d + 0.5f * (float)(g.T - 1);
+    const int t_lo = max(0, (int)ceilf(tc - W / d)), t_hi = min(g.T - 1, (int)floorf(tc + W / d));
+    const int n = min(in ? max(0, t_hi - t_lo + 1) : 0, g.tof_hw);
+    out[0] = __uint_as_float(ent.off);
+    out[1] = __int_as_float(t_lo | n << 8);
+#pragma unroll
+    for (int k = 0; k < KC; ++k) out[2 + k] = ent.w[k];
+    float *h = out + (KC <= 2 ? 4 : 8);
+    float z0 = ((float)(2 * t_lo - g.T) * 0.5f * d - tau) * kk, c0 = erfcf(fabsf(z0));
+    for (int t = 0; t < n; ++t) {
+        const float z1 = ((float)(2 * (t_lo + t) + 2 - g.T) * 0.5f * d - tau) * kk, c1 = erfcf(fabsf(z1));
+        h[t] = z0 >= 0.f ? 0.5f * (c0 - c1) : (z1 <= 0.f ? 0.5f * (c1 - c0) : 1.f - 0.5f * (c0 + c1));
+        z0 = z1;
+        c0 = c1;
+    }
+}
+
+// Adds an entry's rows [bin][T] to a thread's sums: four TOF bins by FMAs, then one compensated step.
+template <int KC, int AR>
+__device__ __forceinline__ void tof_gather(const GeoDev &g, const float *w, const float *ent, f2x (&sm)[4], f2x (&er)[4])
+{
+    const unsigned Pp = (unsigned)g.Pp, TT = (unsigned)g.T;
+    const int tn = __float_as_int(ent[1]), n = tn >> 8;
+    float l[KC];
+#pragma unroll
+    for (int k = 0; k < KC; ++k) l[k] = ent[2 + k];
+    const float *h = ent + (KC <= 2 ? 4 : 8);
+    const float *row = w + (__float_as_uint(ent[0]) * TT + (unsigned)(tn & 255) * Pp);
+    for (int t0 = 0; t0 < n; t0 += 4) {
+        f2x bl[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) bl[k] = 0ull;
+#pragma unroll 2
+        for (int t = t0; t < min(n, t0 + 4); ++t) {
+            const float ht = h[t];
+#pragma unroll
+            for (int kb = 0; kb < KC; ++kb) {
+                f2x x[4];
+                load8x(row + (unsigned)kb * TT * Pp, x);
+                const f2x W = vsplat(ht * l[kb]);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) bl[k] = vfma(W, x[k], bl[k]);
+            }
+            row += Pp;
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            if constexpr (AR == AR_KAHAN) {
+                const f2x y = vadd(bl[k], er[k]);
+                const f2x s = vadd(sm[k], y);
+                er[k] = vsub(y, vsub(s, sm[k]));
+                sm[k] = s;
+            } else {
+                sm[k] = vadd(sm[k], bl[k]);
+            }
+        }
+    }
+}
 
 // FP32 update for 8-plane groups held as four f32x2 pairs.  Same step as update_kernel, with:
 //   - the 3x3 stencil loading every neighbour with missing ones (image border) replaced by the
@@ -25,15 +111,21 @@ constexpr int X8_Z3 = 1, X8_VOX = 2, X8_TV = 4;
 // FL: X8_Z3, the 3-D prior: RDP over the 26 neighbours and nu from the 3-D gradient (each in-plane
 // position's group is used as it is and shifted by one plane up and down); X8_VOX, 1/p per voxel
 // (scans with per-bin detection factors); X8_TV, the TV variant (no RDP term, the unclamped z and
-// the metric W written for the proximal step).
-template <int KC, int AR, int FL>
-__global__ void __launch_bounds__(256, FL & X8_Z3 ? 2 : UPDATE_X8_BLOCKS) update_kernel_x8(
+// the metric W written for the proximal step); X8_TOF, time of flight (see x8_patch).
+// UV: views whose rows are loaded together in the gather.  Four take 128 registers, two blocks per
+// SM and 8 loads in flight per thread; one takes 80 and three blocks.  The rates per tile are about
+// the same (four 2.6 % faster), so what decides is how evenly the tiles fill the resident blocks
+// (x8_views); the sums are the same bits.
+template <int KC, int AR, int FL, int UV = 4>
+__global__ void __launch_bounds__(256, UV == 1 ? 3 : 2) update_kernel_x8(
     const __grid_constant__ UpdateArgs one, const Batch bt)
 {
     static_assert(AR != AR_FP64, "FP32 arithmetic only");
     // 16 KB of (pixel, view) entries: the rest of the SM's shared memory stays L1 for the gather
     using Table = BpTable<KC, AR, 1024 / (KC > 2 ? 2 : 1)>;
-    __shared__ Table tb;
+    constexpr bool TOF = FL & X8_TOF;
+    __shared__ typename std::conditional<TOF, X8Patch, Table>::type tb;
+    __shared__ __align__(16) float tofs[TOF ? X8_TOF_WORDS : 4];
     // launched behind the projection (see launch_update): nothing is read before it has completed
     grid_dependency_wait();
     // the next subiteration's projection (launched after this kernel with programmatic stream
@@ -47,9 +139,11 @@ __global__ void __launch_bounds__(256, FL & X8_Z3 ? 2 : UPDATE_X8_BLOCKS) update
         const GeoDev &g = a.g;
         const int N = g.N, NG = g.NG, npix = N * N;
         const unsigned Pp = (unsigned)g.Pp;
-        const int TP = 256 / NG;
+        const X8Patch pa = TOF ? x8_patch<KC>(g) : X8Patch{0, 0, 0};
+        const int TP = TOF ? pa.tx * pa.ty : 256 / NG;
         const int pl = threadIdx.x / NG, grp = threadIdx.x % NG;
-        const int VC = max(1, min(a.nviews, Table::CAP / TP));
+        const int VC = max(1, min(a.nviews, TOF ? X8_TOF_WORDS / (TP * pa.es) : Table::CAP / TP));
+        const int ntx = TOF ? (N + pa.tx - 1) / pa.tx : 1;
         const bool dyn = a.nu_mode == 1 || a.nu_mode == 2;
         const double q = (double)npix * g.P;
         // per-scan scalars in FP32 (an FP64 division per thread is costly at GB300's FP64 rate)
@@ -61,27 +155,32 @@ __global__ void __launch_bounds__(256, FL & X8_Z3 ? 2 : UPDATE_X8_BLOCKS) update
         const float *f = reinterpret_cast<const float *>(a.f) + grp * 8;
         const float *w = reinterpret_cast<const float *>(a.w) + grp * 8;
         const float *invp = reinterpret_cast<const float *>(a.invp);
-        const int ntiles = (npix + TP - 1) / TP;
+        const int ntiles = TOF ? ntx * ((N + pa.ty - 1) / pa.ty) : (npix + TP - 1) / TP;
         // the subset's precomputed entries (one contiguous block per tile) when two tiles' entries
         // fit the table: double-buffered, the next tile's block copied with cp.async while this
         // tile is gathered and the next one's stencil runs (one barrier per tile)
-        const bool pre = a.bptab && 2 * a.nviews * TP <= Table::CAP;
+        const bool pre = !TOF && a.bptab && 2 * a.nviews * TP <= Table::CAP;
         const int t0 = vloc * a.tpv, t1 = min(ntiles, (vloc + 1) * a.tpv);
         auto copy_tile = [&](int tile) {
             const int tbytes = a.nviews * TP * (int)sizeof(typename Table::E);
             const char *src = static_cast<const char *>(a.bptab) + (size_t)tile * tbytes;
-            char *dst = reinterpret_cast<char *>(tb.e) + ((tile - t0) & 1) * tbytes;
-            for (int o = threadIdx.x * 16; o < tbytes; o += 256 * 16) cp_async16(dst + o, src + o);
-            cp_async_commit();
+            if constexpr (!TOF) {
+                char *dst = reinterpret_cast<char *>(tb.e) + ((tile - t0) & 1) * tbytes;
+                for (int o = threadIdx.x * 16; o < tbytes; o += 256 * 16) cp_async16(dst + o, src + o);
+                cp_async_commit();
+            }
         };
         if (pre && t0 < t1) copy_tile(t0);
         float part = 0.f;
         for (int tile = t0; tile < t1; ++tile) {
-            const int j0 = tile * TP, j = j0 + pl;
-            const bool active = pl < TP && j < npix;
+            const int j0 = tile * TP;
+            const int qy = TOF ? pl / pa.tx : 0, qx = TOF ? pl - qy * pa.tx : 0;
+            const int px0 = TOF ? (tile % ntx) * pa.tx : 0, py0 = TOF ? (tile / ntx) * pa.ty : 0;
+            const int ix = TOF ? px0 + qx : (j0 + pl) % N, iy = TOF ? py0 + qy : (j0 + pl) / N;
+            const int j = TOF ? iy * N + ix : j0 + pl;
+            const bool active = pl < TP && (TOF ? ix < N && iy < N : j < npix);
             f2x A[4], B[4];
             if (active) {
-                const int ix = j % N, iy = j / N;
                 const unsigned jc = (unsigned)j;
                 const unsigned xm = ix > 0 ? jc - 1 : jc, xp = ix < N - 1 ? jc + 1 : jc;
                 const unsigned ym = iy > 0 ? jc - N : jc, yp = iy < N - 1 ? jc + N : jc;
@@ -240,18 +339,66 @@ __global__ void __launch_bounds__(256, FL & X8_Z3 ? 2 : UPDATE_X8_BLOCKS) update
             for (int k = 0; k < 4; ++k) { sm[k] = 0ull; er[k] = 0ull; }
             for (int u0 = 0; u0 < a.nviews; u0 += VC) {
                 const int nvc = min(VC, a.nviews - u0);
-                if (pre) {
+                if constexpr (TOF) {
+                    __syncthreads();
+                    for (int e = threadIdx.x; e < TP * nvc; e += 256) {
+                        const int uu = e / TP, p = e - uu * TP, yy = p / pa.tx;
+                        const int x = px0 + p - yy * pa.tx, y = py0 + yy;
+                        tof_entry<KC, AR>(g, a.slot0, u0 + uu, x, y, tofs + e * pa.es);
+                    }
+                    __syncthreads();
+                } else if (pre) {
                     cp_async_wait_all();             // this tile's block (this thread's part)
                     __syncthreads();                 // all parts; the previous gather is done
                     if (tile + 1 < t1) copy_tile(tile + 1);
                 } else {
                     __syncthreads();
-                    bp_fill<KC, AR>(g, a.slot0, u0, nvc, j0, TP, tb);
+                    if constexpr (!TOF) bp_fill<KC, AR>(g, a.slot0, u0, nvc, j0, TP, tb);
                     __syncthreads();
                 }
                 if (!active) continue;
+                if constexpr (TOF) {
+                    for (int uu = 0; uu < nvc; ++uu)
+                        tof_gather<KC, AR>(g, w, tofs + (uu * TP + pl) * pa.es, sm, er);
+                    continue;
+                } else {
                 const typename Table::E *te = tb.e + (pre ? ((tile - t0) & 1) * a.nviews * TP : 0);
-                for (int uu = 0; uu < nvc; ++uu) {
+                // two bins of a view, one compensated step
+                auto add = [&](float w0, const f2x(&x0)[4], float w1, const f2x(&x1)[4]) {
+                    const f2x W0 = vsplat(w0), W1 = vsplat(w1);
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        if constexpr (AR == AR_KAHAN) {
+                            const f2x y = vfma(W1, x1[k], vfma(W0, x0[k], er[k]));
+                            const f2x t = vadd(sm[k], y);
+                            er[k] = vsub(y, vsub(t, sm[k]));
+                            sm[k] = t;
+                        } else {
+                            sm[k] = vfma(W1, x1[k], vfma(W0, x0[k], sm[k]));
+                        }
+                    }
+                };
+                int uu = 0;
+                if constexpr (UV > 1) {
+                    for (; uu + UV <= nvc; uu += UV) {
+                        f2x x[UV][KC][4];
+                        float l[UV][KC];
+#pragma unroll
+                        for (int i = 0; i < UV; ++i) {
+                            const typename Table::E ent = te[(uu + i) * TP + pl];
+#pragma unroll
+                            for (int kb = 0; kb < KC; ++kb) {
+                                load8x(w + ent.off + kb * Pp, x[i][kb]);
+                                l[i][kb] = ent.w[kb];
+                            }
+                        }
+#pragma unroll
+                        for (int i = 0; i < UV; ++i)
+#pragma unroll
+                            for (int kb = 0; kb < KC; kb += 2) add(l[i][kb], x[i][kb], l[i][kb + 1], x[i][kb + 1]);
+                    }
+                }
+                for (; uu < nvc; ++uu) {
                     const typename Table::E ent = te[uu * TP + pl];
                     const float *row = w + ent.off;
 #pragma unroll
@@ -259,19 +406,9 @@ __global__ void __launch_bounds__(256, FL & X8_Z3 ? 2 : UPDATE_X8_BLOCKS) update
                         f2x x0[4], x1[4];
                         load8x(row + kb * Pp, x0);
                         load8x(row + (kb + 1) * Pp, x1);
-                        const f2x W0 = vsplat(ent.w[kb]), W1 = vsplat(ent.w[kb + 1]);
-#pragma unroll
-                        for (int k = 0; k < 4; ++k) {
-                            if constexpr (AR == AR_KAHAN) {
-                                const f2x y = vfma(W1, x1[k], vfma(W0, x0[k], er[k]));
-                                const f2x t = vadd(sm[k], y);
-                                er[k] = vsub(y, vsub(t, sm[k]));
-                                sm[k] = t;
-                            } else {
-                                sm[k] = vfma(W1, x1[k], vfma(W0, x0[k], sm[k]));
-                            }
-                        }
+                        add(ent.w[kb], x0, ent.w[kb + 1], x1);
                     }
+                }
                 }
             }
             if (!active) continue;
@@ -376,18 +513,43 @@ pet_status build_bp_table(pet_geometry *g, cudaStream_t st)
     return PET_OK;
 }
 
-// Stacks in FP32 with uniform bins and no TOF run the packed kernel.
-bool update_x8_path(const GeoDev &g, int arith)
+// Stacks in FP32 with uniform bins run the packed kernel; TOF ones with the in-plane RDP prior.
+bool update_x8_path(const UpdateArgs &a, int arith)
 {
-    return g.G == 8 && arith != AR_FP64 && !g.table && g.T == 1;
+    return a.g.G == 8 && arith != AR_FP64 && !a.g.table && (a.g.T == 1 || (!a.z3 && !a.tv));
+}
+
+// pixel tiles of the packed kernel
+int update_x8_tiles(const UpdateArgs &a)
+{
+    const int N = a.g.N;
+    if (a.g.T > 1) {
+        const X8Patch p = a.g.K <= 2 ? x8_patch<2>(a.g) : x8_patch<4>(a.g);
+        return (N + p.tx - 1) / p.tx * ((N + p.ty - 1) / p.ty);
+    }
+    const int TP = 256 / a.g.NG;
+    return (N * N + TP - 1) / TP;
+}
+
+// Views loaded together (see update_kernel_x8): 256 x 256 x 89 has 3121 tiles, 6.8 per block of 456
+// (3 blocks per SM) and 10.3 of 304: 7 and 11 rounds, and one view is 1.4 us of 66 faster; 128 x
+// 128 x 64 has 512, where one view took 503 us an iteration and four 438.  A batched launch (N = 0
+// here) takes four.
+static int x8_views(const UpdateArgs &a)
+{
+    if (a.g.N == 0 || a.z3 || a.tv || a.vox || a.g.T > 1) return 4;
+    const double nt = update_x8_tiles(a), s3 = 3.0 * sm_count(), s2 = 2.0 * sm_count();
+    return 1.026 * ceil(nt / s3) * s3 < ceil(nt / s2) * s2 ? 1 : 4;
 }
 
 template <int KC, int AR>
 static auto x8_fn(const UpdateArgs &a) -> void (*)(const UpdateArgs, const Batch)
 {
+    if (a.g.T > 1) return a.vox ? update_kernel_x8<KC, AR, X8_TOF | X8_VOX> : update_kernel_x8<KC, AR, X8_TOF>;
     if (a.tv) return a.vox ? update_kernel_x8<KC, AR, X8_TV | X8_VOX> : update_kernel_x8<KC, AR, X8_TV>;
     if (a.z3) return a.vox ? update_kernel_x8<KC, AR, X8_Z3 | X8_VOX> : update_kernel_x8<KC, AR, X8_Z3>;
-    return a.vox ? update_kernel_x8<KC, AR, X8_VOX> : update_kernel_x8<KC, AR, 0>;
+    if (a.vox) return update_kernel_x8<KC, AR, X8_VOX>;
+    return x8_views(a) == 1 ? update_kernel_x8<KC, AR, 0, 1> : update_kernel_x8<KC, AR, 0>;
 }
 
 static auto x8_any(const UpdateArgs &a, int arith)
