@@ -246,14 +246,16 @@ __device__ __forceinline__ void p1_neighbour(const float *f, int N, int ix, int 
 }
 
 // The patches of one virtual block that fall to warp `wid`; returns this lane's sum of new pixels.
-template <int KC, int AR, bool SUB, int C>
+// CT: the lanes per pixel, or 0 for a.C (sub-ray bins: their entries are too much code to repeat).
+template <int KC, int AR, bool SUB, int CT>
 __device__ __forceinline__ float p1_patches(const UpdateArgs &a, P1View *vt, int vloc, int wid, int lane,
                                             float inv_mean_f, float mean_mu)
 {
     const GeoDev &g = a.g;
     const int N = g.N, NB = g.NB, npix = N * N, stride = NB + 2 * P1_PAD;
     const bool dyn = a.nu_mode == 1 || a.nu_mode == 2;
-    constexpr int PX = 32 / C, TX = C == 1 ? 8 : (C == 8 ? 2 : 4), TY = PX / TX;
+    const int C = CT ? CT : a.C;
+    const int PX = 32 / C, TX = C == 1 ? 8 : (C == 8 ? 2 : 4), TY = PX / TX;
     const int c = lane / PX, pl = lane - c * PX, py = pl / TX, px = pl - py * TX;
     const int ntx = (N + TX - 1) / TX, npatch = ntx * ((N + TY - 1) / TY);
     const float *w = reinterpret_cast<const float *>(a.w);
@@ -382,7 +384,7 @@ __device__ __forceinline__ float p1_patches(const UpdateArgs &a, P1View *vt, int
 // the sinogram needs no test per bin.  A virtual block is 8 warps x a.tpv patches; only its sum
 // ends in barriers.
 template <int KC, int AR, bool SUB>
-__global__ void __launch_bounds__(256, SUB ? 3 : 4) update_kernel_p1(const __grid_constant__ UpdateArgs one, const Batch bt)
+__global__ void __launch_bounds__(256, 4) update_kernel_p1(const __grid_constant__ UpdateArgs one, const Batch bt)
 {
     __shared__ __align__(16) P1View views[SUB ? 1 : 8][P1_VIEWS];
     __shared__ UpdateArgs sh_args;
@@ -411,7 +413,8 @@ __global__ void __launch_bounds__(256, SUB ? 3 : 4) update_kernel_p1(const __gri
         }
         float part = 0.f;
         P1View *vt = views[SUB ? 0 : wid];
-        switch (a.C) {
+        if constexpr (SUB) part = p1_patches<KC, AR, SUB, 0>(a, vt, vloc, wid, lane, inv_mean_f, mean_mu);
+        else switch (a.C) {
         case 1: part = p1_patches<KC, AR, SUB, 1>(a, vt, vloc, wid, lane, inv_mean_f, mean_mu); break;
         case 2: part = p1_patches<KC, AR, SUB, 2>(a, vt, vloc, wid, lane, inv_mean_f, mean_mu); break;
         case 4: part = p1_patches<KC, AR, SUB, 4>(a, vt, vloc, wid, lane, inv_mean_f, mean_mu); break;

@@ -208,7 +208,7 @@ __global__ void __launch_bounds__(256) tof_fwd_kernel(const __grid_constant__ Fw
 //   3. thread (ray, slice of TOF_TW bins, half-group) reads each pixel once (16 bytes) and adds it to
 //      its slice's sums, 8 pixels by FMAs and then one compensated step.
 // ------------------------------------------------------------------------------------------
-constexpr int TOF_TW = 7, TOF_WP = 8, TOF_THREADS = 256, TOF_HG = 24, TOF_STEPS = 32, TOF_BLOCK = 8;
+constexpr int TOF_TW = 7, TOF_WP = 8, TOF_THREADS = 256, TOF_HG = 24, TOF_STEPS = 32;
 
 // dynamic shared memory of a block at most, and of one ray: 2 TOF_STEPS entries of ts slices x 8
 // weight pairs, an offset, and (length, position)
@@ -357,39 +357,51 @@ __global__ void __launch_bounds__(TOF_THREADS, 2) tof_fwd_stack(const __grid_con
                 if (work) {
                     const int n = count[rl];
                     const f2x *we = wts + (rl * E * sh.ts + slice) * TOF_WP;
-                    for (int e0 = 0; e0 < n; e0 += TOF_BLOCK) {
-                        f2x bl[TOF_TW][2];
-#pragma unroll
-                        for (int t = 0; t < TOF_TW; ++t) bl[t][0] = bl[t][1] = 0ull;
-                        const int e1 = min(n, e0 + TOF_BLOCK);
-#pragma unroll 2
-                        for (int e = e0; e < e1; ++e) {
-                            f2x x0, x1;
-                            const float *px = img + off[rl * E + e];
-                            asm("ld.global.nc.v2.b64 {%0, %1}, [%2];" : "=l"(x0), "=l"(x1) : "l"(px));
-                            const ulonglong2 *wp = reinterpret_cast<const ulonglong2 *>(we + e * sh.ts * TOF_WP);
-                            const ulonglong2 w01 = wp[0], w23 = wp[1], w45 = wp[2];
-                            const f2x wv[TOF_TW] = {w01.x, w01.y, w23.x, w23.y, w45.x, w45.y, wp[3].x};
-#pragma unroll
-                            for (int t = 0; t < TOF_TW; ++t) {
-                                bl[t][0] = vfma(wv[t], x0, bl[t][0]);
-                                bl[t][1] = vfma(wv[t], x1, bl[t][1]);
-                            }
-                        }
+                    // eight pixels by FMAs onto the compensation term, then one compensated step
+                    auto merge = [&]() {
 #pragma unroll
                         for (int t = 0; t < TOF_TW; ++t)
 #pragma unroll
                             for (int q = 0; q < 2; ++q) {
                                 if constexpr (AR == AR_KAHAN) {
-                                    const f2x y = vadd(bl[t][q], er[t][q]);
-                                    const f2x s = vadd(sm[t][q], y);
-                                    er[t][q] = vsub(y, vsub(s, sm[t][q]));
+                                    const f2x s = vadd(sm[t][q], er[t][q]);
+                                    er[t][q] = vsub(er[t][q], vsub(s, sm[t][q]));
                                     sm[t][q] = s;
-                                } else {
-                                    sm[t][q] = vadd(sm[t][q], bl[t][q]);
                                 }
                             }
+                    };
+                    auto pixels = [&](auto number, int e) {
+                        constexpr int U = decltype(number)::value;
+                        f2x x0[U], x1[U];
+#pragma unroll
+                        for (int i = 0; i < U; ++i) {
+                            const float *px = img + off[rl * E + e + i];
+                            asm("ld.global.nc.v2.b64 {%0, %1}, [%2];" : "=l"(x0[i]), "=l"(x1[i]) : "l"(px));
+                        }
+#pragma unroll
+                        for (int i = 0; i < U; ++i) {
+                            const ulonglong2 *wp = reinterpret_cast<const ulonglong2 *>(we + (e + i) * sh.ts * TOF_WP);
+                            const ulonglong2 w01 = wp[0], w23 = wp[1], w45 = wp[2];
+                            const f2x wv[TOF_TW] = {w01.x, w01.y, w23.x, w23.y, w45.x, w45.y, wp[3].x};
+#pragma unroll
+                            for (int t = 0; t < TOF_TW; ++t) {
+                                if constexpr (AR == AR_KAHAN) {
+                                    er[t][0] = vfma(wv[t], x0[i], er[t][0]);
+                                    er[t][1] = vfma(wv[t], x1[i], er[t][1]);
+                                } else {
+                                    sm[t][0] = vfma(wv[t], x0[i], sm[t][0]);
+                                    sm[t][1] = vfma(wv[t], x1[i], sm[t][1]);
+                                }
+                            }
+                        }
+                    };
+                    int e = 0;
+                    for (; e + 4 <= n; e += 4) {
+                        pixels(std::integral_constant<int, 4>{}, e);
+                        if (e & 4) merge();
                     }
+                    for (; e < n; ++e) pixels(std::integral_constant<int, 1>{}, e);
+                    merge();
                 }
                 __syncthreads();                        // the lists are free again
             }

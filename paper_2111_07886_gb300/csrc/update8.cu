@@ -56,7 +56,8 @@ __device__ __forceinline__ void tof_entry(const GeoDev &g, int slot0, int u, int
     }
 }
 
-// Adds an entry's rows [bin][T] to a thread's sums: four TOF bins by FMAs, then one compensated step.
+// Adds an entry's rows [bin][T] to a thread's sums: four TOF bins by FMAs onto the compensation term,
+// then one compensated step.
 template <int KC, int AR>
 __device__ __forceinline__ void tof_gather(const GeoDev &g, const float *w, const float *ent, f2x (&sm)[4], f2x (&er)[4])
 {
@@ -67,35 +68,44 @@ __device__ __forceinline__ void tof_gather(const GeoDev &g, const float *w, cons
     for (int k = 0; k < KC; ++k) l[k] = ent[2 + k];
     const float *h = ent + (KC <= 2 ? 4 : 8);
     const float *row = w + (__float_as_uint(ent[0]) * TT + (unsigned)(tn & 255) * Pp);
-    for (int t0 = 0; t0 < n; t0 += 4) {
-        f2x bl[4];
+    auto merge = [&]() {
+        if constexpr (AR == AR_KAHAN) {
 #pragma unroll
-        for (int k = 0; k < 4; ++k) bl[k] = 0ull;
-#pragma unroll 2
-        for (int t = t0; t < min(n, t0 + 4); ++t) {
-            const float ht = h[t];
+            for (int k = 0; k < 4; ++k) {
+                const f2x s = vadd(sm[k], er[k]);
+                er[k] = vsub(er[k], vsub(s, sm[k]));
+                sm[k] = s;
+            }
+        }
+    };
+    auto bins = [&](auto count, int t) {
+        constexpr int U = decltype(count)::value;
+        f2x x[U][KC][4];
+#pragma unroll
+        for (int i = 0; i < U; ++i)
+#pragma unroll
+            for (int kb = 0; kb < KC; ++kb) load8x(row + ((unsigned)kb * TT + (unsigned)i) * Pp, x[i][kb]);
+#pragma unroll
+        for (int i = 0; i < U; ++i)
 #pragma unroll
             for (int kb = 0; kb < KC; ++kb) {
-                f2x x[4];
-                load8x(row + (unsigned)kb * TT * Pp, x);
-                const f2x W = vsplat(ht * l[kb]);
+                const f2x W = vsplat(h[t + i] * l[kb]);
 #pragma unroll
-                for (int k = 0; k < 4; ++k) bl[k] = vfma(W, x[k], bl[k]);
+                for (int k = 0; k < 4; ++k) {
+                    if constexpr (AR == AR_KAHAN) er[k] = vfma(W, x[i][kb][k], er[k]);
+                    else sm[k] = vfma(W, x[i][kb][k], sm[k]);
+                }
             }
-            row += Pp;
-        }
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            if constexpr (AR == AR_KAHAN) {
-                const f2x y = vadd(bl[k], er[k]);
-                const f2x s = vadd(sm[k], y);
-                er[k] = vsub(y, vsub(s, sm[k]));
-                sm[k] = s;
-            } else {
-                sm[k] = vadd(sm[k], bl[k]);
-            }
-        }
+        row += U * Pp;
+    };
+    constexpr int U = KC <= 2 ? 4 : 2;               // TOF bins whose rows are loaded together
+    int t = 0;
+    for (; t + U <= n; t += U) {
+        bins(std::integral_constant<int, U>{}, t);
+        if (U == 4 || (t & 2)) merge();
     }
+    for (; t < n; ++t) bins(std::integral_constant<int, 1>{}, t);
+    merge();
 }
 
 // FP32 update for 8-plane groups held as four f32x2 pairs.  Same step as update_kernel, with:
