@@ -517,7 +517,9 @@ static const void *update_p1_fn(const GeoDev &g)
     return g.K <= 2 ? (const void *)update_kernel_p1<2, AR, false> : (const void *)update_kernel_p1<4, AR, false>;
 }
 
-// Lanes per pixel C: the fewest that give 16 warps per SM, at least two views each.
+// Lanes per pixel C: the fewest that give 8 warps per SM (16 for sub-ray bins, whose entries are about
+// ten times the work), at least two views each.  24 mixed 2-D scans: 67.8 ms with 8 warps, 72.8 with
+// 16; an iteration of the 256 x 256 ring scan with 32 rays per bin: 1.53 and 1.17 ms.
 void update_shape_p1(UpdateArgs &a, int arith)
 {
     const int N = a.g.N;
@@ -526,7 +528,7 @@ void update_shape_p1(UpdateArgs &a, int arith)
         return (N + TX - 1) / TX * ((N + TY - 1) / TY);
     };
     int C = 1;
-    while (C < 8 && patches(C) < 16 * sm_count() && a.nviews >= 4 * C) C *= 2;
+    while (C < 8 && patches(C) < (a.g.table ? 16 : 8) * sm_count() && a.nviews >= 4 * C) C *= 2;
     a.C = C;
     const int slots = sm_count() * resident_blocks(arith == AR_KAHAN ? update_p1_fn<AR_KAHAN>(a.g) : update_p1_fn<AR_FP32>(a.g));
     const int nt = (patches(C) + 7) / 8;

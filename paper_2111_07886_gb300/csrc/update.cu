@@ -447,9 +447,12 @@ static void back_dispatch(const BackArgs &a, int arith, int grid, cudaStream_t s
         else back_kernel<G, 4, AR_FP64, true><<<grid, 256, 0, st>>>(a);
         return;
     }
-    if (arith == AR_FP32) back_kernel<G, KC, AR_FP32><<<grid, 256, 0, st>>>(a);
-    else if (arith == AR_KAHAN) back_kernel<G, KC, AR_KAHAN><<<grid, 256, 0, st>>>(a);
-    else back_kernel<G, KC, AR_FP64><<<grid, 256, 0, st>>>(a);
+    // (FP32 stacks of at most two candidate bins run back_quad_kernel)
+    if constexpr (G == 1 || KC > 2) {
+        if (arith == AR_FP32) { back_kernel<G, KC, AR_FP32><<<grid, 256, 0, st>>>(a); return; }
+        if (arith == AR_KAHAN) { back_kernel<G, KC, AR_KAHAN><<<grid, 256, 0, st>>>(a); return; }
+    }
+    back_kernel<G, KC, AR_FP64><<<grid, 256, 0, st>>>(a);
 }
 
 pet_status launch_back(const BackArgs &a, int arith, cudaStream_t st)
