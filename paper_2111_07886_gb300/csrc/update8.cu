@@ -43,7 +43,7 @@ __device__ __forceinline__ void tof_entry(const GeoDev &g, int slot0, int u, int
     const int t_lo = max(0, (int)ceilf(tc - W / d)), t_hi = min(g.T - 1, (int)floorf(tc + W / d));
     const int n = min(in ? max(0, t_hi - t_lo + 1) : 0, g.tof_hw);
     out[0] = __uint_as_float(ent.off);
-    out[1] = __int_as_float(t_lo | n << 8);
+    out[1] = __int_as_float(n > 0 ? t_lo | n << 8 : 0);      // t_lo < T <= 64 when n > 0
 #pragma unroll
     for (int k = 0; k < KC; ++k) out[2 + k] = ent.w[k];
     float *h = out + (KC <= 2 ? 4 : 8);

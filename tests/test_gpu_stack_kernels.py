@@ -47,7 +47,9 @@ def test_tv_steps(N, P, iters):
 # (N, P, T, TOF bin mm, FWHM mm, rho): planes on both sides of the stack kernel's bound, one to three
 # slices of TOF bins, windows narrower and wider than the field, three candidate bins
 TOF = [(40, 41, 13, 20.0, 30.0, 1.0), (33, 57, 21, 9.0, 12.0, 1.0), (24, 48, 7, 60.0, 80.0, 0.6),
-       (30, 17, 15, 12.0, 25.0, 1.0), (28, 43, 5, 8.0, 10.0, 1.0)]
+       (30, 17, 15, 12.0, 25.0, 1.0), (28, 43, 5, 8.0, 10.0, 1.0),
+       # TOF bins so short that the field spans hundreds of them: many pixels lie outside all windows
+       (80, 9, 64, 0.8, 12.0, 1.0)]
 
 
 @pytest.mark.parametrize("geom", TOF)
