@@ -166,7 +166,6 @@ static pet_status build_tables(pet_geometry *g, std::vector<ViewGeo> &views,
         vg.hq = to_q32(vg.h);
         vg.axis = minor == 0.0 ? 1 : 0;
         vg.wslope = minor > 0.0 ? rho / (major * minor) : 0.0;
-        vg.hf = (float)vg.h;
         vg.wslopef = (float)vg.wslope;
         vg.wslopel = (float)(vg.wslope - (double)vg.wslopef);
         // forward walk: cross coordinate (grid units) at the start of driving step 0

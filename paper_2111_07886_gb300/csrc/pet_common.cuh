@@ -72,8 +72,7 @@ struct ViewGeo {
     long long t0q, cxq, cyq, hq;   // t(ix,iy) = t0 + ix cx + iy cy; half-width h; Q32.32
     double t0, cx, cy, h;
     double wslope;        // length per bin unit of (h - |delta|): rho / (major * minor)
-    float hf;             // h
-    float wslopef, wslopel;   // (and wslope - wslopef)
+    float wslopef, wslopel;   // wslope, and wslope - wslopef
     int axis;             // minor == 0: half-open rule, length L for delta in [-h, h)
     // sub-ray model: cross-coordinate shift of half a sub-ray spacing (rho / (2 R a), a the
     // driving component of the view's direction), grid units; sub-ray s of a bin starts

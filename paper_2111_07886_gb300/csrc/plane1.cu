@@ -28,7 +28,8 @@ bool plane1_path(const GeoDev &g, int arith) { return g.G == 1 && arith != AR_FP
 constexpr int P1_PAD = 4;           // zero bins on both sides of a row of w (see update_kernel_p1)
 int plane1_pad() { return P1_PAD; }
 
-constexpr int P1_MAX_CHUNKS = 32;   // most threads sharing one ray (built-in chunking)
+// Bins whose lines are summed in closed form (kernels.cuh)
+static __host__ __device__ __forceinline__ bool closed_sums(const GeoDev &g) { return g.table && g.R >= SUB_CLOSED_MIN; }
 
 // One compensated (Kahan) or plain step of a running sum.
 template <int AR>
@@ -44,37 +45,54 @@ __device__ __forceinline__ void p1_add(float y, float &s, float &e)
     }
 }
 
+// The same for w0 x0 + w1 x1: one driving step of a ray, or two bins of a (pixel, view) entry.
+template <int AR>
+__device__ __forceinline__ void p1_add2(float w0, float x0, float w1, float x1, float &s, float &e)
+{
+    if constexpr (AR == AR_KAHAN) {
+        const float y = fmaf(w1, x1, fmaf(w0, x0, e)), t = s + y;
+        e = y - (t - s);
+        s = t;
+    } else {
+        s = fmaf(w1, x1, fmaf(w0, x0, s));
+    }
+}
+
 // `steps` driving steps of one line from cross coordinate lo (Q32.32), reading rows of stride N from
-// img + base; four steps at a time (their loads are issued together), each block of four added with
-// one compensated step.  A step rises by ast < 1 pixel, so the carry of the 32-bit fractions says
-// whether it crosses into the next pixel; ast = 1 (45 degrees) is taken as 1 - 2^-32.
+// img + base; the loads of four steps are issued together, and every step is one compensated step of
+// the sum.  The carry of the 32-bit fractions says whether a step crosses into the next pixel (a
+// step rises by at most one pixel, and by exactly one only at 45 degrees, where all do).
 template <int AR>
 __device__ __forceinline__ void p1_walk(const float *__restrict__ img, unsigned N, unsigned base, long long lo,
                                         long long stp, long long ast, float L, float im, int steps, float &s,
                                         float &e)
 {
-    const unsigned rise = ast > 0xFFFFFFFFLL ? 0xFFFFFFFFu : (unsigned)ast;
-    auto step = [&](float &bl) {
+    const unsigned rise = (unsigned)ast;
+    const bool all = (ast >> 32) != 0;
+    auto step = [&](float &l0, float &x0, float &l1, float &x1) {
         const unsigned r = (unsigned)(int)(lo >> 32), fr = (unsigned)lo, up = fr + rise;
-        const bool cross = up < fr;
-        const float l1 = cross ? __uint2float_rn(up) * im : 0.f;
+        const bool cross = all || up < fr;
+        l1 = cross ? __uint2float_rn(up) * im : 0.f;
+        l0 = L - l1;
         const float *q = img + (int)(base + r);     // r may be -1
-        float x0 = 0.f, x1 = 0.f;
+        x0 = x1 = 0.f;
         if (r < N) x0 = __ldg(q);
         if (cross && r + 1u < N) x1 = __ldg(q + 1);
-        bl = fmaf(l1, x1, fmaf(L - l1, x0, bl));
         lo += stp;
         base += N;
     };
     for (; steps >= 4; steps -= 4) {
-        float bl = 0.f;
+        float l0[4], x0[4], l1[4], x1[4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) step(bl);
-        p1_add<AR>(bl, s, e);
+        for (int j = 0; j < 4; ++j) step(l0[j], x0[j], l1[j], x1[j]);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) p1_add2<AR>(l0[j], x0[j], l1[j], x1[j], s, e);
     }
-    float bl = 0.f;
-    for (; steps > 0; --steps) step(bl);
-    p1_add<AR>(bl, s, e);
+    for (; steps > 0; --steps) {
+        float l0, x0, l1, x1;
+        step(l0, x0, l1, x1);
+        p1_add2<AR>(l0, x0, l1, x1, s, e);
+    }
 }
 
 // Thread layout: 256 threads = S chunks x R rays (thread = chunk * R + ray), rays in view order so
@@ -118,7 +136,7 @@ __device__ __forceinline__ void fwd_p1_vblock(const FwdArgs &a, int vloc, float 
             const long long lo = rg.loq + (long long)k0 * stp;
             if constexpr (SUB) {
                 const int nsr = g.R;
-                if (nsr >= SUB_CLOSED_MIN && !vw.axis && (long long)nsr * (rg.shq < 0 ? -rg.shq : rg.shq) < SUB_CLOSED_SPAN) {
+                if (nsr >= SUB_CLOSED_MIN && !vw.axis && 2ll * nsr * (rg.shq < 0 ? -rg.shq : rg.shq) < SUB_CLOSED_SPAN) {
                     const LineFan fan = line_fan(nsr, rg.shq, ast, vw.inv_minorf, vw.inv_minorl);
                     long long b = lo - (long long)(nsr - 1) * (rg.shq < 0 ? -rg.shq : rg.shq);
                     unsigned row = base;
@@ -152,18 +170,28 @@ __device__ __forceinline__ void fwd_p1_vblock(const FwdArgs &a, int vloc, float 
             comb_e[threadIdx.x] = e;
             __syncthreads();
             if (live && c == 0)
-                for (int cc = 1; cc < S; ++cc) p1_add<AR>(comb_s[cc * R + rl] + comb_e[cc * R + rl], s, e);
+                for (int cc = 1; cc < S; ++cc) {
+                    if constexpr (AR == AR_KAHAN) e += comb_e[cc * R + rl];
+                    p1_add<AR>(comb_s[cc * R + rl], s, e);
+                }
         }
         if (live && c == 0) {
             const float tot = s + e, scale = (float)g.scale;
             if constexpr (MODE == FWD_PLAIN) {
-                reinterpret_cast<float *>(a.out)[ray] = scale * tot;
+                reinterpret_cast<float *>(a.out)[ray] = SUB && closed_sums(g) ? fmaf(scale, s, scale * e) : scale * tot;
             } else {
                 const float af = scale * (tot * m);
                 if constexpr (MODE == FWD_RATIO) {
                     const int u = ray / NB, b = ray - u * NB;
                     float *out = reinterpret_cast<float *>(a.out) + (size_t)u * (NB + 2 * a.pad) + a.pad;
-                    out[b] = m * (1.f - (float)cnt / (af + gam));
+                    float y = af + gam;
+                    if (SUB && closed_sums(g)) {
+                        // scale m (s + e) + gamma with the rounding of the result only (the closed sums
+                        // are exact to that): sm + sml is scale m
+                        const float sm = scale * m, sml = fmaf(scale, m, -sm);
+                        y = fmaf(sm, s, fmaf(sm, e, fmaf(sml, s, gam)));
+                    }
+                    out[b] = m * (1.f - (float)cnt / y);
                     // the zero bins on both sides of the row (see update_kernel_p1)
                     if (b == 0)
                         for (int q = 1; q <= a.pad; ++q) out[-q] = 0.f;
@@ -217,32 +245,49 @@ __global__ void __launch_bounds__(256, 4) fwd_mu_kernel_p1(const __grid_constant
     else mu_p1_vblock(mu, vb - nfwd, mu.nvb);
 }
 
-// What a patch's (pixel, view) entries need of a view: x = t - h at the patch's first pixel relative
-// to bin `bin`, and its slopes, in Q6.26 (a patch spans less than 32 bins: at most 10 pixel steps
-// of at most 1 / 0.36 bins); the row's first bin in w; the trapezoid (0 for views along an axis).
+// What a patch's (pixel, view) entries need of a view: t - h at the patch's first pixel, its slopes
+// and 2 h (Q32.32 bins), the row's first bin in w, and the trapezoid.
 struct __align__(16) P1View {
-    int x, cx, cy, bin;
+    long long x, cx, cy, h2;
     unsigned row;
-    float h2, ws, L;           // 2 h, length per bin unit, L
+    float ws, L;               // length per 2^-24 bin, L
+    int axis;
 };
 constexpr int P1_VIEWS = 32;   // views of the subset a warp holds at a time
 
-// One of the 8 neighbours of pixel (ix, iy): the RDP gradient term (without its factor 2), and the
-// part in the Matlab-style gradient (q < 4: the axial ones; a missing one counts as the centre).
+// Neighbour q of pixel (ix, iy), row by row without the centre: numerator and 1 / denominator of the
+// RDP gradient term (without its factor 2), and the part in the Matlab-style gradient (a missing axial
+// neighbour counts as the centre).
 __device__ __forceinline__ void p1_neighbour(const float *f, int N, int ix, int iy, int q, float fc, float gamma_r,
-                                             float eps, float &gr, float &gx, float &gy)
+                                             float eps, float &num, float &rden, float &gx, float &gy)
 {
-    const int dx = q < 4 ? (q < 2 ? 2 * q - 1 : 0) : 2 * (q & 1) - 1;
-    const int dy = q < 4 ? (q < 2 ? 0 : 2 * q - 5) : (q & 2) - 1;
+    const int r = q < 4 ? q : q + 1, dy = r / 3 - 1, dx = r - 3 * (dy + 1) - 1;
     const int x = ix + dx, y = iy + dy;
     float fk = fc;
+    num = rden = 0.f;
     if ((unsigned)x < (unsigned)N && (unsigned)y < (unsigned)N) {
         fk = __ldg(f + y * N + x);
         const float d = fc - fk, ad = fabsf(d), den = fc + fk + gamma_r * ad + eps;
-        gr += __fdividef(d * (gamma_r * ad + fc + 3.f * fk + 2.f * eps), den * den);
+        num = d * (gamma_r * ad + fc + 3.f * fk + 2.f * eps);
+        rden = __fdividef(1.f, den * den);
     }
-    if (q < 2) gx += (float)dx * fk;
-    else if (q < 4) gy += (float)dy * fk;
+    if (dy == 0) gx += (float)dx * fk;
+    else if (dx == 0) gy += (float)dy * fk;
+}
+
+// The KC lengths and row values of pixel (ix, iy) and view u of the subset: sub-ray bins, and views
+// along an axis (membership from the forward walk's own coordinates).
+template <int KC, int AR, bool SUB>
+__device__ __forceinline__ void p1_any_entry(const UpdateArgs &a, int u, int ix, int iy, float (&l)[KC], float (&x)[KC])
+{
+    const GeoDev &g = a.g;
+    const auto ent = bp_entry<KC, AR, 0, SUB>(g, a.slot0 + u, 0, true, ix, iy);
+    const float *row = reinterpret_cast<const float *>(a.w) + (size_t)u * (g.NB + 2 * P1_PAD) + P1_PAD + ent.off;
+#pragma unroll
+    for (int k = 0; k < KC; ++k) {
+        l[k] = ent.w[k];
+        x[k] = __ldg(row + k);
+    }
 }
 
 // The patches of one virtual block that fall to warp `wid`; returns this lane's sum of new pixels.
@@ -268,87 +313,101 @@ __device__ __forceinline__ float p1_patches(const UpdateArgs &a, P1View *vt, int
         const int x0 = (patch % ntx) * TX, y0 = (patch / ntx) * TY;
         const int ix = x0 + px, iy = y0 + py, j = iy * N + ix;
         const bool active = ix < N && iy < N;
-        // stencil
+        // stencil: each lane takes the neighbours c, c + C, ..., and the terms are added in row order
         float fc = 0.f, gr = 0.f, gx = 0.f, gy = 0.f;
-        if (active) {
-            fc = __ldg(f + j);
+        if (active) fc = __ldg(f + j);
 #pragma unroll
-            for (int q8 = 0; q8 < 8 / C; ++q8) {
-                const int q = q8 * C + c;
-                p1_neighbour(f, N, ix, iy, q, fc, a.fs_gamma_r, a.fs_eps, gr, gx, gy);
+        for (int q8 = 0; q8 < 8 / C; ++q8) {
+            float num = 0.f, rden = 0.f;
+            if (active) p1_neighbour(f, N, ix, iy, q8 * C + c, fc, a.fs_gamma_r, a.fs_eps, num, rden, gx, gy);
+#pragma unroll
+            for (int cc = 0; cc < C; ++cc) {
+                const float n1 = C == 1 ? num : __shfl_sync(0xffffffffu, num, cc * PX + pl);
+                const float r1 = C == 1 ? rden : __shfl_sync(0xffffffffu, rden, cc * PX + pl);
+                gr = fmaf(n1, r1, gr);
             }
         }
 #pragma unroll
         for (int o = PX; o < 32; o *= 2) {
-            gr += __shfl_xor_sync(0xffffffffu, gr, o);
             gx += __shfl_xor_sync(0xffffffffu, gx, o);
             gy += __shfl_xor_sync(0xffffffffu, gy, o);
         }
-        // gather
+        // gather: chunk c sets up the entries of the views c, c + C, ...; every lane of the pixel adds
+        // them in view order, two bins per compensated step, whatever C is
         float s = 0.f, e = 0.f;
-        // the general entry: sub-ray bins, and views along an axis (membership from the forward
-        // walk's own coordinates)
-        auto any_view = [&](int u) {
-            int b0;
-            float wk[KC];
-            bp_weights<KC, AR, SUB>(g, g.views[a.slot0 + u], a.slot0 + u, ix, iy, b0, wk);
-            const float *row = w + (size_t)u * stride + P1_PAD;
-            float y = 0.f;
+        auto add = [&](const float (&l)[KC], const float (&x)[KC], int views) {
+            if (C == 1) {
 #pragma unroll
-            for (int q = 0; q < KC; ++q) y = fmaf(wk[q], __ldg(row + min(max(b0 + q, 0), NB - 1)), y);
-            p1_add<AR>(y, s, e);
+                for (int q = 0; q < KC; q += 2) p1_add2<AR>(l[q], x[q], l[q + 1], x[q + 1], s, e);
+            } else {
+#pragma unroll
+                for (int cc = 0; cc < C; ++cc) {
+                    if (cc >= views) break;
+#pragma unroll
+                    for (int q = 0; q < KC; q += 2) {
+                        const int from = cc * PX + pl;
+                        p1_add2<AR>(__shfl_sync(0xffffffffu, l[q], from), __shfl_sync(0xffffffffu, x[q], from),
+                                    __shfl_sync(0xffffffffu, l[q + 1], from), __shfl_sync(0xffffffffu, x[q + 1], from), s, e);
+                    }
+                }
+            }
         };
         if constexpr (SUB) {
-            if (active)
-                for (int u = c; u < a.nviews; u += C) any_view(u);
+            for (int u0 = 0; u0 < a.nviews; u0 += C) {
+                float l[KC] = {}, x[KC] = {};
+                if (active && u0 + c < a.nviews) p1_any_entry<KC, AR, SUB>(a, u0 + c, ix, iy, l, x);
+                add(l, x, a.nviews - u0);
+            }
         } else {
             for (int u0 = 0; u0 < a.nviews; u0 += P1_VIEWS) {
                 const int nvc = min(P1_VIEWS, a.nviews - u0);
-                bool axis = false;
                 __syncwarp();
                 if (lane < nvc) {
                     const ViewGeo &vw = g.views[a.slot0 + u0 + lane];
-                    const long long xq = vw.t0q - vw.hq + (long long)x0 * vw.cxq + (long long)y0 * vw.cyq;
-                    axis = vw.axis;
                     P1View v;
-                    v.bin = (int)(xq >> 32);
-                    v.x = (int)(((unsigned)xq >> 6) + (((unsigned)xq >> 5) & 1u));
-                    v.cx = (int)((vw.cxq + 32) >> 6);
-                    v.cy = (int)((vw.cyq + 32) >> 6);
+                    v.x = vw.t0q - vw.hq + (long long)x0 * vw.cxq + (long long)y0 * vw.cyq;
+                    v.cx = vw.cxq;
+                    v.cy = vw.cyq;
+                    v.h2 = 2 * vw.hq;
                     v.row = (unsigned)(u0 + lane) * (unsigned)stride + P1_PAD;
-                    v.h2 = 2.f * vw.hf;
-                    v.ws = axis ? 0.f : vw.wslopef;
-                    v.L = axis ? 0.f : vw.Lf;
+                    v.ws = vw.wslopef * (kQ32 * 256.f);
+                    v.L = vw.Lf;
+                    v.axis = vw.axis;
                     vt[lane] = v;
                 }
-                const unsigned axes = __ballot_sync(0xffffffffu, axis);
                 __syncwarp();
-                if (!active) continue;
 #pragma unroll 4
-                for (int u = c; u < nvc; u += C) {
-                    const P1View v = vt[u];
-                    const int x = v.x + px * v.cx + py * v.cy;
-                    const int up = (x + 0x3FFFFFF) >> 26;                            // ceil
-                    const float e0 = (float)((up << 26) - x) * 1.4901161193847656e-8f;   // b0 - (t - h)
-                    const int b0 = min(max(v.bin + up, -P1_PAD), NB + P1_PAD - KC);
-                    const float *row = w + (v.row + (unsigned)b0);
-                    float y = fminf(v.L, fmaxf(0.f, fminf(e0, v.h2 - e0)) * v.ws) * __ldg(row);
+                for (int r = 0; r < nvc; r += C) {
+                    float l[KC] = {}, x[KC] = {};
+                    const int u = r + c;
+                    if (u < nvc) {
+                        const P1View v = vt[u];
+                        if (!v.axis) {
+                            // the entry of bp_weights, bit by bit: with d = b0 - (t - h) in [0, 1) the
+                            // distance of bin b0 + q from the nearer foot of the trapezoid is
+                            // min(d + q, 2 h - d - q), taken in 2^-24 bins
+                            const long long t = v.x + px * v.cx + py * v.cy;
+                            const unsigned lo = (unsigned)t, d = 0u - lo;
+                            const int up = (int)(t >> 32) + (lo != 0u);                     // ceil
+                            const int rising = (int)(d >> 8), falling = (int)((v.h2 - (long long)d) >> 8);
+                            const int b0 = min(max(up, -P1_PAD), NB + P1_PAD - KC);
+                            const float *row = w + (v.row + (unsigned)b0);
 #pragma unroll
-                    for (int q = 1; q < KC; ++q) {
-                        // KC = 2 holds geometries with 2 h < 2: the rising side ends before bin 1
-                        const float r = v.h2 - (e0 + (float)q), d = KC == 2 ? r : fminf(e0 + (float)q, r);
-                        y = fmaf(fminf(v.L, fmaxf(0.f, d) * v.ws), __ldg(row + q), y);
+                            for (int q = 0; q < KC; ++q) {
+                                // KC = 2 holds geometries with 2 h < 2: the rising side ends before bin 1
+                                const int fall = falling - (q << 24);
+                                const int dd = KC == 2 && q == 1 ? fall : min(rising + (q << 24), fall);
+                                l[q] = fminf(v.L, __int2float_rn(max(0, dd)) * v.ws);
+                                x[q] = __ldg(row + q);
+                            }
+                        } else if (active) {
+                            p1_any_entry<KC, AR, false>(a, u0 + u, ix, iy, l, x);
+                        }
                     }
-                    p1_add<AR>(y, s, e);
+                    add(l, x, nvc - r);
                 }
-                if (axes)
-                    for (int u = c; u < nvc; u += C)
-                        if (axes >> u & 1) any_view(u0 + u);
             }
         }
-        const float mine = s + e;
-#pragma unroll
-        for (int cc = 1; cc < C; ++cc) p1_add<AR>(__shfl_sync(0xffffffffu, mine, cc * PX + pl), s, e);
         // step
         if (c == 0 && active) {
             float nu = 1.f;
@@ -358,12 +417,16 @@ __device__ __forceinline__ float p1_patches(const UpdateArgs &a, P1View *vt, int
                 // central differences inside, one-sided at the border
                 gx *= ix > 0 && ix < N - 1 ? 0.5f : 1.f;
                 gy *= iy > 0 && iy < N - 1 ? 0.5f : 1.f;
-                nu = nu_of<float>(gx, gy, 0.f, inv_mean_f, mean_mu, a.fs_nu1, a.fs_nu2);
+                const float x2 = fmaf(gx, gx, __fmul_rn(gy, gy));
+                float mu = (x2 > 0.f ? x2 * rsqrtf(x2) : 0.f) * inv_mean_f;
+                mu = mu < 0.01f ? 0.01f : mu;
+                nu = clampT<float>(fast_div(mean_mu, mu), a.fs_nu1, a.fs_nu2);
                 if (a.nu_mode == 2) reinterpret_cast<float *>(a.nu_frozen)[j] = nu;
             }
             const float ip = __ldg(reinterpret_cast<const float *>(a.invp) + j) * a.fs_ips;
             const float coef = a.fs_lam * nu * ((fc < 0.5f * U ? fc : U - fc) * ip);
-            float ft = fc - coef * (scale * (s + e) + a.fs_bm * (2.f * gr));
+            const float rg = __fmul_rn(a.fs_bm, 2.f * gr);
+            float ft = fmaf(-coef, SUB && closed_sums(g) ? fmaf(scale, s, fmaf(scale, e, rg)) : fmaf(scale, s + e, rg), fc);
             ft = ft <= 0.f ? tt : (ft >= U ? U - tt : ft);
             part += ft;
             reinterpret_cast<float *>(a.fout)[j] = ft;
@@ -376,13 +439,14 @@ __device__ __forceinline__ float p1_patches(const UpdateArgs &a, P1View *vt, int
 // f^{k,i} = P_t(f - lambda_k alpha_{k,i} nu S(f) (A_i^T w + (beta/M) grad R(f))) for one plane.
 // A warp works alone, without block barriers: it takes a patch of 32 / C pixels (8 x 4, 4 x 4,
 // 4 x 2 or 2 x 2, so that one view's bins are a few sectors of the row of w) with C lanes per
-// pixel, lane = chunk * (32 / C) + pixel.  Its lanes first set up one view each for the patch (the
-// 64-bit positions), then chunk c takes the neighbours and gathers the views c, c + C, ... with one
-// compensated step per view; the chunks are added in order through shuffles.  Candidate bins
-// b0 + k of a view: with e = b0 - (t - h) in [0, 1) the length is min(L, ws min(e + k, 2 h - e - k))
-// where positive; rows of w carry P1_PAD zero bins on both sides, so that an entry at the edge of
-// the sinogram needs no test per bin.  A virtual block is 8 warps x a.tpv patches; only its sum
-// ends in barriers.
+// pixel, lane = chunk * (32 / C) + pixel.  Its lanes first set up one view each for the patch, then
+// chunk c sets up the neighbours and the (pixel, view) entries c, c + C, ...; their terms go through
+// shuffles and are added in the order of the rows and views, so that the result has the same bits for
+// every C, those of one thread per pixel (sums of the chunks, each rounded, and positions in 2^-26
+// bins cost up to 1.9 times the error against 64 bits in batches of scans that amplify rounding; the
+// exact order costs 24 mixed scans x 10 iterations 68.2 ms instead of 67.8).
+// Rows of w carry P1_PAD zero bins on both sides: an entry at the edge of the sinogram needs no test
+// per bin.  A virtual block is 8 warps x a.tpv patches; only its sum ends in barriers.
 template <int KC, int AR, bool SUB>
 __global__ void __launch_bounds__(256, 4) update_kernel_p1(const __grid_constant__ UpdateArgs one, const Batch bt)
 {
@@ -454,16 +518,19 @@ static const void *fwd_p1_fn(int mode, int sub)
                                : (const void *)fwd_kernel_p1<AR, FWD_OBJECTIVE, false>;
 }
 
-// Chunks per ray: enough threads for one wave of 2048 per SM, at least 16 driving steps each (8 for
-// sub-ray bins, whose steps are about ten times the work).
+// Chunks per ray as for stacks (forward_shape): one wave of 2048 threads per SM where the rays allow it,
+// at most 16 of at least 16 driving steps each.  A step of closed sums is about ten times the work of a
+// line's, so there up to 32 chunks of 8 steps (the 256 x 256 ring scan with 32 rays per bin: an iteration
+// takes 1.50 ms with 16 chunks and 1.30 with 32).
 void forward_shape_p1(FwdArgs &a, int mode, int arith)
 {
-    const long long nrays = (long long)a.nviews * a.g.NB;
+    const bool closed = closed_sums(a.g);
+    const long long nrays = std::max(1LL, (long long)a.nviews * a.g.NB);
     const long long want = (long long)sm_count() * 2048;
-    const int least = a.g.table ? 8 : 16;
-    int S = 1;
-    while (S < P1_MAX_CHUNKS && nrays * S < want && a.g.N / (2 * S) >= least) S *= 2;
+    int S = (int)std::min<long long>(closed ? 32 : 16, (want + nrays - 1) / nrays);
+    S = std::max(1, std::min(S, a.g.N / (closed ? 8 : 16)));
     if (a.g.tuneS > 0 && mode != FWD_OBJECTIVE) S = a.g.tuneS;
+    while (256 % S) --S;
     a.S = S;
     a.R = 256 / S;
     const long long ntiles = (nrays + a.R - 1) / a.R;
