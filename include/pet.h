@@ -174,7 +174,8 @@ void pet_geometry_destroy(pet_geometry *g);
 
 /* Autotuner (no counterpart in the paper): times the forward projector of subset 0 for each
  * admissible number of ray chunks (threads sharing one ray) and keeps the fastest in the
- * geometry; *best_S (optional) receives it.  Tune before creating states on the geometry (the
+ * geometry; *best_S (optional) receives it (0: the built-in choice, where that lies outside the
+ * range of pet_set_ray_chunks and is the fastest).  Tune before creating states on the geometry (the
  * chunking changes the order of the ray sums, within rounding).  The projection is timed on an
  * image of ones, best of 7 runs of 4 launches after a warm-up (pet_autotune_batch: best of 5
  * single batched launches); a larger chunk count replaces a smaller one only when it is more

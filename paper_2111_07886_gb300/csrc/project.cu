@@ -575,15 +575,18 @@ static pet_status autotune_any(pet_geometry *g, int concurrent, cudaStream_t st,
     int bestS = 0;
     const int save = gd.tuneS;
     pet_status r = PET_OK;
-    for (int S = 1; S <= FWD_MAX_CHUNKS && r == PET_OK; ++S) {
-        if ((256 / gd.NG) % S) continue;
-        gd.tuneS = S;
+    for (int S = 1; S <= FWD_MAX_CHUNKS + 1 && r == PET_OK; ++S) {
+        // last candidate: the built-in choice, where it is outside the range
+        const bool built_in = S > FWD_MAX_CHUNKS;
+        if (!built_in && (256 / gd.NG) % S) continue;
+        gd.tuneS = built_in ? 0 : S;
         FwdArgs fa{};
         fa.g = gd;
         fa.slot0 = g->voff[0];
         fa.nviews = nv;
         fa.img = img;
         forward_shape(fa, FWD_PLAIN, AR_KAHAN);
+        if (built_in && fa.S <= FWD_MAX_CHUNKS) break;
         for (int c = 0; c < concurrent; ++c) {
             h_args[c] = fa;
             h_args[c].out = outs + (size_t)c * pb;
@@ -616,7 +619,7 @@ static pet_status autotune_any(pet_geometry *g, int concurrent, cudaStream_t st,
         }
         // a larger S must win by more than 3 %: timings that close are noise, and fewer chunks
         // leave more of the GPU to whatever runs beside the projection
-        if (r == PET_OK && tmin < best * 0.97f) { best = tmin; bestS = S; }
+        if (r == PET_OK && tmin < best * 0.97f) { best = tmin; bestS = gd.tuneS; }
     }
     cudaEventDestroy(a);
     cudaEventDestroy(b);
