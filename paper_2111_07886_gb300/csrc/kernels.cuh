@@ -194,6 +194,13 @@ __device__ __forceinline__ f2x vrcp(f2x a)
     asm("rcp.approx.ftz.f32 %0, %0;" : "+f"(y));
     return vpk(x, y);
 }
+// 1 / a, a >= 0 (below the smallest normal float: of that), so that 0 times it is 0
+__device__ __forceinline__ f2x vrcp_finite(f2x a)
+{
+    float x, y;
+    vunpk(a, x, y);
+    return vrcp(vpk(fmaxf(x, 1.17549435e-38f), fmaxf(y, 1.17549435e-38f)));
+}
 __device__ __forceinline__ f2x vrsqrt(f2x a)
 {
     float x, y;
@@ -201,6 +208,19 @@ __device__ __forceinline__ f2x vrsqrt(f2x a)
     asm("rsqrt.approx.ftz.f32 %0, %0;" : "+f"(x));
     asm("rsqrt.approx.ftz.f32 %0, %0;" : "+f"(y));
     return vpk(x, y);
+}
+
+// s += w0 x0 + w1 x1: one compensated step (Kahan; e: the compensation), or FMAs
+template <int AR>
+__device__ __forceinline__ void add2x(f2x w0, f2x x0, f2x w1, f2x x1, f2x &s, f2x &e)
+{
+    if constexpr (AR == AR_KAHAN) {
+        const f2x y = vfma(w1, x1, vfma(w0, x0, e)), t = vadd(s, y);
+        e = vsub(y, vsub(t, s));
+        s = t;
+    } else {
+        s = vfma(w1, x1, vfma(w0, x0, s));
+    }
 }
 
 // Programmatic dependent launch: a kernel launched with programmatic stream serialization may

@@ -206,7 +206,7 @@ __global__ void __launch_bounds__(256) tof_fwd_kernel(const __grid_constant__ Fw
 //   1. a warp per ray lists the pixels the line crosses in these steps (offset, length, position);
 //   2. all threads compute the weights length x h_t of every listed pixel and TOF bin;
 //   3. thread (ray, slice of TOF_TW bins, half-group) reads each pixel once (16 bytes) and adds it to
-//      its slice's sums, 8 pixels by FMAs and then one compensated step.
+//      its slice's sums, two pixels (about a driving step) per compensated step.
 // ------------------------------------------------------------------------------------------
 constexpr int TOF_TW = 7, TOF_WP = 8, TOF_THREADS = 256, TOF_HG = 24, TOF_STEPS = 32;
 
@@ -318,7 +318,7 @@ __global__ void __launch_bounds__(TOF_THREADS, 2) tof_fwd_stack(const __grid_con
                 for (int q = wid; q < sh.rb; q += TOF_THREADS / 32) {
                     const int n = min(TOF_STEPS, steps_of[q] - c0);
                     bool ok0 = false, ok1 = false;
-                    float l0 = 0.f, l1 = 0.f, tau0 = 0.f;
+                    float l0 = 0.f, l1 = 0.f, tau0 = 0.f, tau1 = 0.f;
                     unsigned o0 = 0, o1 = 0;
                     if (lane < n) {
                         const RayGeo &rg = g.rays[(size_t)slot * NB + tb * sh.rb + q];
@@ -329,7 +329,9 @@ __global__ void __launch_bounds__(TOF_THREADS, 2) tof_fwd_stack(const __grid_con
                         l0 = vw.Lf - l1;
                         ok0 = (unsigned)r0 < (unsigned)N;
                         ok1 = l1 > 0.f && (unsigned)r1 < (unsigned)N;
-                        tau0 = vw.tau0f + (float)dd * tpd + (float)r0 * tpr;
+                        const float taud = fmaf((float)dd, tpd, vw.tau0f);
+                        tau0 = fmaf((float)r0, tpr, taud);
+                        tau1 = fmaf((float)r1, tpr, taud);
                         o0 = (unsigned)dd * ds + (unsigned)r0 * cs;
                         o1 = o0 + cs;
                     }
@@ -337,7 +339,7 @@ __global__ void __launch_bounds__(TOF_THREADS, 2) tof_fwd_stack(const __grid_con
                     const unsigned below = (1u << lane) - 1u;
                     int at = q * E + __popc(m0 & below) + __popc(m1 & below);
                     if (ok0) { off[at] = o0; lt[at] = make_float2(l0, tau0); ++at; }
-                    if (ok1) { off[at] = o1; lt[at] = make_float2(l1, tau0 + tpr); }
+                    if (ok1) { off[at] = o1; lt[at] = make_float2(l1, tau1); }
                     if (lane == 0) count[q] = __popc(m0) + __popc(m1);
                 }
                 __syncthreads();
@@ -347,7 +349,8 @@ __global__ void __launch_bounds__(TOF_THREADS, 2) tof_fwd_stack(const __grid_con
                     for (int i = threadIdx.x; i < count[q] * TT; i += TOF_THREADS) {
                         const int e = i / TT, t = i - e * TT;
                         const float2 p = lt[q * E + e];
-                        const float x = (p.y - (float)(2 * t - (T - 1)) * 0.5f * d + Wt) * idt;
+                        // (the position minus the TOF bin's centre, as tof_fwd_kernel rounds it)
+                        const float x = (fmaf((float)(1 - T + 2 * t) * -0.5f, d, p.y) + Wt) * idt;
                         float h = 0.f;
                         if (t < T && x >= 0.f && x < (float)(TOF_TAB - 1)) h = p.x * tof_table(tab, x, dt_);
                         wts[((q * E + e) * sh.ts + t / TOF_TW) * TOF_WP + t % TOF_TW] = vsplat(h);
@@ -357,19 +360,6 @@ __global__ void __launch_bounds__(TOF_THREADS, 2) tof_fwd_stack(const __grid_con
                 if (work) {
                     const int n = count[rl];
                     const f2x *we = wts + (rl * E * sh.ts + slice) * TOF_WP;
-                    // eight pixels by FMAs onto the compensation term, then one compensated step
-                    auto merge = [&]() {
-#pragma unroll
-                        for (int t = 0; t < TOF_TW; ++t)
-#pragma unroll
-                            for (int q = 0; q < 2; ++q) {
-                                if constexpr (AR == AR_KAHAN) {
-                                    const f2x s = vadd(sm[t][q], er[t][q]);
-                                    er[t][q] = vsub(er[t][q], vsub(s, sm[t][q]));
-                                    sm[t][q] = s;
-                                }
-                            }
-                    };
                     auto pixels = [&](auto number, int e) {
                         constexpr int U = decltype(number)::value;
                         f2x x0[U], x1[U];
@@ -378,30 +368,30 @@ __global__ void __launch_bounds__(TOF_THREADS, 2) tof_fwd_stack(const __grid_con
                             const float *px = img + off[rl * E + e + i];
                             asm("ld.global.nc.v2.b64 {%0, %1}, [%2];" : "=l"(x0[i]), "=l"(x1[i]) : "l"(px));
                         }
-#pragma unroll
-                        for (int i = 0; i < U; ++i) {
-                            const ulonglong2 *wp = reinterpret_cast<const ulonglong2 *>(we + (e + i) * sh.ts * TOF_WP);
+                        auto weights = [&](int i, f2x(&wv)[TOF_TW]) {
+                            const ulonglong2 *wp = reinterpret_cast<const ulonglong2 *>(we + i * sh.ts * TOF_WP);
                             const ulonglong2 w01 = wp[0], w23 = wp[1], w45 = wp[2];
-                            const f2x wv[TOF_TW] = {w01.x, w01.y, w23.x, w23.y, w45.x, w45.y, wp[3].x};
+                            wv[0] = w01.x; wv[1] = w01.y; wv[2] = w23.x; wv[3] = w23.y;
+                            wv[4] = w45.x; wv[5] = w45.y; wv[6] = wp[3].x;
+                        };
 #pragma unroll
-                            for (int t = 0; t < TOF_TW; ++t) {
-                                if constexpr (AR == AR_KAHAN) {
-                                    er[t][0] = vfma(wv[t], x0[i], er[t][0]);
-                                    er[t][1] = vfma(wv[t], x1[i], er[t][1]);
-                                } else {
-                                    sm[t][0] = vfma(wv[t], x0[i], sm[t][0]);
-                                    sm[t][1] = vfma(wv[t], x1[i], sm[t][1]);
+                        for (int i = 0; i < U; i += 2) {
+                            f2x w0[TOF_TW], w1[TOF_TW];
+                            weights(e + i, w0);
+                            if (U > 1) weights(e + i + 1, w1);
+#pragma unroll
+                            for (int t = 0; t < TOF_TW; ++t)
+#pragma unroll
+                                for (int q = 0; q < 2; ++q) {
+                                    const f2x *xq = q ? x1 : x0;
+                                    if (U > 1) add2x<AR>(w0[t], xq[i], w1[t], xq[i + (U > 1)], sm[t][q], er[t][q]);
+                                    else add2x<AR>(w0[t], xq[i], 0ull, 0ull, sm[t][q], er[t][q]);
                                 }
-                            }
                         }
                     };
                     int e = 0;
-                    for (; e + 4 <= n; e += 4) {
-                        pixels(std::integral_constant<int, 4>{}, e);
-                        if (e & 4) merge();
-                    }
+                    for (; e + 4 <= n; e += 4) pixels(std::integral_constant<int, 4>{}, e);
                     for (; e < n; ++e) pixels(std::integral_constant<int, 1>{}, e);
-                    merge();
                 }
                 __syncthreads();                        // the lists are free again
             }

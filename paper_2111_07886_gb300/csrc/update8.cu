@@ -56,8 +56,7 @@ __device__ __forceinline__ void tof_entry(const GeoDev &g, int slot0, int u, int
     }
 }
 
-// Adds an entry's rows [bin][T] to a thread's sums: four TOF bins by FMAs onto the compensation term,
-// then one compensated step.
+// Adds an entry's rows [bin][T] to a thread's sums: two bins of a TOF bin per compensated step.
 template <int KC, int AR>
 __device__ __forceinline__ void tof_gather(const GeoDev &g, const float *w, const float *ent, f2x (&sm)[4], f2x (&er)[4])
 {
@@ -68,16 +67,6 @@ __device__ __forceinline__ void tof_gather(const GeoDev &g, const float *w, cons
     for (int k = 0; k < KC; ++k) l[k] = ent[2 + k];
     const float *h = ent + (KC <= 2 ? 4 : 8);
     const float *row = w + (__float_as_uint(ent[0]) * TT + (unsigned)(tn & 255) * Pp);
-    auto merge = [&]() {
-        if constexpr (AR == AR_KAHAN) {
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const f2x s = vadd(sm[k], er[k]);
-                er[k] = vsub(er[k], vsub(s, sm[k]));
-                sm[k] = s;
-            }
-        }
-    };
     auto bins = [&](auto count, int t) {
         constexpr int U = decltype(count)::value;
         f2x x[U][KC][4];
@@ -88,24 +77,17 @@ __device__ __forceinline__ void tof_gather(const GeoDev &g, const float *w, cons
 #pragma unroll
         for (int i = 0; i < U; ++i)
 #pragma unroll
-            for (int kb = 0; kb < KC; ++kb) {
-                const f2x W = vsplat(h[t + i] * l[kb]);
+            for (int kb = 0; kb < KC; kb += 2) {
+                const f2x W0 = vsplat(h[t + i] * l[kb]), W1 = vsplat(h[t + i] * l[kb + 1]);
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    if constexpr (AR == AR_KAHAN) er[k] = vfma(W, x[i][kb][k], er[k]);
-                    else sm[k] = vfma(W, x[i][kb][k], sm[k]);
-                }
+                for (int k = 0; k < 4; ++k) add2x<AR>(W0, x[i][kb][k], W1, x[i][kb + 1][k], sm[k], er[k]);
             }
         row += U * Pp;
     };
     constexpr int U = KC <= 2 ? 4 : 2;               // TOF bins whose rows are loaded together
     int t = 0;
-    for (; t + U <= n; t += U) {
-        bins(std::integral_constant<int, U>{}, t);
-        if (U == 4 || (t & 2)) merge();
-    }
+    for (; t + U <= n; t += U) bins(std::integral_constant<int, U>{}, t);
     for (; t < n; ++t) bins(std::integral_constant<int, 1>{}, t);
-    merge();
 }
 
 // FP32 update for 8-plane groups held as four f32x2 pairs.  Same step as update_kernel, with:
@@ -122,6 +104,12 @@ __device__ __forceinline__ void tof_gather(const GeoDev &g, const float *w, cons
 // position's group is used as it is and shifted by one plane up and down); X8_VOX, 1/p per voxel
 // (scans with per-bin detection factors); X8_TV, the TV variant (no RDP term, the unclamped z and
 // the metric W written for the proximal step); X8_TOF, time of flight (see x8_patch).
+// With any of these the stencil, nu and the step are the general kernel's operations in its order (GEN):
+// the neighbours row by row with one division per pair, and f - c (scale b + (beta/M) grad R) from c
+// read again after the gather, rounded once at f's ulp.  Folded into A + B b, the step rounds twice:
+// 0.41 instead of 0.29 ulp rms per subiteration, and 2.9e-7 instead of 2.7e-7 from the 64-bit result
+// after one iteration of the 256 x 256 x 89 scan with both the 3-D prior and attenuation (4.19 ms,
+// 4.65 in this form).
 // UV: views whose rows are loaded together in the gather.  Four take 128 registers, two blocks per
 // SM and 8 loads in flight per thread; one takes 80 and three blocks.  The rates per tile are about
 // the same (four 2.6 % faster), so what decides is how evenly the tiles fill the resident blocks
@@ -133,7 +121,7 @@ __global__ void __launch_bounds__(256, UV == 1 ? 3 : 2) update_kernel_x8(
     static_assert(AR != AR_FP64, "FP32 arithmetic only");
     // 16 KB of (pixel, view) entries: the rest of the SM's shared memory stays L1 for the gather
     using Table = BpTable<KC, AR, 1024 / (KC > 2 ? 2 : 1)>;
-    constexpr bool TOF = FL & X8_TOF;
+    constexpr bool TOF = FL & X8_TOF, Z3 = FL & X8_Z3, VOX = FL & X8_VOX, TV = FL & X8_TV, GEN = FL != 0;
     __shared__ typename std::conditional<TOF, X8Patch, Table>::type tb;
     __shared__ __align__(16) float tofs[TOF ? X8_TOF_WORDS : 4];
     // launched behind the projection (see launch_update): nothing is read before it has completed
@@ -158,10 +146,11 @@ __global__ void __launch_bounds__(256, UV == 1 ? 3 : 2) update_kernel_x8(
         const double q = (double)npix * g.P;
         // per-scan scalars in FP32 (an FP64 division per thread is costly at GB300's FP64 rate)
         const float mean_f = dyn ? (float)*a.sum_f / (float)q : 1.f;
+        const float inv_mean_f = GEN && dyn ? (float)q / (float)*a.sum_f : 1.f;
         const float mean_mu = dyn ? (float)*a.sum_mu / (float)q : 1.f;
         const float U = a.fs_U, tt = a.fs_t;
         // eps >= 1e-30 keeps 1/den finite, so that a zero-difference term stays exactly zero
-        const float eps = fmaxf(a.fs_eps, 1e-30f);
+        const float eps = GEN ? a.fs_eps : fmaxf(a.fs_eps, 1e-30f);
         const float *f = reinterpret_cast<const float *>(a.f) + grp * 8;
         const float *w = reinterpret_cast<const float *>(a.w) + grp * 8;
         const float *invp = reinterpret_cast<const float *>(a.invp);
@@ -194,20 +183,28 @@ __global__ void __launch_bounds__(256, UV == 1 ? 3 : 2) update_kernel_x8(
                 const unsigned jc = (unsigned)j;
                 const unsigned xm = ix > 0 ? jc - 1 : jc, xp = ix < N - 1 ? jc + 1 : jc;
                 const unsigned ym = iy > 0 ? jc - N : jc, yp = iy < N - 1 ? jc + N : jc;
-                constexpr bool Z3 = FL & X8_Z3, VOX = FL & X8_VOX, TV = FL & X8_TV;
                 const f2x GR = vsplat(a.fs_gamma_r), EP = vsplat(eps), TWO = vsplat(2.f);
-                f2x c[4], ce[4], gr[4], g2[4], nb0[4], nb1[4];
+                f2x c[4], ce[4], gr[4], g2[4], nb0[4], nb1[4], nu[4];
                 load8x(f + jc * Pp, c);
 #pragma unroll
-                for (int k = 0; k < 4; ++k) { ce[k] = vadd(c[k], EP); gr[k] = 0ull; }
+                for (int k = 0; k < 4; ++k) { if (!GEN) ce[k] = vadd(c[k], EP); gr[k] = 0ull; }
                 auto rdp = [&](const f2x(&x)[4]) {
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {
-                        const f2x d = vsub(c[k], x[k]);
-                        const f2x den = vfma(GR, vabs(d), vadd(ce[k], x[k]));
-                        const f2x num = vadd(den, vfma(TWO, x[k], EP));
-                        const f2x r = vrcp(den);
-                        gr[k] = vfma(vmul(d, vmul(num, r)), r, gr[k]);
+                        const f2x d = vsub(c[k], x[k]), ad = vabs(d);
+                        if constexpr (GEN) {
+                            const f2x EP2 = vadd(EP, EP), THREE = vsplat(3.f);
+                            const f2x den = Z3 ? vadd(vfma(GR, ad, vadd(c[k], x[k])), EP)
+                                               : vfma(GR, ad, vadd(vadd(c[k], x[k]), EP));
+                            const f2x t = Z3 ? vadd(vfma(THREE, x[k], vfma(GR, ad, c[k])), EP2)
+                                             : vfma(GR, ad, vfma(THREE, x[k], vadd(c[k], EP2)));
+                            gr[k] = vfma(vmul(d, t), vrcp_finite(vmul(den, den)), gr[k]);
+                        } else {
+                            const f2x den = vfma(GR, ad, vadd(ce[k], x[k]));
+                            const f2x num = vadd(den, vfma(TWO, x[k], EP));
+                            const f2x r = vrcp(den);
+                            gr[k] = vfma(vmul(d, vmul(num, r)), r, gr[k]);
+                        }
                     }
                 };
                 // 3-D: the planes z - 1 (dn) and z + 1 (up) of a position's group x; a missing plane
@@ -243,105 +240,167 @@ __global__ void __launch_bounds__(256, UV == 1 ? 3 : 2) update_kernel_x8(
                         rdp(up);
                     }
                 };
-                // axial neighbours: RDP terms and the Matlab-style gradient
-                load8x(f + xm * Pp, nb0);
-                load8x(f + xp * Pp, nb1);
-                position(nb0, xm, ix > 0);
-                position(nb1, xp, ix < N - 1);
-                if (dyn) {
-                    const f2x HX = vsplat((ix > 0 && ix < N - 1) ? 0.5f : 1.f);
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        const f2x t = vmul(HX, vsub(nb1[k], nb0[k]));
-                        g2[k] = vmul(t, t);
+                if constexpr (GEN) {
+                    // row by row, as the general stencil adds them
+                    const bool xl = ix > 0, xr = ix < N - 1, yl = iy > 0, yr = iy < N - 1;
+                    const unsigned dm = iy > 0 ? jc - N : jc, dp = iy < N - 1 ? jc + N : jc;
+                    const unsigned j0_ = xl && yl ? dm - 1 : jc, j1_ = xr && yl ? dm + 1 : jc;
+                    const unsigned j2_ = xl && yr ? dp - 1 : jc, j3_ = xr && yr ? dp + 1 : jc;
+                    f2x vu[4], vl[4];
+                    if (!TV) {
+                        load8x(f + j0_ * Pp, nb0);
+                        load8x(f + j1_ * Pp, nb1);
                     }
-                }
-                load8x(f + ym * Pp, nb0);
-                load8x(f + yp * Pp, nb1);
-                position(nb0, ym, iy > 0);
-                position(nb1, yp, iy < N - 1);
-                if constexpr (Z3) {
-                    // the centre column: two neighbours, and the gradient across the planes
+                    if (!TV || dyn) {
+                        load8x(f + ym * Pp, vu);
+                        load8x(f + xm * Pp, vl);
+                    }
+                    position(nb0, j0_, xl && yl);
+                    position(vu, ym, yl);
+                    position(nb1, j1_, xr && yl);
+                    position(vl, xm, xl);
                     f2x dn[4], up[4];
-                    shifted(c, jc, dn, up);
-                    rdp(dn);
-                    rdp(up);
-                    if (dyn) {
+                    if constexpr (Z3) {
+                        // the centre column: two neighbours, and the gradient across the planes
+                        shifted(c, jc, dn, up);
+                        rdp(dn);
+                        rdp(up);
 #pragma unroll
                         for (int k = 0; k < 4; ++k) {
                             const int z0 = grp * 8 + 2 * k;
                             const f2x HZ = vpk(z0 > 0 && z0 + 1 < g.P ? 0.5f : 1.f, z0 + 2 < g.P ? 0.5f : 1.f);
-                            const f2x t = vmul(HZ, vsub(up[k], dn[k]));
-                            g2[k] = vfma(t, t, g2[k]);
+                            g2[k] = vmul(HZ, vsub(up[k], dn[k]));
                         }
                     }
-                }
-                f2x nu[4];
-                if (dyn) {
-                    const f2x HY = vsplat((iy > 0 && iy < N - 1) ? 0.5f : 1.f);
-                    const float nu1 = a.fs_nu1, nu2 = a.fs_nu2;
+                    if (!TV || dyn) load8x(f + xp * Pp, nb0);
+                    position(nb0, xp, xr);
+                    if (dyn) {
+                        const f2x HX = vsplat((ix > 0 && ix < N - 1) ? 0.5f : 1.f);
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        const f2x t = vmul(HY, vsub(nb1[k], nb0[k]));
-                        float r0, r1;
-                        vunpk(vrsqrt(vfma(t, t, g2[k])), r0, r1);
-                        // 1 / mu = 1 / max(0.01, |grad f| / mean f) = min(100, mean f / |grad f|)
-                        r0 = fminf(100.f, r0 * mean_f);
-                        r1 = fminf(100.f, r1 * mean_f);
-                        nu[k] = vpk(fminf(fmaxf(mean_mu * r0, nu1), nu2),
-                                    fminf(fmaxf(mean_mu * r1, nu1), nu2));
+                        for (int k = 0; k < 4; ++k) vl[k] = vmul(HX, vsub(nb0[k], vl[k]));
                     }
-                    if (a.nu_mode == 2)
-                        store8x(reinterpret_cast<float *>(a.nu_frozen) + jc * Pp + grp * 8, nu);
-                } else if (a.nu_mode == 3) {
-                    load8x(reinterpret_cast<const float *>(a.nu_frozen) + jc * Pp + grp * 8, nu);
-                } else {
+                    if (!TV || dyn) load8x(f + yp * Pp, nb1);
+                    if (!TV) load8x(f + j2_ * Pp, nb0);
+                    position(nb0, j2_, xl && yr);
+                    position(nb1, yp, yr);
+                    if (dyn) {
+                        // nu_of: |grad f|^2 below the smallest normal float counts as zero, as in the mu pass
+                        const f2x HY = vsplat((iy > 0 && iy < N - 1) ? 0.5f : 1.f);
+                        const float nu1 = a.fs_nu1, nu2 = a.fs_nu2;
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) nu[k] = vsplat(1.f);
-                }
-                // diagonal neighbours
-                if constexpr (!TV) {
-                    const unsigned dm = iy > 0 ? jc - N : jc, dp = iy < N - 1 ? jc + N : jc;
+                        for (int k = 0; k < 4; ++k) {
+                            const f2x gy = vmul(HY, vsub(nb1[k], vu[k]));
+                            f2x q2 = vfma(vl[k], vl[k], vmul(gy, gy));
+                            if (Z3) q2 = vfma(g2[k], g2[k], q2);
+                            float x0, x1, r0, r1;
+                            vunpk(q2, x0, x1);
+                            vunpk(vrsqrt(q2), r0, r1);
+                            r0 = fmaxf(0.01f, x0 >= 1.17549435e-38f ? x0 * r0 * inv_mean_f : 0.f);
+                            r1 = fmaxf(0.01f, x1 >= 1.17549435e-38f ? x1 * r1 * inv_mean_f : 0.f);
+                            vunpk(vmul(vsplat(mean_mu), vrcp(vpk(r0, r1))), r0, r1);
+                            nu[k] = vpk(fminf(fmaxf(r0, nu1), nu2), fminf(fmaxf(r1, nu1), nu2));
+                        }
+                    }
+                    if (!TV) load8x(f + j3_ * Pp, nb0);
+                    position(nb0, j3_, xr && yr);
+                    if (a.nu_mode == 2) store8x(reinterpret_cast<float *>(a.nu_frozen) + jc * Pp + grp * 8, nu);
+                    if (a.nu_mode == 3) load8x(reinterpret_cast<const float *>(a.nu_frozen) + jc * Pp + grp * 8, nu);
+                    if (a.nu_mode == 0) nu[0] = nu[1] = nu[2] = nu[3] = vsplat(1.f);
+                } else {
+                    // axial neighbours: RDP terms and the Matlab-style gradient
+                    load8x(f + xm * Pp, nb0);
+                    load8x(f + xp * Pp, nb1);
+                    rdp(nb0);
+                    rdp(nb1);
+                    if (dyn) {
+                        const f2x HX = vsplat((ix > 0 && ix < N - 1) ? 0.5f : 1.f);
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            const f2x t = vmul(HX, vsub(nb1[k], nb0[k]));
+                            g2[k] = vmul(t, t);
+                        }
+                    }
+                    load8x(f + ym * Pp, nb0);
+                    load8x(f + yp * Pp, nb1);
+                    rdp(nb0);
+                    rdp(nb1);
+                    if (dyn) {
+                        const f2x HY = vsplat((iy > 0 && iy < N - 1) ? 0.5f : 1.f);
+                        const float nu1 = a.fs_nu1, nu2 = a.fs_nu2;
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            const f2x t = vmul(HY, vsub(nb1[k], nb0[k]));
+                            float r0, r1;
+                            vunpk(vrsqrt(vfma(t, t, g2[k])), r0, r1);
+                            // 1 / mu = 1 / max(0.01, |grad f| / mean f) = min(100, mean f / |grad f|)
+                            r0 = fminf(100.f, r0 * mean_f);
+                            r1 = fminf(100.f, r1 * mean_f);
+                            nu[k] = vpk(fminf(fmaxf(mean_mu * r0, nu1), nu2),
+                                        fminf(fmaxf(mean_mu * r1, nu1), nu2));
+                        }
+                        if (a.nu_mode == 2)
+                            store8x(reinterpret_cast<float *>(a.nu_frozen) + jc * Pp + grp * 8, nu);
+                    } else if (a.nu_mode == 3) {
+                        load8x(reinterpret_cast<const float *>(a.nu_frozen) + jc * Pp + grp * 8, nu);
+                    } else {
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) nu[k] = vsplat(1.f);
+                    }
+                    // diagonal neighbours
                     const bool xl = ix > 0, xr = ix < N - 1, yl = iy > 0, yr = iy < N - 1;
+                    const unsigned dm = iy > 0 ? jc - N : jc, dp = iy < N - 1 ? jc + N : jc;
                     const unsigned j0_ = xl && yl ? dm - 1 : jc, j1_ = xr && yl ? dm + 1 : jc;
                     const unsigned j2_ = xl && yr ? dp - 1 : jc, j3_ = xr && yr ? dp + 1 : jc;
                     load8x(f + j0_ * Pp, nb0);
                     load8x(f + j1_ * Pp, nb1);
-                    position(nb0, j0_, xl && yl);
-                    position(nb1, j1_, xr && yl);
+                    rdp(nb0);
+                    rdp(nb1);
                     load8x(f + j2_ * Pp, nb0);
                     load8x(f + j3_ * Pp, nb1);
-                    position(nb0, j2_, xl && yr);
-                    position(nb1, j3_, xr && yr);
+                    rdp(nb0);
+                    rdp(nb1);
                 }
-                // c = lambda alpha nu S, S = min(f, U - f) / p;  A = f - c (beta/M) 2 gr;  B = -c scale
-                f2x NK[4];
-                if constexpr (VOX) {
-                    load8x(invp + jc * Pp + grp * 8, NK);
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) NK[k] = vmul(NK[k], vsplat(-a.fs_lam * a.fs_ips));
-                } else {
-                    NK[0] = vsplat(-a.fs_lam * invp[j] * a.fs_ips);
-                    NK[1] = NK[2] = NK[3] = NK[0];
-                }
-                const f2x BM = vsplat(2.f * a.fs_bm), SC = vsplat(a.fs_scale);
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    float c0, c1;
-                    vunpk(c[k], c0, c1);
-                    const f2x S = vpk(fminf(c0, U - c0), fminf(c1, U - c1));
-                    const f2x cn = vmul(vmul(nu[k], S), NK[k]);
-                    if constexpr (TV) {
-                        A[k] = c[k];
-                        float w0, w1;
-                        vunpk(cn, w0, w1);
-                        nb0[k] = vpk(2 * k < nlive ? -w0 : 1.f, 2 * k + 1 < nlive ? -w1 : 1.f);
+                if constexpr (GEN) {
+                    // A = -lambda alpha nu S, S = min(f, U - f) / p;  B = (beta/M) grad R
+                    f2x IP[4];
+                    if constexpr (VOX) {
+                        load8x(invp + jc * Pp + grp * 8, IP);
                     } else {
-                        A[k] = vfma(cn, vmul(BM, gr[k]), c[k]);
+                        IP[0] = IP[1] = IP[2] = IP[3] = vsplat(invp[j]);
                     }
-                    B[k] = vmul(cn, SC);
+                    const f2x LAM = vsplat(-a.fs_lam), IPS = vsplat(a.fs_ips), BM = vsplat(a.fs_bm);
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        float c0, c1;
+                        vunpk(c[k], c0, c1);
+                        const f2x S = vmul(vpk(c0 < 0.5f * U ? c0 : U - c0, c1 < 0.5f * U ? c1 : U - c1),
+                                           vmul(IP[k], IPS));
+                        A[k] = vmul(vmul(LAM, nu[k]), S);
+                        B[k] = vmul(BM, vadd(gr[k], gr[k]));
+                    }
+                    if constexpr (TV) {
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            float w0, w1;
+                            vunpk(A[k], w0, w1);
+                            nb0[k] = vpk(2 * k < nlive ? -w0 : 1.f, 2 * k + 1 < nlive ? -w1 : 1.f);
+                        }
+                        store8x(reinterpret_cast<float *>(a.wbuf) + jc * Pp + grp * 8, nb0);
+                    }
+                } else {
+                    // c = lambda alpha nu S, S = min(f, U - f) / p;  A = f - c (beta/M) 2 gr;  B = -c scale
+                    const f2x NK = vsplat(-a.fs_lam * invp[j] * a.fs_ips);
+                    const f2x BM = vsplat(2.f * a.fs_bm), SC = vsplat(a.fs_scale);
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        float c0, c1;
+                        vunpk(c[k], c0, c1);
+                        const f2x S = vpk(fminf(c0, U - c0), fminf(c1, U - c1));
+                        const f2x cn = vmul(vmul(nu[k], S), NK);
+                        A[k] = vfma(cn, vmul(BM, gr[k]), c[k]);
+                        B[k] = vmul(cn, SC);
+                    }
                 }
-                if constexpr (TV) store8x(reinterpret_cast<float *>(a.wbuf) + jc * Pp + grp * 8, nb0);
             }
             // gather backprojection b = A_i^T w with the tile's shared (pixel, view) weights
             f2x sm[4], er[4];
@@ -377,16 +436,7 @@ __global__ void __launch_bounds__(256, UV == 1 ? 3 : 2) update_kernel_x8(
                 auto add = [&](float w0, const f2x(&x0)[4], float w1, const f2x(&x1)[4]) {
                     const f2x W0 = vsplat(w0), W1 = vsplat(w1);
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        if constexpr (AR == AR_KAHAN) {
-                            const f2x y = vfma(W1, x1[k], vfma(W0, x0[k], er[k]));
-                            const f2x t = vadd(sm[k], y);
-                            er[k] = vsub(y, vsub(t, sm[k]));
-                            sm[k] = t;
-                        } else {
-                            sm[k] = vfma(W1, x1[k], vfma(W0, x0[k], sm[k]));
-                        }
-                    }
+                    for (int k = 0; k < 4; ++k) add2x<AR>(W0, x0[k], W1, x1[k], sm[k], er[k]);
                 };
                 int uu = 0;
                 if constexpr (UV > 1) {
@@ -423,12 +473,14 @@ __global__ void __launch_bounds__(256, UV == 1 ? 3 : 2) update_kernel_x8(
             }
             if (!active) continue;
             // step and clamp P_t
-            f2x out[4];
+            f2x out[4], fc[4];
+            if constexpr (GEN) load8x(f + (unsigned)j * Pp, fc);
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 const f2x b = AR == AR_KAHAN ? vadd(sm[k], er[k]) : sm[k];
                 float f0, f1;
-                vunpk(vfma(B[k], b, A[k]), f0, f1);
+                if constexpr (GEN) vunpk(vfma(A[k], vfma(vsplat(a.fs_scale), b, B[k]), fc[k]), f0, f1);
+                else vunpk(vfma(B[k], b, A[k]), f0, f1);
                 if constexpr (!(FL & X8_TV)) {
                     f0 = f0 <= 0.f ? tt : (f0 >= U ? U - tt : f0);
                     f1 = f1 <= 0.f ? tt : (f1 >= U ? U - tt : f1);
@@ -436,7 +488,7 @@ __global__ void __launch_bounds__(256, UV == 1 ? 3 : 2) update_kernel_x8(
                 const int p0 = grp * 8 + 2 * k;
                 f0 = p0 < g.P ? f0 : 0.f;
                 f1 = p0 + 1 < g.P ? f1 : 0.f;
-                part += f0 + f1;
+                part = GEN ? part + f0 + f1 : part + (f0 + f1);
                 out[k] = vpk(f0, f1);
             }
             store8x(reinterpret_cast<float *>(a.fout) + (unsigned)j * Pp + grp * 8, out);
@@ -471,8 +523,7 @@ __global__ void __launch_bounds__(256) bp_table_kernel(const __grid_constant__ G
     }
 }
 
-// The packed update kernel runs for 8-plane groups with uniform bins and without TOF; its table
-// holds 1024 (KC = 2) or 512 (KC = 4) entries of 16 or 32 bytes, two tiles' worth when copied.
+// The entries of 8-plane groups with uniform bins and without TOF; the packed kernel's table holds 1024 (KC = 2) or 512 (KC = 4) entries of 16 or 32 bytes, two tiles' worth when copied.
 size_t bp_table_bytes_bound(const pet_geometry_desc &d)
 {
     if (d.nplanes <= 1 || d.subrays > 1 || d.ring_mm > 0 || d.tof_bins > 1) return 0;
