@@ -417,10 +417,12 @@ template <int KC, int AR, int CAPX = 0> struct BpTable {
 // integers up to where a line falls on a kink (a line assigned to the wrong side of one, by the
 // rounding of the float index, adds at most that rounding: every sum is continuous).  Lines are
 // taken one by one below SUB_CLOSED_MIN (a closed sum costs about as much as six lines), on views
-// along an axis (whose half-open membership is not continuous), and for bins wider than
-// SUB_CLOSED_SPAN pixels or bins (the 32-bit index arithmetic).
+// along an axis (whose half-open membership is not continuous), and for bins whose lines span
+// SUB_CLOSED_SPAN pixels or more: the index rounds to 2^-22 of the span, which must stay small
+// beside one line's length (2e-6 pixels here), and its 32-bit arithmetic ends at 256 pixels.  The
+// gather of uniform bins works in bins, whose lines span one bin.
 constexpr int SUB_CLOSED_MIN = 6;
-constexpr long long SUB_CLOSED_SPAN = 64ll << 32;
+constexpr long long SUB_CLOSED_SPAN = 8ll << 32;
 
 // right shift that leaves 30 bits of values up to `top`, and its power of two over Q32.32
 __device__ __forceinline__ int q32_shift(long long top) { return max(0, 34 - __clzll(top)); }
@@ -554,27 +556,21 @@ __device__ __forceinline__ void bp_weights_ring(const GeoDev &g, const ViewGeo &
         }
     } else {
         const long long pq = vw.pn0q + (long long)ix * vw.pnxq + (long long)iy * vw.pnyq;
-        if (R >= SUB_CLOSED_MIN) {
-            const int shift = q32_shift((long long)R * (vw.hpq - vw.htpq));
-            const float one = q32_scale(shift), scale = vw.islopef * one, scale_l = vw.islopel * one;
-#pragma unroll
-            for (int k = 0; k < KC; ++k) {
-                const int b = b0 + k;
-                if ((unsigned)b >= (unsigned)NB) continue;
-                const long long ds = bg[b].dsq;
-                w[k] = trapezoid_sum(bg[b].c0q - pq, ds, 512.f / (float)ds, R, vw.hpq, vw.htpq, shift, scale,
-                                     scale_l);
-            }
-            return;
-        }
+        const int shift = q32_shift((long long)R * (vw.hpq - vw.htpq));
+        const float one = q32_scale(shift), scale = vw.islopef * one, scale_l = vw.islopel * one;
         const float ws = vw.islopef * (kQ32 * 256.f);
 #pragma unroll
         for (int k = 0; k < KC; ++k) {
             const int b = b0 + k;
             if ((unsigned)b >= (unsigned)NB) continue;
+            const long long ds = bg[b].dsq, u0 = bg[b].c0q - pq;
+            if (R >= SUB_CLOSED_MIN && R * ds < SUB_CLOSED_SPAN) {
+                w[k] = trapezoid_sum(u0, ds, 512.f / (float)ds, R, vw.hpq, vw.htpq, shift, scale, scale_l);
+                continue;
+            }
             float ww = 0.f;
             for (int sr = 0; sr < R; ++sr) {
-                const long long dq = bg[b].c0q + (long long)sr * bg[b].dsq - pq;
+                const long long dq = u0 + (long long)sr * ds;
                 const long long dd = vw.hpq - (dq < 0 ? -dq : dq);
                 ww += dd > 0 ? fminf(vw.Lf, __int2float_rn((int)(dd >> 8)) * ws) : 0.f;
             }
