@@ -11,8 +11,9 @@ pytestmark = pytest.mark.gpu
 DEV = torch.device("cuda:0")
 
 
-# three and four bins per two by two block, few and many views
-@pytest.mark.parametrize("N,P,V,rho", [(64, 9, 96, 1.0), (51, 17, 40, 1.1), (48, 8, 200, 0.9)])
+# three and four bins per two by two block, few and many views (0.93: at 0.9 the tenth line of an axis view
+# lies on a pixel edge but for the rounding of 1.17 / 1.3, and FP32 and FP64 take either side)
+@pytest.mark.parametrize("N,P,V,rho", [(64, 9, 96, 1.0), (51, 17, 40, 1.1), (48, 8, 200, 0.93)])
 def test_error_against_single_planes(N, P, V, rho):
     nb = int(1.45 * N / rho) | 1
     y = np.random.default_rng(N).uniform(0.1, 2.0, (P, V, nb)).astype(np.float32)
