@@ -71,6 +71,18 @@ pet_status geometry_scratch(const pet_geometry *gc, size_t bytes, void **out)
     return PET_OK;
 }
 
+// Whether `bytes` of device memory can be taken for speed alone: as much again stays free for what is
+// needed later.
+bool memory_to_spare(size_t bytes)
+{
+    size_t free_now = 0, all = 0;
+    if (cudaMemGetInfo(&free_now, &all) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return free_now / 2 >= bytes;
+}
+
 // p_j = (A^T 1)_j / M, or 1/M where (A^T 1)_j == 0 (Eq. pj); also 1/p_j in FP32 and FP64.
 __global__ void finish_sensitivity(const double *bp, int npix, int M, float *p, float *invp,
                                    double *invp64)

@@ -335,8 +335,9 @@ struct pet_state {
     void *invp_vox = nullptr;       // 1 / p_j per voxel [N*N][Pp] for diag(a) A (with mult)
     void *nu_frozen = nullptr;
     bool have_frozen = false;
-    void *tvmem = nullptr;          // TV variant: z, W, xbar, px, py (each q_bytes) and, FP32, five
-                                    // more fields of the tiled proximal step
+    void *tvmem = nullptr;          // TV variant: z, W, xbar, px, py (each q_bytes)
+    void *tvtiles = nullptr;        // FP32: the other fields of the tiled proximal step (4 x q_bytes), where
+                                    // the memory for them was to spare
     double *sums = nullptr;         // [0..1] sum f (ping-pong), [2] sum mu, [3..5] objective
     double *objhist = nullptr;      // [(T+1) * 3] objective parts per outer iteration
     int objcap = 0;
@@ -370,7 +371,7 @@ struct TvArgs {
     void *xbar;                // extrapolated primal iterate
     const void *z, *w;         // z = f - W grad F_i and the metric W
     void *px, *py;             // dual variable (kept across subiterations)
-    void *x1, *x2, *xbar2, *px2, *py2;   // FP32: the passes' other fields (see tv_run_tiles)
+    void *x2, *xbar2, *px2, *py2;   // FP32: the tiled passes' other fields (NULL: steps one by one)
     double b;                  // beta / M
     double t, U;               // P_t
     Reducer red;
@@ -431,6 +432,7 @@ bool batch_can_step(const pet_batch *b);   // batch.cu: a step would not wait fo
 
 // geometry helpers (geometry.cu)
 pet_status geometry_scratch(const pet_geometry *g, size_t bytes, void **out);
+bool memory_to_spare(size_t bytes);
 size_t reducer_bytes(int capacity, int nvals);
 void reducer_bind(Reducer &r, void *mem, int capacity, int nvals);
 

@@ -85,9 +85,11 @@ static void state_free(pet_state *s)
     rel(s->redmem);
     rel(s->flag);
     rel(s->tvmem);
+    rel(s->tvtiles);
     rel(s->mult);
     rel(s->invp_vox);
     s->tvmem = nullptr;
+    s->tvtiles = nullptr;
     s->mult = nullptr;
     s->invp_vox = nullptr;
     s->attn = false;
@@ -143,10 +145,18 @@ static pet_status state_alloc(pet_state *s, const pet_geometry *g, int arith, in
     PET_CUDA(cudaMemsetAsync(s->redmem, 0, reducer_bytes(kRedCap, 2), as));
     reducer_bind(s->red, s->redmem, kRedCap, 2);
     PET_CUDA(get((void **)&s->flag, sizeof(int)));
-    if (tv) PET_CUDA(get(&s->tvmem, (arith == AR_FP64 ? 5 : 10) * q_bytes));
+    if (tv) PET_CUDA(get(&s->tvmem, 5 * q_bytes));
     if (attn) {
         PET_CUDA(get((void **)&s->mult, sino * sizeof(float)));
         PET_CUDA(get(&s->invp_vox, q_bytes));
+    }
+    if (tv && arith != AR_FP64 && memory_to_spare(4 * q_bytes)) {
+        const cudaError_t e = get(&s->tvtiles, 4 * q_bytes);
+        if (e != cudaSuccess) {                  // single steps need no more than the state has
+            s->tvtiles = nullptr;
+            if (e != cudaErrorMemoryAllocation) return cuda_fail(e, "TV fields");
+            cudaGetLastError();
+        }
     }
     if (!as) PET_CUDA(cudaStreamSynchronize(nullptr));
     return PET_OK;
@@ -363,12 +373,12 @@ void pet::plan_subiter(pet_state *s, SubiterPlan *pl, bool with_objective)
         ta.xbar = tvm + 2 * s->q_bytes;
         ta.px = tvm + 3 * s->q_bytes;
         ta.py = tvm + 4 * s->q_bytes;
-        if (s->arith != AR_FP64) {
-            ta.x1 = tvm + 5 * s->q_bytes;
-            ta.x2 = tvm + 6 * s->q_bytes;
-            ta.xbar2 = tvm + 7 * s->q_bytes;
-            ta.px2 = tvm + 8 * s->q_bytes;
-            ta.py2 = tvm + 9 * s->q_bytes;
+        if (s->tvtiles) {
+            char *t2 = reinterpret_cast<char *>(s->tvtiles);
+            ta.x2 = t2;
+            ta.xbar2 = t2 + s->q_bytes;
+            ta.px2 = t2 + 2 * s->q_bytes;
+            ta.py2 = t2 + 3 * s->q_bytes;
         }
         ta.b = p.beta / M;
         ta.t = p.t;
