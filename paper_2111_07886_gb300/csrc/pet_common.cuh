@@ -264,7 +264,6 @@ void update_fp32_scalars(UpdateArgs &a);
 // after_kernel: as for launch_forward, behind the projection of the same subiteration
 pet_status launch_update(const UpdateArgs &a, int arith, cudaStream_t st, bool after_kernel = false);
 void update_shape(UpdateArgs &a, int arith);               // fills tpv, nvb
-GeoDev update_geo(const GeoDev &g);                        // plane grouping of the update kernel
 pet_status launch_update_batch(const UpdateArgs &shape, const Batch &b, int arith,
                                cudaStream_t st);
 // stacks in FP32 with uniform bins (update8.cu; launch_update forwards to these)

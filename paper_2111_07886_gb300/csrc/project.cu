@@ -16,14 +16,9 @@
 #include "kernels.cuh"
 #include "profile.cuh"
 
-#ifndef FWD_MAX_CHUNKS
-#define FWD_MAX_CHUNKS 16       // most threads sharing one ray (built-in chunking and autotuner)
-#endif
-#ifndef FWD_TILE_ORDER
-#define FWD_TILE_ORDER 1         // ray tiles within one view, centre bins first (long rays first),
-#endif                           // in the ratio mode (2: in the objective mode too; 0: neither)
-
 namespace pet {
+
+constexpr int FWD_MAX_CHUNKS = 16;   // most threads sharing one ray (built-in chunking and autotuner)
 
 constexpr int Q52_MAX_N = 1024;  // image sides whose FP64 walk keeps its positions in Q11.52
 
@@ -47,7 +42,7 @@ __device__ __forceinline__ void fwd_vblock(const FwdArgs &a, int vloc, int nv,
     const GeoDev &g = a.g;
     const int NG = g.NG, NB = g.NB, N = g.N, Pp = g.Pp, S = a.S, R = a.R;
     const int nrays = a.nviews * NB;
-    constexpr bool kOrder = FWD_TILE_ORDER && (MODE != FWD_OBJECTIVE || FWD_TILE_ORDER > 1);
+    constexpr bool kOrder = MODE != FWD_OBJECTIVE;    // ray tiles of a view from its centre outwards
     const int tpv_view = (NB + R - 1) / R;       // tiles of one view
     const int ntiles = kOrder ? a.nviews * tpv_view : (nrays + R - 1) / R;
     const bool lane_ok = (int)threadIdx.x < R * S * NG;
@@ -371,14 +366,16 @@ static void fwd_dispatch_mode(const FwdArgs &a, const Batch &b, int mode, int gr
 }
 
 template <int G>
-static void fwd_dispatch(const FwdArgs &a, const Batch &b, int mode, int arith, int grid,
-                         cudaStream_t st, bool pdl = false)
+static pet_status fwd_dispatch(const FwdArgs &a, const Batch &b, int mode, int arith, int grid,
+                               cudaStream_t st, bool pdl = false)
 {
     if constexpr (G == 8) {
-        if (arith == AR_FP32) return fwd_dispatch_mode<G, AR_FP32>(a, b, mode, grid, st, pdl);
-        if (arith == AR_KAHAN) return fwd_dispatch_mode<G, AR_KAHAN>(a, b, mode, grid, st, pdl);
+        if (arith == AR_FP32) { fwd_dispatch_mode<G, AR_FP32>(a, b, mode, grid, st, pdl); return PET_OK; }
+        if (arith == AR_KAHAN) { fwd_dispatch_mode<G, AR_KAHAN>(a, b, mode, grid, st, pdl); return PET_OK; }
     }
+    if (arith != AR_FP64) return fail(PET_ERR_INVALID, "projection: no FP32 kernel for this geometry");
     fwd_dispatch_mode<G, AR_FP64>(a, b, mode, grid, st, pdl);
+    return PET_OK;
 }
 
 template <int G, int AR>
@@ -450,7 +447,7 @@ void forward_shape(FwdArgs &a, int mode, int arith)
     while (S > 1 && (256 / a.g.NG) % S) --S;          // S divides the rays-per-block budget
     a.S = S;
     a.R = std::max(1, 256 / (S * a.g.NG));
-    const bool order = FWD_TILE_ORDER && (mode != FWD_OBJECTIVE || FWD_TILE_ORDER > 1);
+    const bool order = mode != FWD_OBJECTIVE;
     const long long ntiles = order ? (long long)a.nviews * ((a.g.NB + a.R - 1) / a.R)
                                    : (nrays + a.R - 1) / a.R;
     a.tpv = 1;
@@ -479,8 +476,8 @@ pet_status launch_forward(const FwdArgs &a0, int mode, int arith, cudaStream_t s
     LaunchScope ls(mode == FWD_RATIO ? PET_K_FORWARD_RATIO
                    : (mode == FWD_OBJECTIVE ? PET_K_OBJ_FORWARD : PET_K_OTHER), st);
     if (plane1_path(a.g, arith)) forward_p1_dispatch(a, b, mode, arith, grid, st, after_kernel);
-    else if (a.g.G == 1) fwd_dispatch<1>(a, b, mode, arith, grid, st, after_kernel);
-    else fwd_dispatch<8>(a, b, mode, arith, grid, st, after_kernel);
+    else if (a.g.G == 1) PET_TRY(fwd_dispatch<1>(a, b, mode, arith, grid, st, after_kernel));
+    else PET_TRY(fwd_dispatch<8>(a, b, mode, arith, grid, st, after_kernel));
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "fwd_kernel launch");
     return PET_OK;
@@ -526,8 +523,8 @@ pet_status launch_forward_batch(const FwdArgs &shape, const Batch &b, int mode, 
     LaunchScope ls(mode == FWD_RATIO ? PET_K_FORWARD_RATIO
                    : (mode == FWD_OBJECTIVE ? PET_K_OBJ_FORWARD : PET_K_OTHER), st);
     if (plane1_path(shape.g, arith)) forward_p1_dispatch(shape, b, mode, arith, b.grid, st, false);
-    else if (shape.g.G == 1) fwd_dispatch<1>(shape, b, mode, arith, b.grid, st);
-    else fwd_dispatch<8>(shape, b, mode, arith, b.grid, st);
+    else if (shape.g.G == 1) PET_TRY(fwd_dispatch<1>(shape, b, mode, arith, b.grid, st));
+    else PET_TRY(fwd_dispatch<8>(shape, b, mode, arith, b.grid, st));
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "fwd_kernel batch launch");
     return PET_OK;

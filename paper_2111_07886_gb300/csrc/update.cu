@@ -11,10 +11,6 @@
 #include "kernels.cuh"
 #include "profile.cuh"
 
-#ifndef UPDATE_G1_BLOCKS
-#define UPDATE_G1_BLOCKS 4      // resident blocks per SM the single-plane update kernel is built for
-#endif
-
 namespace pet {
 
 int sm_count();
@@ -46,7 +42,7 @@ __device__ __forceinline__ T scal(double d, float f)
 // group); the (pixel, view) weights of each tile are computed once into shared memory.  A
 // persistent grid strides over the virtual blocks of one scan or of a batch of scans.
 template <int G, int KC, int AR, bool SUB = false, bool TOF = false>
-__global__ void __launch_bounds__(256, G == 1 ? UPDATE_G1_BLOCKS : 3) update_kernel(
+__global__ void __launch_bounds__(256, G == 1 ? 4 : 3) update_kernel(
     const __grid_constant__ UpdateArgs one, const Batch bt)
 {
     using T = typename ArithT<AR>::T;
@@ -300,10 +296,6 @@ __global__ void __launch_bounds__(256) mu_kernel_x8(const __grid_constant__ Imag
     }
 }
 
-// Plane grouping of the update kernel: the full 8-plane groups (measured faster at three blocks
-// per SM than 4-plane half groups, whose per-thread overheads double).
-GeoDev update_geo(const GeoDev &g) { return g; }
-
 // pixel tiles per virtual block so that a scan never needs more partial sums than its reducer
 int resident_blocks(const void *fn);
 
@@ -365,32 +357,34 @@ void image_shape(ImageArgs &a)
 static int persistent_grid(int nvb) { return std::max(1, std::min(nvb, sm_count() * 8)); }
 
 template <int G, int KC>
-static void update_dispatch(const UpdateArgs &a, const Batch &b, int arith, int grid, cudaStream_t st,
-                            bool pdl)
+static pet_status update_dispatch(const UpdateArgs &a, const Batch &b, int arith, int grid, cudaStream_t st,
+                                  bool pdl)
 {
     if (a.g.T > 1 && a.g.table) {                // TOF on ring-sampled bins: KC = 4
         if (arith == AR_FP32) launch_pdl(update_kernel<G, 4, AR_FP32, true, true>, grid, st, pdl, a, b);
         else if (arith == AR_KAHAN) launch_pdl(update_kernel<G, 4, AR_KAHAN, true, true>, grid, st, pdl, a, b);
         else launch_pdl(update_kernel<G, 4, AR_FP64, true, true>, grid, st, pdl, a, b);
-        return;
+        return PET_OK;
     }
     if (a.g.T > 1) {                             // TOF geometries: generic kernel
         if (arith == AR_FP32) launch_pdl(update_kernel<G, KC, AR_FP32, false, true>, grid, st, pdl, a, b);
         else if (arith == AR_KAHAN) launch_pdl(update_kernel<G, KC, AR_KAHAN, false, true>, grid, st, pdl, a, b);
         else launch_pdl(update_kernel<G, KC, AR_FP64, false, true>, grid, st, pdl, a, b);
-        return;
+        return PET_OK;
     }
     if (a.g.table) {                             // sub-ray / ring geometries: KC = 4, generic kernel
         if (arith == AR_FP32) launch_pdl(update_kernel<G, 4, AR_FP32, true>, grid, st, pdl, a, b);
         else if (arith == AR_KAHAN) launch_pdl(update_kernel<G, 4, AR_KAHAN, true>, grid, st, pdl, a, b);
         else launch_pdl(update_kernel<G, 4, AR_FP64, true>, grid, st, pdl, a, b);
-        return;
+        return PET_OK;
     }
     if constexpr (G == 1) {                      // single-plane FP32: the TV variant only
-        if (arith == AR_FP32) return launch_pdl(update_kernel<G, KC, AR_FP32>, grid, st, pdl, a, b);
-        if (arith == AR_KAHAN) return launch_pdl(update_kernel<G, KC, AR_KAHAN>, grid, st, pdl, a, b);
+        if (arith == AR_FP32) { launch_pdl(update_kernel<G, KC, AR_FP32>, grid, st, pdl, a, b); return PET_OK; }
+        if (arith == AR_KAHAN) { launch_pdl(update_kernel<G, KC, AR_KAHAN>, grid, st, pdl, a, b); return PET_OK; }
     }
+    if (arith != AR_FP64) return fail(PET_ERR_INVALID, "update: no FP32 kernel for this scan");
     launch_pdl(update_kernel<G, KC, AR_FP64>, grid, st, pdl, a, b);
+    return PET_OK;
 }
 
 static pet_status update_any(const UpdateArgs &a, const Batch &b, int arith, int grid, cudaStream_t st,
@@ -402,11 +396,11 @@ static pet_status update_any(const UpdateArgs &a, const Batch &b, int arith, int
     } else if (update_x8_path(a, arith)) {
         update_x8_dispatch(a, b, arith, grid, st, pdl);
     } else if (a.g.G == 1) {
-        if (a.g.K <= 2) update_dispatch<1, 2>(a, b, arith, grid, st, pdl);
-        else update_dispatch<1, 4>(a, b, arith, grid, st, pdl);
+        if (a.g.K <= 2) PET_TRY((update_dispatch<1, 2>(a, b, arith, grid, st, pdl)));
+        else PET_TRY((update_dispatch<1, 4>(a, b, arith, grid, st, pdl)));
     } else {
-        if (a.g.K <= 2) update_dispatch<8, 2>(a, b, arith, grid, st, pdl);
-        else update_dispatch<8, 4>(a, b, arith, grid, st, pdl);
+        if (a.g.K <= 2) PET_TRY((update_dispatch<8, 2>(a, b, arith, grid, st, pdl)));
+        else PET_TRY((update_dispatch<8, 4>(a, b, arith, grid, st, pdl)));
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "update_kernel launch");
@@ -427,32 +421,34 @@ pet_status launch_update_batch(const UpdateArgs &shape, const Batch &b, int arit
 }
 
 template <int G, int KC>
-static void back_dispatch(const BackArgs &a, int arith, int grid, cudaStream_t st)
+static pet_status back_dispatch(const BackArgs &a, int arith, int grid, cudaStream_t st)
 {
     if (a.g.T > 1 && a.g.table) {
         if (arith == AR_FP32) back_kernel<G, 4, AR_FP32, true, true><<<grid, 256, 0, st>>>(a);
         else if (arith == AR_KAHAN) back_kernel<G, 4, AR_KAHAN, true, true><<<grid, 256, 0, st>>>(a);
         else back_kernel<G, 4, AR_FP64, true, true><<<grid, 256, 0, st>>>(a);
-        return;
+        return PET_OK;
     }
     if (a.g.T > 1) {
         if (arith == AR_FP32) back_kernel<G, KC, AR_FP32, false, true><<<grid, 256, 0, st>>>(a);
         else if (arith == AR_KAHAN) back_kernel<G, KC, AR_KAHAN, false, true><<<grid, 256, 0, st>>>(a);
         else back_kernel<G, KC, AR_FP64, false, true><<<grid, 256, 0, st>>>(a);
-        return;
+        return PET_OK;
     }
     if (a.g.table) {
         if (arith == AR_FP32) back_kernel<G, 4, AR_FP32, true><<<grid, 256, 0, st>>>(a);
         else if (arith == AR_KAHAN) back_kernel<G, 4, AR_KAHAN, true><<<grid, 256, 0, st>>>(a);
         else back_kernel<G, 4, AR_FP64, true><<<grid, 256, 0, st>>>(a);
-        return;
+        return PET_OK;
     }
     // (FP32 stacks of at most two candidate bins run back_quad_kernel)
     if constexpr (G == 1 || KC > 2) {
-        if (arith == AR_FP32) { back_kernel<G, KC, AR_FP32><<<grid, 256, 0, st>>>(a); return; }
-        if (arith == AR_KAHAN) { back_kernel<G, KC, AR_KAHAN><<<grid, 256, 0, st>>>(a); return; }
+        if (arith == AR_FP32) { back_kernel<G, KC, AR_FP32><<<grid, 256, 0, st>>>(a); return PET_OK; }
+        if (arith == AR_KAHAN) { back_kernel<G, KC, AR_KAHAN><<<grid, 256, 0, st>>>(a); return PET_OK; }
     }
+    if (arith != AR_FP64) return fail(PET_ERR_INVALID, "backprojection: no FP32 kernel for this geometry");
     back_kernel<G, KC, AR_FP64><<<grid, 256, 0, st>>>(a);
+    return PET_OK;
 }
 
 pet_status launch_back(const BackArgs &a, int arith, cudaStream_t st)
@@ -464,11 +460,11 @@ pet_status launch_back(const BackArgs &a, int arith, cudaStream_t st)
     if (back_quad_path(a, arith)) {
         back_quad_dispatch(a, arith, st);
     } else if (a.g.G == 1) {
-        if (a.g.K <= 2) back_dispatch<1, 2>(a, arith, grid, st);
-        else back_dispatch<1, 4>(a, arith, grid, st);
+        if (a.g.K <= 2) PET_TRY((back_dispatch<1, 2>(a, arith, grid, st)));
+        else PET_TRY((back_dispatch<1, 4>(a, arith, grid, st)));
     } else {
-        if (a.g.K <= 2) back_dispatch<8, 2>(a, arith, grid, st);
-        else back_dispatch<8, 4>(a, arith, grid, st);
+        if (a.g.K <= 2) PET_TRY((back_dispatch<8, 2>(a, arith, grid, st)));
+        else PET_TRY((back_dispatch<8, 4>(a, arith, grid, st)));
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "back_kernel launch");
