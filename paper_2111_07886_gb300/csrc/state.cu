@@ -329,7 +329,7 @@ void pet::plan_subiter(pet_state *s, SubiterPlan *pl, bool with_objective)
     fa.mult = s->attn ? s->mult + (size_t)slot0 * gd.SB * gd.Pp : nullptr;
     forward_shape(fa, FWD_RATIO, s->arith);
     UpdateArgs &ua = pl->upd;
-    ua.g = update_geo(gd);
+    ua.g = gd;
     ua.slot0 = slot0;
     ua.nviews = nv;
     ua.w = s->w;
