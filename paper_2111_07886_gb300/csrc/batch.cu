@@ -36,9 +36,9 @@ constexpr int kKinds = 5;                     // mu pass, forward + ratio, updat
 
 struct BatchClass {
     int G = 0, arith = 0, KC = 0;
-    int z3 = 0;                               // 3-D prior (the generic update and mu kernels)
+    int z3 = 0;                               // 3-D prior (its update and the generic mu kernel)
     int sub = 0;                              // sub-ray geometry (the sub-ray update kernel)
-    int vox = 0;                              // detection factors: p per voxel (generic update)
+    int vox = 0;                              // detection factors: p per voxel (its update)
     int tof = 0;                              // TOF geometries (the TOF projector and gather):
                                               // 1, or 2 for those of tof_fwd_stack
     int cap = 0;                              // scan slots of this class

@@ -230,7 +230,10 @@ static __host__ __device__ __forceinline__ TofShape tof_shape(int NG, int T)
     if (s.rb > most) s.rb = most;
     return s;
 }
-// enough planes and TOF bins that a block's threads have sums to hold (below, the walk per TOF bin)
+// Enough planes and TOF bins that a third of a block's threads have sums to hold; below, the walk per TOF
+// bin.  Iterations of 128 x 128 scans (12 views per subset), this kernel and the walk: 17 planes x 9 TOF bins
+// 1359 and 1473 us, 33 x 21 2526 and 3125, 48 x 7 1470 and 1736.  The line is on the safe side: at 16
+// planes x 9 bins 1328 and 1356 us, 16 x 13 1437 and 1467, 40 x 5 1352 and 1664; 8 x 21 1752 and 1721.
 bool tof_stack_shape(int NG, int T)
 {
     const TofShape s = tof_shape(NG, T);
@@ -491,6 +494,8 @@ void forward_shape_tof(FwdArgs &a, int mode, int arith)
     a.R = 1;
     a.tpv = 1;
     if (mode == FWD_OBJECTIVE) {
+        // (asked without the stack kernel's dynamic shared memory: its registers allow two blocks per SM, whose
+        // 2 x 90 KB fit)
         const void *fn = stack ? tof_stack_fn(mode, arith) : a.g.G == 1 ? tof_fwd_fn<1>(mode, arith) : tof_fwd_fn<8>(mode, arith);
         const long long slots = (long long)sm_count() * resident_blocks(fn);
         long long tpv = (blocks + slots - 1) / slots;

@@ -523,7 +523,8 @@ __global__ void __launch_bounds__(256) bp_table_kernel(const __grid_constant__ G
     }
 }
 
-// The entries of 8-plane groups with uniform bins and without TOF; the packed kernel's table holds 1024 (KC = 2) or 512 (KC = 4) entries of 16 or 32 bytes, two tiles' worth when copied.
+// The entries of 8-plane groups with uniform bins and without TOF; the packed kernel's table holds
+// 1024 (KC = 2) or 512 (KC = 4) entries of 16 or 32 bytes, two tiles' worth when copied.
 size_t bp_table_bytes_bound(const pet_geometry_desc &d)
 {
     if (d.nplanes <= 1 || d.subrays > 1 || d.ring_mm > 0 || d.tof_bins > 1) return 0;
