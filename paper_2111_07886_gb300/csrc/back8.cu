@@ -1,4 +1,4 @@
-// FP32 stand-alone backprojection of stacks with uniform bins (no TOF), two by two pixels per thread.
+// FP32 stand-alone backprojection of large stacks with uniform bins (no TOF), two by two pixels per thread.
 //
 // A thread that gathers one pixel reads KC = 2 rows per view and group.  The lines of one view that
 // meet a 2 x 2 block of pixels are at most KQ = 3 neighbouring bins (4 for bins below 0.94
@@ -23,6 +23,16 @@ template <int KQ> struct __align__(16) QuadEntry {
     unsigned off, pad[3];
 };
 constexpr int QUAD_BYTES = 32 * 1024;
+template <int KQ> __host__ __device__ constexpr int quad_cap() { return QUAD_BYTES / (int)sizeof(QuadEntry<KQ>); }
+
+// a tile's 2 x 2 blocks, about square
+__host__ __device__ __forceinline__ void quad_tile(int NG, int cap, int &tx, int &ty)
+{
+    const int TP = 256 / NG < cap ? 256 / NG : cap;
+    ty = 1;
+    while ((ty + 1) * (ty + 1) <= TP) ++ty;
+    tx = TP / ty;
+}
 
 // One entry: pixels (x, y), (x + 1, y), (x, y + 1), (x + 1, y + 1) against view u of the subset.
 template <int KQ>
@@ -55,13 +65,13 @@ template <int KQ, int AR>
 __global__ void __launch_bounds__(256, 2) back_quad_kernel(const __grid_constant__ BackArgs a)
 {
     using E = QuadEntry<KQ>;
-    constexpr int CAP = QUAD_BYTES / (int)sizeof(E);
+    constexpr int CAP = quad_cap<KQ>();
     __shared__ E tb[CAP];
     const GeoDev &g = a.g;
-    const int N = g.N, NG = g.NG, TP = min(256 / NG, CAP);
-    int ty = 1;
-    while ((ty + 1) * (ty + 1) <= TP) ++ty;
-    const int tx = TP / ty, nq = tx * ty;                             // blocks of a tile
+    const int N = g.N, NG = g.NG;
+    int tx, ty;
+    quad_tile(NG, CAP, tx, ty);
+    const int nq = tx * ty;                                           // blocks of a tile
     const int ntx = (N + 2 * tx - 1) / (2 * tx), ntiles = ntx * ((N + 2 * ty - 1) / (2 * ty));
     const int q = threadIdx.x / NG, grp = threadIdx.x - q * NG, qy = q / tx, qx = q - qy * tx;
     const int VC = min(a.nviews, CAP / nq);
@@ -135,11 +145,21 @@ __global__ void __launch_bounds__(256, 2) back_quad_kernel(const __grid_constant
     }
 }
 
-// Stacks in FP32 whose 2 x 2 pixel blocks meet at most four bins of a view.
+// Stacks in FP32 whose 2 x 2 pixel blocks meet at most four bins of a view, with at least five plane groups
+// to share a tile's entries and tiles that fill the rounds of two blocks per SM to 5/6; the others run the
+// general kernel.  All of 45 drawn sizes on this side are faster than there (1.04 to 1.39 times).  Few groups
+// leave large tiles, few of them and their entries to few threads: 100 x 100 x 2 (180 views) takes 461 us here
+// and 169 there, 256 x 256 x 17 255 and 241; 200 x 200 x 64, whose 340 tiles are 1.1 rounds, 279 and 202;
+// 128 x 128 x 128 (0.84 of a round) 146 and 173.
 bool back_quad_path(const BackArgs &a, int arith)
 {
-    return a.proj && a.g.G == 8 && arith != AR_FP64 && !a.g.table && a.g.T == 1 && a.g.K <= 2 && a.g.KQ <= 4 &&
-           a.g.NG <= 256;
+    if (!a.proj || a.g.G != 8 || arith == AR_FP64 || a.g.table || a.g.T > 1 || a.g.K > 2 || a.g.KQ > 4 || a.g.NG < 5)
+        return false;
+    int tx, ty;
+    quad_tile(a.g.NG, a.g.KQ <= 3 ? quad_cap<3>() : quad_cap<4>(), tx, ty);
+    const long long nt = (long long)((a.g.N + 2 * tx - 1) / (2 * tx)) * ((a.g.N + 2 * ty - 1) / (2 * ty));
+    const long long slots = 2LL * sm_count(), rounds = (nt + slots - 1) / slots;
+    return 6 * nt >= 5 * rounds * slots;
 }
 
 void back_quad_dispatch(const BackArgs &a, int arith, cudaStream_t st)

@@ -441,13 +441,9 @@ static pet_status back_dispatch(const BackArgs &a, int arith, int grid, cudaStre
         else back_kernel<G, 4, AR_FP64, true><<<grid, 256, 0, st>>>(a);
         return PET_OK;
     }
-    // (FP32 stacks of at most two candidate bins run back_quad_kernel)
-    if constexpr (G == 1 || KC > 2) {
-        if (arith == AR_FP32) { back_kernel<G, KC, AR_FP32><<<grid, 256, 0, st>>>(a); return PET_OK; }
-        if (arith == AR_KAHAN) { back_kernel<G, KC, AR_KAHAN><<<grid, 256, 0, st>>>(a); return PET_OK; }
-    }
-    if (arith != AR_FP64) return fail(PET_ERR_INVALID, "backprojection: no FP32 kernel for this geometry");
-    back_kernel<G, KC, AR_FP64><<<grid, 256, 0, st>>>(a);
+    if (arith == AR_FP32) back_kernel<G, KC, AR_FP32><<<grid, 256, 0, st>>>(a);
+    else if (arith == AR_KAHAN) back_kernel<G, KC, AR_KAHAN><<<grid, 256, 0, st>>>(a);
+    else back_kernel<G, KC, AR_FP64><<<grid, 256, 0, st>>>(a);
     return PET_OK;
 }
 

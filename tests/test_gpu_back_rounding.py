@@ -11,9 +11,13 @@ pytestmark = pytest.mark.gpu
 DEV = torch.device("cuda:0")
 
 
-# three and four bins per two by two block, few and many views (0.93: at 0.9 the tenth line of an axis view
-# lies on a pixel edge but for the rounding of 1.17 / 1.3, and FP32 and FP64 take either side)
-@pytest.mark.parametrize("N,P,V,rho", [(64, 9, 96, 1.0), (51, 17, 40, 1.1), (48, 8, 200, 0.93)])
+# three and four bins per two by two block, stacks on the two by two kernel's side of its bound: six to 32
+# plane groups and tiles that fill the SMs (no line of an axis view lies on a pixel edge but for rounding,
+# where FP32 and FP64 may take either side)
+SIZES = [(127, 121, 24, 1.0), (200, 41, 16, 1.13), (91, 250, 40, 0.93)]
+
+
+@pytest.mark.parametrize("N,P,V,rho", SIZES)
 def test_error_against_single_planes(N, P, V, rho):
     nb = int(1.45 * N / rho) | 1
     y = np.random.default_rng(N).uniform(0.1, 2.0, (P, V, nb)).astype(np.float32)
@@ -27,3 +31,19 @@ def test_error_against_single_planes(N, P, V, rho):
         torch.cuda.synchronize()
         err.append(np.linalg.norm(out.cpu().numpy() - ref) / np.linalg.norm(ref))
     assert err[0] <= err[1]
+
+
+# and the largest group count, one group per block row, against the oracle; all views and a subset
+@pytest.mark.parametrize("N,P,V,rho", [(34, 2040, 6, 1.0), (129, 128, 9, 0.93), (199, 48, 7, 2.0)])
+def test_two_by_two_against_oracle(N, P, V, rho):
+    nb = int(1.45 * N / rho) | 1
+    g = pet.Geometry(N, P, 1.3, V, nb, 1.3 * rho, 3, 0.7)
+    og = oracle.geom(N, P, V, nb, 3, pixel_mm=1.3, bin_mm=1.3 * rho, sens=0.7)
+    for i in (-1, 1):
+        nv = V if i < 0 else g.subset_size(i)
+        y = np.random.default_rng(P).uniform(-1.0, 1.0, (P, nv, nb)).astype(np.float32)
+        out = torch.empty((P, N, N), device=DEV)
+        pet.back_subset(g, i, torch.from_numpy(y).to(DEV), out)
+        torch.cuda.synchronize()
+        ref = oracle.back(og, i, y.astype(np.float64))
+        assert np.abs(out.cpu().numpy() - ref).max() <= 1e-5 * np.abs(ref).max(), i
