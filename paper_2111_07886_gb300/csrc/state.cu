@@ -416,7 +416,9 @@ static pet_status tv_step(const SubiterPlan &pl, cudaStream_t st)
 // take the SM slots that the kernel before leaves, and wait for its completion).  beside: other
 // work (an objective evaluation) runs beside the subiterations; it makes better use of the slots
 // that waiting update blocks would hold, so the update is launched plainly (stacked
-// reconstruction with its objective 76.3 ms with, 75.6 without).
+// reconstruction with its objective 76.3 ms with, 75.6 without).  FP64 updates are launched plainly
+// too: blocks waiting behind an FP64 projection of 2.5 or more blocks per SM made it half as fast
+// (iteration of 104 x 104 x 21 with 52 views per subset 2.34 ms, 1.27 without).
 pet_status pet::launch_subiter(const SubiterPlan &pl, cudaStream_t st, bool beside,
                                pet_status (*fork)(void *, MuFork *), void *ctx)
 {
@@ -441,7 +443,7 @@ pet_status pet::launch_subiter(const SubiterPlan &pl, cudaStream_t st, bool besi
     }
     PET_TRY(launch_forward(pl.fwd, FWD_RATIO, pl.arith, st, true));
     if (pl.mu) PET_CUDA(cudaStreamWaitEvent(st, mf.join, 0));
-    PET_TRY(launch_update(pl.upd, pl.arith, st, !pl.mu && !beside));
+    PET_TRY(launch_update(pl.upd, pl.arith, st, !pl.mu && !beside && pl.arith != AR_FP64));
     return tv_step(pl, st);
 }
 
