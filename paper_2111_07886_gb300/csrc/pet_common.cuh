@@ -209,6 +209,7 @@ enum Arith { AR_FP32 = 0, AR_KAHAN = 1, AR_FP64 = 2 };
 pet_status launch_forward(const FwdArgs &a, int mode, int arith, cudaStream_t st,
                           bool after_kernel = false);
 void forward_shape(FwdArgs &a, int mode, int arith);      // fills S, R, tpv, nvb
+bool forward_fills(const FwdArgs &a, int arith);   // an FP32 stack's projection fills the GPU
 bool tof_stack_shape(int NG, int T);   // the shapes tof_fwd_stack is for
 // time-of-flight geometries (g.T > 1; launch_forward / forward_shape forward to these)
 pet_status launch_forward_tof(const FwdArgs &a, int mode, int arith, cudaStream_t st);
@@ -237,6 +238,7 @@ struct UpdateArgs {
     const void *f;             // f^{k,i-1} [N*N][Pp]
     void *fout;                // f^{k,i}
     int C;                     // single-plane FP32 scans: lanes sharing one pixel
+    int beside;                // 1: an objective evaluation takes the slots left (see x8_views)
     const void *invp;          // [N*N], or [N*N][Pp] when vox (float or double)
     int vox;                   // 1: p differs per voxel (a scan with per-bin detection factors)
     const void *bptab;         // the subset's precomputed (pixel, view) entries (pet_geometry::

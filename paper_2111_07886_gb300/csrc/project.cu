@@ -467,6 +467,14 @@ void forward_shape(FwdArgs &a, int mode, int arith)
     a.nvb = (int)((ntiles + a.tpv - 1) / a.tpv);
 }
 
+bool forward_fills(const FwdArgs &a0, int arith)
+{
+    if (a0.g.G != 8 || arith == AR_FP64 || a0.g.T > 1 || a0.g.table) return false;
+    FwdArgs a = a0;
+    forward_shape(a, FWD_RATIO, arith);
+    return fwd_steps(a) == 2;
+}
+
 pet_status launch_forward(const FwdArgs &a0, int mode, int arith, cudaStream_t st,
                           bool after_kernel)
 {

@@ -467,6 +467,7 @@ static pet_status state_subiter(pet_state *s, cudaStream_t st, bool beside = fal
     TraceRange tr("pet_subiter");
     SubiterPlan pl;
     plan_subiter(s, &pl, false);
+    pl.upd.beside = beside && forward_fills(pl.fwd, pl.arith);
     return launch_subiter(pl, st, beside, state_fork, s);
 }
 

@@ -596,10 +596,13 @@ int update_x8_tiles(const UpdateArgs &a)
 // Views loaded together (see update_kernel_x8): 256 x 256 x 89 has 3121 tiles, 6.8 per block of 456
 // (3 blocks per SM) and 10.3 of 304: 7 and 11 rounds, and one view is 1.4 us of 66 faster; 128 x
 // 128 x 64 has 512, where one view took 503 us an iteration and four 438.  A batched launch (N = 0
-// here) takes four.
+// here) takes four.  Beside an objective evaluation, where the projection fills the GPU, one view and
+// three blocks: of 21 drawn reconstructions 7 took 2 to 4 % longer than with the kernels before this file
+// with four views (155 x 155 x 14: 1.67 ms, one view 1.60), 1 does with one.
 static int x8_views(const UpdateArgs &a)
 {
     if (a.g.N == 0 || a.z3 || a.tv || a.vox || a.g.T > 1) return 4;
+    if (a.beside) return 1;
     const double nt = update_x8_tiles(a), s3 = 3.0 * sm_count(), s2 = 2.0 * sm_count();
     return 1.026 * ceil(nt / s3) * s3 < ceil(nt / s2) * s2 ? 1 : 4;
 }
