@@ -20,7 +20,7 @@ struct SinoMap {               // rows u of NB entries, row u being row v(u) of 
     int slot0, NB;
     __device__ __forceinline__ long long at(long long j) const
     {
-        const int u = (int)(j / NB), b = (int)(j - (long long)u * NB);
+        const int u = (int)((unsigned)j / (unsigned)NB), b = (int)(j - (long long)u * NB);   // j < 2^32
         return (long long)(view_of_slot ? __ldg(view_of_slot + slot0 + u) : u) * NB + b;
     }
 };
@@ -68,6 +68,24 @@ __global__ void __launch_bounds__(256) planes_outward(const S *__restrict__ src,
     for (int r = threadIdx.x / TR_J; r < pw; r += 256 / TR_J) col[(long long)(p0 + r) * plane] = t[r][jx];
 }
 
+// One plane group (Pp = 8): a position is one 32-byte sector of the inner array, so plain copies touch
+// nothing twice, and the tiles would be a few planes high (100 positions x planes per block of 256).
+template <typename S, typename D, class Map, bool IN>
+__global__ void __launch_bounds__(256) group_copy(const S *__restrict__ src, D *__restrict__ dst, const Map m,
+                                                  long long n, long long plane, int P, D pad)
+{
+    const unsigned t = blockIdx.x * 256u + threadIdx.x;      // n Pp < 2^32 (geometry limits)
+    if (IN) {                                                // [P][plane] -> [n][8]
+        const unsigned j = t / 8u, p = t & 7u;
+        if (j >= n) return;
+        dst[t] = (int)p < P ? (D)src[(long long)p * plane + m.at(j)] : pad;
+    } else {                                                 // [n][8] -> [P][plane]
+        const unsigned p = t / (unsigned)n, j = t - p * (unsigned)n;
+        if ((int)p >= P) return;
+        dst[(long long)p * plane + m.at(j)] = (D)src[(size_t)j * 8u + p];
+    }
+}
+
 // one plane: dst[j] = src[at(j)] (in) or dst[at(j)] = src[j] (out)
 template <typename S, typename D, class Map, bool IN>
 __global__ void __launch_bounds__(256) plane_copy(const S *__restrict__ src, D *__restrict__ dst, const Map m, long long n)
@@ -86,6 +104,10 @@ static void inward(const void *src, void *dst, const Map &m, long long n, long l
         plane_copy<S, D, Map, true><<<blocks(n), 256, 0, st>>>((const S *)src, (D *)dst, m, n);
         return;
     }
+    if (Pp == 8) {
+        group_copy<S, D, Map, true><<<blocks(8 * n), 256, 0, st>>>((const S *)src, (D *)dst, m, n, plane, P, pad);
+        return;
+    }
     const dim3 grid((unsigned)((n + TR_J - 1) / TR_J), (unsigned)((Pp + TR_P - 1) / TR_P));
     planes_inward<S, D, Map><<<grid, 256, 0, st>>>((const S *)src, (D *)dst, m, n, plane, P, Pp, pad);
 }
@@ -95,6 +117,10 @@ static void outward(const void *src, void *dst, const Map &m, long long n, long 
 {
     if (Pp == 1) {
         plane_copy<S, D, Map, false><<<blocks(n), 256, 0, st>>>((const S *)src, (D *)dst, m, n);
+        return;
+    }
+    if (Pp == 8) {
+        group_copy<S, D, Map, false><<<blocks(P * n), 256, 0, st>>>((const S *)src, (D *)dst, m, n, plane, P, D(0));
         return;
     }
     const dim3 grid((unsigned)((n + TR_J - 1) / TR_J), (unsigned)((P + TR_P - 1) / TR_P));

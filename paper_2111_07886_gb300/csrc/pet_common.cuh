@@ -66,13 +66,12 @@ struct ViewGeo {
     double L;             // length per driving step = 1 / major, pixel units
     double inv_minor;     // 1 / minor (0 when minor == 0)
     float Lf, inv_minorf;
-    float inv_minorl;     // inv_minor - inv_minorf (closed sub-ray sums: see fan_length)
     int xdrive;           // 1: driving index is ix (columns), cross index is iy
     // backprojection footprint (bin units, measured from bin 0)
     long long t0q, cxq, cyq, hq;   // t(ix,iy) = t0 + ix cx + iy cy; half-width h; Q32.32
     double t0, cx, cy, h;
     double wslope;        // length per bin unit of (h - |delta|): rho / (major * minor)
-    float wslopef, wslopel;   // wslope, and wslope - wslopef
+    float wslopef;
     int axis;             // minor == 0: half-open rule, length L for delta in [-h, h)
     // sub-ray model: cross-coordinate shift of half a sub-ray spacing (rho / (2 R a), a the
     // driving component of the view's direction), grid units; sub-ray s of a bin starts
@@ -88,11 +87,14 @@ struct ViewGeo {
     // normal in pixel units, pn = pn0 + ix pnx + iy pny (double and Q32.32), the pixel's
     // half-footprint hp = (|c| + |s|) / 2 and 1 / (major minor) (pixel units)
     long long pn0q, pnxq, pnyq, hpq;
-    // half-width of the flat top of the pixel's trapezoid (where a line's length is L), bin units
-    // and pixel units: h - minor / rho and hp - minor
-    long long htq, htpq;
     double pn0, pnx, pny, hp, islope;
-    float islopef, islopel;
+    float islopef;
+    // closed sub-ray sums (see fan_length, trapezoid_sum): inv_minor - inv_minorf, wslope - wslopef and
+    // islope - islopef; half-width of the flat top of the pixel's trapezoid (where a line's length is
+    // L), bin units and pixel units: h - minor / rho and hp - minor.  After the fields that every gather
+    // and walk reads, which share their cache lines
+    float inv_minorl, wslopel, islopel;
+    long long htq, htpq;
 };
 
 // One bin of a table-driven geometry: its first line's offset c0 and the spacing ds of its R
