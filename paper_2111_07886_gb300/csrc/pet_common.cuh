@@ -273,6 +273,7 @@ pet_status launch_update_batch(const UpdateArgs &shape, const Batch &b, int arit
 // stacks in FP32 with uniform bins (update8.cu; launch_update forwards to these)
 bool update_x8_path(const UpdateArgs &a, int arith);
 int update_x8_tiles(const UpdateArgs &a);
+int update_x8_tpv(const UpdateArgs &a);
 const void *update_x8_fn(const UpdateArgs &a, int arith);
 void update_x8_dispatch(const UpdateArgs &a, const Batch &b, int arith, int grid, cudaStream_t st,
                         bool pdl);

@@ -338,6 +338,7 @@ void update_shape(UpdateArgs &a, int arith)
                                   : (a.g.K <= 2 ? update_fn<8, 2>(arith, sub, tof) : update_fn<8, 4>(arith, sub, tof));
     const int slots = sm_count() * resident_blocks(fn);
     a.tpv = std::max({1, (ntiles + a.red.capacity - 1) / a.red.capacity, (ntiles + slots - 1) / slots});
+    if (update_x8_path(a, arith) && (a.z3 || a.vox) && !a.tv && a.g.T == 1) a.tpv = update_x8_tpv(a);
     a.nvb = (ntiles + a.tpv - 1) / a.tpv;
 }
 

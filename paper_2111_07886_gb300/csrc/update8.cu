@@ -109,7 +109,7 @@ __device__ __forceinline__ void tof_gather(const GeoDev &g, const float *w, cons
 // read again after the gather, rounded once at f's ulp.  Folded into A + B b, the step rounds twice:
 // 0.41 instead of 0.29 ulp rms per subiteration, and 2.9e-7 instead of 2.7e-7 from the 64-bit result
 // after one iteration of the 256 x 256 x 89 scan with both the 3-D prior and attenuation (4.19 ms,
-// 4.65 in this form).
+// 4.76 in this form, with its sums shared out as update_x8_tpv says).
 // UV: views whose rows are loaded together in the gather.  Four take 128 registers, two blocks per
 // SM and 8 loads in flight per thread; one takes 80 and three blocks.  The rates per tile are about
 // the same (four 2.6 % faster), so what decides is how evenly the tiles fill the resident blocks
@@ -593,6 +593,21 @@ int update_x8_tiles(const UpdateArgs &a)
     return (N * N + TP - 1) / TP;
 }
 
+// The 3-D prior and detection factors: tiles per virtual block, whose sum of new voxels is taken in FP32 by
+// thread, as the general kernel shared them out over its three blocks per SM.  The sums' rounding decides
+// the last bit of mean(f), and with it of every nu; another sharing gave results whose single voxels
+// differ by 1e-3 of the image's rms where a scan amplifies rounding.
+int update_x8_tpv(const UpdateArgs &a)
+{
+    const int nt = update_x8_tiles(a), slots = 3 * sm_count();
+    return std::max({1, (nt + a.red.capacity - 1) / a.red.capacity, (nt + slots - 1) / slots});
+}
+static int update_x8_blocks(const UpdateArgs &a)
+{
+    const int tpv = update_x8_tpv(a);
+    return (update_x8_tiles(a) + tpv - 1) / tpv;
+}
+
 // Views loaded together (see update_kernel_x8): 256 x 256 x 89 has 3121 tiles, 6.8 per block of 456
 // (3 blocks per SM) and 10.3 of 304: 7 and 11 rounds, and one view is 1.4 us of 66 faster; 128 x
 // 128 x 64 has 512, where one view took 503 us an iteration and four 438.  A batched launch (N = 0
@@ -601,7 +616,8 @@ int update_x8_tiles(const UpdateArgs &a)
 // with four views (155 x 155 x 14: 1.67 ms, one view 1.60), 1 does with one.
 static int x8_views(const UpdateArgs &a)
 {
-    if (a.g.N == 0 || a.z3 || a.tv || a.vox || a.g.T > 1) return 4;
+    if (a.g.N == 0 || a.tv || a.g.T > 1) return 4;
+    if (a.z3 || a.vox) return update_x8_blocks(a) <= 2 * sm_count() ? 4 : 1;
     if (a.beside) return 1;
     const double nt = update_x8_tiles(a), s3 = 3.0 * sm_count(), s2 = 2.0 * sm_count();
     return 1.026 * ceil(nt / s3) * s3 < ceil(nt / s2) * s2 ? 1 : 4;
@@ -612,9 +628,11 @@ static auto x8_fn(const UpdateArgs &a) -> void (*)(const UpdateArgs, const Batch
 {
     if (a.g.T > 1) return a.vox ? update_kernel_x8<KC, AR, X8_TOF | X8_VOX> : update_kernel_x8<KC, AR, X8_TOF>;
     if (a.tv) return a.vox ? update_kernel_x8<KC, AR, X8_TV | X8_VOX> : update_kernel_x8<KC, AR, X8_TV>;
-    if (a.z3) return a.vox ? update_kernel_x8<KC, AR, X8_Z3 | X8_VOX> : update_kernel_x8<KC, AR, X8_Z3>;
-    if (a.vox) return update_kernel_x8<KC, AR, X8_VOX>;
-    return x8_views(a) == 1 ? update_kernel_x8<KC, AR, 0, 1> : update_kernel_x8<KC, AR, 0>;
+    const bool one = x8_views(a) == 1;
+    if (a.z3 && a.vox) return one ? update_kernel_x8<KC, AR, X8_Z3 | X8_VOX, 1> : update_kernel_x8<KC, AR, X8_Z3 | X8_VOX>;
+    if (a.z3) return one ? update_kernel_x8<KC, AR, X8_Z3, 1> : update_kernel_x8<KC, AR, X8_Z3>;
+    if (a.vox) return one ? update_kernel_x8<KC, AR, X8_VOX, 1> : update_kernel_x8<KC, AR, X8_VOX>;
+    return one ? update_kernel_x8<KC, AR, 0, 1> : update_kernel_x8<KC, AR, 0>;
 }
 
 static auto x8_any(const UpdateArgs &a, int arith)
